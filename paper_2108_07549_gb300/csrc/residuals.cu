@@ -5,7 +5,8 @@
 //  vertex pass  Delta_ik (eq. (3), (3h)) and h_ik = Delta_ik / delta_i
 //               (eq. (2)) in FP64 (FP32 flows summed error-free in FP32
 //               pairs first); per block: sum delta h^2, max |Delta|,
-//               max |Delta| / d_k.
+//               max |Delta| / d_k.  With FP32 flows it overwrites the sweeps'
+//               heights with those of the stored flows.
 //  edge pass    sum_k f_e,k, psi_e (eq. (41)), the certificate length
 //               l_e = max(0, max_k (h_ik - h_jk)) and min_k f_e,k; per block:
 //               sum psi^2, max psi, max psi/scale, sum u_e l_e, min f.
@@ -19,7 +20,7 @@
 //   sum_k d_k (pi_{s_k,k} - pi_{t_k,k}) = sum_{e,k} f_e,k (pi_ik - pi_jk)
 //                                      <= sum_e l_e sum_k f_e,k <= sum_e u_e l_e,
 // so margin > 0 proves that eq. (1) has no solution.
-#include "pdr_internal.cuh"
+#include "widen.cuh"
 
 #include <math.h>
 
@@ -110,12 +111,113 @@ __device__ __forceinline__ void load4(const double* p, double* x)
 // that could be the maximum is skipped.
 constexpr float kSlack = 0.99999619f;  // 1 - 2^-18
 
-// Vertex pass: one warp per vertex, each lane four commodities at a time.
+// The certificate length max_k (h_ik - h_jk) likewise: with FP32 heights a
+// and b (each within 3 x 2^-24 of the FP64 ones) the FP64 difference lies
+// within kHeightSlack (|a| + |b|) of a - b.  Only elements whose upper bound
+// reaches the row's largest lower bound can be the maximum.
+constexpr float kHeightSlack = 4.76837158e-7f;  // 2^-21
+
+// Vertex pass, FP32 flows: one thread per (vertex, four commodities).
 // Delta_ik = sum over in-edges (ascending id) - sum over out-edges
-// (ascending) + the source/sink term (eq. (3), (3h)); h = Delta / delta_i
-// (eq. (2)).  FP32 flows are summed error-free (PairSum), FP64 flows in FP64.
-template <typename T>
-__global__ void __launch_bounds__(256) resid_vertex_kernel(SweepArgs<T> a, ResidIn r, double* __restrict__ h64,
+// (ascending) + the source/sink term (eq. (3), (3h)), the flows summed
+// error-free (PairSum).  Stored: Delta in FP64, from which the later passes
+// form h = Delta / delta_i (eq. (2)), and h rounded to FP32.
+//
+// GB300 issues two FP64 operations per clock and SM, conversions included,
+// and that rate bounded the first form of this pass (83 % of the FP64 pipe,
+// 19 % of HBM: 384 us at n = 10,000, m = 39,600, K = 2,500).  Here FP64 takes
+// one addition and one multiply-add per element: the pair is widened on the
+// integer pipe (widen), h is left to the few elements that need it in FP64,
+// and 1/delta_i is applied once per four squares.  The three kernels of a
+// residual pass at n = 10,000, m = 39,600, K = 10,000: 5.0 ms before, 2.04 ms
+// now (vertex 1.31 ms, edge 0.68 ms).
+__global__ void __launch_bounds__(256) resid_vertex_pair_kernel(SweepArgs<float> a, ResidIn r, float* __restrict__ h32,
+                                                                double* __restrict__ delta, double* __restrict__ part)
+{
+    __shared__ double smem[5][32];
+    const uint32_t nvec = (uint32_t)(a.Kp / 4);
+    const uint64_t total = (uint64_t)a.n * nvec;
+    double zsum = 0.0, cabs = 0.0, crel = 0.0;
+    float cabs32 = 0.f, crel32 = 0.f;  // FP32 estimates of the elements behind cabs, crel
+    for (uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+         idx += (uint64_t)gridDim.x * blockDim.x) {
+        const uint32_t i = total <= 0xffffffffull ? (uint32_t)idx / nvec : (uint32_t)(idx / nvec);
+        const uint32_t v = (uint32_t)(idx - (uint64_t)i * nvec);
+        const int k0 = 4 * (int)v;
+        PairSum acc[4];
+        const int64_t q0 = a.inc_ptr[i], q1 = a.inc_ptr[i + 1];
+        auto add = [&](int32_t ev, const float4& x) {
+            const float sg = ev >= 0 ? 1.f : -1.f;  // in-edges e, then out-edges ~e
+            acc[0].add(sg * x.x), acc[1].add(sg * x.y), acc[2].add(sg * x.z), acc[3].add(sg * x.w);
+        };
+        auto row = [&](int32_t ev) {
+            const int64_t e = ev >= 0 ? ev : ~ev;
+            return __ldg(reinterpret_cast<const float4*>(a.f + e * a.Kp) + v);
+        };
+        int64_t q = q0;
+        for (; q + 4 <= q1; q += 4) {  // four rows in flight
+            int32_t ev[4];
+            float4 x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) ev[u] = a.inc[q + u];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] = row(ev[u]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) add(ev[u], x[u]);
+        }
+        for (; q < q1; ++q) {
+            const int32_t ev = a.inc[q];
+            add(ev, row(ev));
+        }
+        const int4 sv = __ldg(reinterpret_cast<const int4*>(a.s + k0));
+        const int4 tv = __ldg(reinterpret_cast<const int4*>(a.t + k0));
+        const float4 iv = __ldg(reinterpret_cast<const float4*>(r.inv_dem_f + k0));
+        const int ss[4] = {sv.x, sv.y, sv.z, sv.w}, tt[4] = {tv.x, tv.y, tv.z, tv.w};
+        const float idm[4] = {iv.x, iv.y, iv.z, iv.w};
+        const float idg = a.inv_deg[i];
+        double D[4], sq = 0.0;
+        float hf[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int k = k0 + j;
+            D[j] = widen(acc[j].hi) + widen(acc[j].lo);
+            float D32 = __fadd_rn(acc[j].hi, acc[j].lo);
+            if (k >= a.K) D[j] = 0.0, D32 = 0.f;  // the padding carries no commodity
+            if (ss[j] == (int)i || tt[j] == (int)i) {  // padding has s = t = -1
+                D[j] += ss[j] == (int)i ? r.dem_d[k] : -r.dem_d[k];
+                D32 = (float)D[j];
+            }
+            hf[j] = D32 * idg;
+            sq = fma(D[j], D[j], sq);
+            const float ad = fabsf(D32);
+            if (ad > 0.f) {
+                if (ad >= cabs32 * kSlack) {
+                    cabs = fmax(cabs, fabs(D[j]));
+                    cabs32 = fmaxf(cabs32, ad);
+                }
+                const float rel = ad * idm[j];
+                if (rel >= crel32 * kSlack) {
+                    crel = fmax(crel, fabs(D[j]) / r.dem_d[k]);
+                    crel32 = fmaxf(crel32, rel);
+                }
+            }
+        }
+        zsum = fma(sq, r.inv_deg_d[i], zsum);  // delta_i h^2 = Delta^2 / delta_i
+        double2* dp = reinterpret_cast<double2*>(delta + (int64_t)i * a.Kp + k0);
+        dp[0] = make_double2(D[0], D[1]);
+        dp[1] = make_double2(D[2], D[3]);
+        *reinterpret_cast<float4*>(h32 + (int64_t)i * a.Kp + k0) = make_float4(hf[0], hf[1], hf[2], hf[3]);
+    }
+    double v[3] = {zsum, cabs, crel};
+    const int op[3] = {0, 1, 1};
+    block_reduce<3>(v, op, smem);
+    if (threadIdx.x == 0)
+        for (int q = 0; q < kVParts; ++q) part[(int64_t)blockIdx.x * kVParts + q] = v[q];
+}
+
+// Vertex pass, FP64 flows: one warp per vertex, each lane four commodities at
+// a time; h = Delta / delta_i stored in FP64.
+__global__ void __launch_bounds__(256) resid_vertex_kernel(SweepArgs<double> a, ResidIn r, double* __restrict__ h64,
                                                            double* __restrict__ part)
 {
     __shared__ double smem[5][32];
@@ -130,40 +232,21 @@ __global__ void __launch_bounds__(256) resid_vertex_kernel(SweepArgs<T> a, Resid
         const double invdeg = r.inv_deg_d[i];
         for (int v = lane; v < nvec; v += 32) {
             const int k0 = 4 * v;
-            double D[4];
+            double D[4] = {0.0, 0.0, 0.0, 0.0};
             float D32[4];
-            if constexpr (sizeof(T) == 4) {
-                PairSum acc[4];
-                for (int64_t q = i0; q < i1; ++q) {
-                    const float4 x = __ldg(reinterpret_cast<const float4*>(a.f + (int64_t)a.in_eid[q] * a.Kp + k0));
-                    acc[0].add(x.x), acc[1].add(x.y), acc[2].add(x.z), acc[3].add(x.w);
-                }
-                for (int64_t e = o0; e < o1; ++e) {
-                    const float4 x = __ldg(reinterpret_cast<const float4*>(a.f + e * a.Kp + k0));
-                    acc[0].add(-x.x), acc[1].add(-x.y), acc[2].add(-x.z), acc[3].add(-x.w);
-                }
+            double x[4];
+            for (int64_t q = i0; q < i1; ++q) {
+                load4(a.f + (int64_t)a.in_eid[q] * a.Kp + k0, x);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    D[j] = acc[j].value();
-                    D32[j] = __fadd_rn(acc[j].hi, acc[j].lo);
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) D[j] = 0.0;
-                double x[4];
-                for (int64_t q = i0; q < i1; ++q) {
-                    load4(reinterpret_cast<const double*>(a.f) + (int64_t)a.in_eid[q] * a.Kp + k0, x);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) D[j] += x[j];
-                }
-                for (int64_t e = o0; e < o1; ++e) {
-                    load4(reinterpret_cast<const double*>(a.f) + e * a.Kp + k0, x);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) D[j] -= x[j];
-                }
-#pragma unroll
-                for (int j = 0; j < 4; ++j) D32[j] = (float)D[j];
+                for (int j = 0; j < 4; ++j) D[j] += x[j];
             }
+            for (int64_t e = o0; e < o1; ++e) {
+                load4(a.f + e * a.Kp + k0, x);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) D[j] -= x[j];
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) D32[j] = (float)D[j];
             const int4 sv = __ldg(reinterpret_cast<const int4*>(a.s + k0));
             const int4 tv = __ldg(reinterpret_cast<const int4*>(a.t + k0));
             const int ss[4] = {sv.x, sv.y, sv.z, sv.w}, tt[4] = {tv.x, tv.y, tv.z, tv.w};
@@ -207,9 +290,13 @@ __global__ void __launch_bounds__(256) resid_vertex_kernel(SweepArgs<T> a, Resid
 // sum_k f_e,k (error-free pairs for FP32 flows), psi_e (eq. (41)), min_k f_e,k
 // and the certificate length l_e = max(0, max_k (h_ik - h_jk)) in FP64 (only
 // where u_e > 0: an edge without capacity adds nothing to sum_e u_e l_e).
+// FP32 flows: h64 holds Delta, and the FP32 heights h32 decide which
+// elements need their FP64 difference, so a row costs 12 bytes per element
+// and FP64 only at its few candidates (both height rows in FP64 made the
+// FP64 pipe the bound: 559 us at m = 39,600, K = 2,500).
 template <typename T>
-__global__ void __launch_bounds__(256) resid_edge_kernel(SweepArgs<T> a, ResidIn r, const double* __restrict__ h64,
-                                                         double* __restrict__ part)
+__global__ void __launch_bounds__(256) resid_edge_kernel(SweepArgs<T> a, ResidIn r, const float* __restrict__ h32,
+                                                         const double* __restrict__ h64, double* __restrict__ part)
 {
     __shared__ double smem[5][32];
     const int lane = threadIdx.x & 31;
@@ -220,30 +307,62 @@ __global__ void __launch_bounds__(256) resid_edge_kernel(SweepArgs<T> a, ResidIn
     for (int64_t e = warp; e < a.m; e += nwarps) {
         const double ue = r.u_d[e];
         const bool need_l = ue > 0.0;
-        const double* hi = h64 + (int64_t)a.src[e] * a.Kp;
-        const double* hj = h64 + (int64_t)a.col[e] * a.Kp;
+        const int64_t ro = (int64_t)a.src[e] * a.Kp, co = (int64_t)a.col[e] * a.Kp;
         double tot = 0.0, l = 0.0, mn = INFINITY;
         if constexpr (sizeof(T) == 4) {
             PairSum acc;
-            float mn32 = INFINITY;
+            // the largest lower bound, and the element with the largest
+            // difference: its index and upper bound, and the largest upper
+            // bound of the lane's other elements
+            float mn32 = INFINITY, lb = 0.f, best = 0.f, up = 0.f, up2 = 0.f;
+            int at = -1;
+            const float4* fr = reinterpret_cast<const float4*>(a.f + e * a.Kp);
+            const float4* hi = reinterpret_cast<const float4*>(h32 + ro);
+            const float4* hj = reinterpret_cast<const float4*>(h32 + co);
+            double wi = 0.0, wj = 0.0;
+            if (need_l) {
+                wi = r.inv_deg_d[a.src[e]];
+                wj = r.inv_deg_d[a.col[e]];
+            }
+#pragma unroll 4
             for (int v = lane; v < nvec; v += 32) {
                 const int k0 = 4 * v;
-                const float4 x = __ldg(reinterpret_cast<const float4*>(a.f + e * a.Kp + k0));
+                const float4 x = __ldg(fr + v);
                 const float xs[4] = {x.x, x.y, x.z, x.w};
-                const int nk = a.K - k0 < 4 ? a.K - k0 : 4;  // the padding carries no commodity
-                for (int j = 0; j < nk; ++j) {
+                float p[4] = {}, q[4] = {};
+                if (need_l) {
+                    const float4 y = __ldg(hi + v), z = __ldg(hj + v);
+                    p[0] = y.x, p[1] = y.y, p[2] = y.z, p[3] = y.w;
+                    q[0] = z.x, q[1] = z.y, q[2] = z.z, q[3] = z.w;
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (k0 + j >= a.K) continue;  // the padding carries no commodity
                     acc.add(xs[j]);
                     mn32 = fminf(mn32, xs[j]);
-                }
-                if (need_l) {
-                    double p[4], q[4];
-                    load4(hi + k0, p);
-                    load4(hj + k0, q);
-                    for (int j = 0; j < nk; ++j) l = fmax(l, p[j] - q[j]);
+                    const float x0 = p[j] - q[j], sl = kHeightSlack * (fabsf(p[j]) + fabsf(q[j]));
+                    lb = fmaxf(lb, x0 - sl);
+                    const bool more = x0 > best;
+                    up2 = fmaxf(up2, more ? up : x0 + sl);
+                    up = more ? x0 + sl : up;
+                    at = more ? k0 + j : at;
+                    best = more ? x0 : best;
                 }
             }
             tot = (double)acc.hi + (double)acc.lo;
             mn = (double)mn32;
+            if (need_l) {
+                const float low = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(lb)));  // lb >= 0
+                if (at >= 0 && up >= low) l = fmax(l, h64[ro + at] * wi - h64[co + at] * wj);
+                if (__any_sync(0xffffffffu, up2 > 0.f && up2 >= low)) {  // a lane holds several such elements
+                    const float* si = h32 + ro;
+                    const float* sj = h32 + co;
+                    for (int k = lane; k < a.K; k += 32) {
+                        const float x0 = si[k] - sj[k], sl = kHeightSlack * (fabsf(si[k]) + fabsf(sj[k]));
+                        if (x0 + sl > 0.f && x0 + sl >= low) l = fmax(l, h64[ro + k] * wi - h64[co + k] * wj);
+                    }
+                }
+            }
         } else {
             for (int v = lane; v < nvec; v += 32) {
                 const int k0 = 4 * v;
@@ -256,8 +375,8 @@ __global__ void __launch_bounds__(256) resid_edge_kernel(SweepArgs<T> a, ResidIn
                 }
                 if (need_l) {
                     double p[4], q[4];
-                    load4(hi + k0, p);
-                    load4(hj + k0, q);
+                    load4(h64 + ro + k0, p);
+                    load4(h64 + co + k0, q);
                     for (int j = 0; j < nk; ++j) l = fmax(l, p[j] - q[j]);
                 }
             }
@@ -282,16 +401,21 @@ __global__ void __launch_bounds__(256) resid_edge_kernel(SweepArgs<T> a, ResidIn
         for (int q = 0; q < kEParts; ++q) part[(int64_t)blockIdx.x * kEParts + q] = v[q];
 }
 
+// One block; its time is the latency of the K gathers and of the partials, so
+// every thread keeps several of them in flight.  FP32 flows: h64 holds Delta.
 template <typename T>
-__global__ void __launch_bounds__(256) resid_final_kernel(SweepArgs<T> a, const double* __restrict__ dem_d,
-                                                          const double* __restrict__ h64,
-                                                          const double* __restrict__ part, int32_t grid_v,
-                                                          int32_t grid_e, ResidOut* __restrict__ out)
+__global__ void __launch_bounds__(1024) resid_final_kernel(SweepArgs<T> a, ResidIn r, const double* __restrict__ h64,
+                                                           const double* __restrict__ part, int32_t grid_v,
+                                                           int32_t grid_e, ResidOut* __restrict__ out)
 {
     __shared__ double smem[5][32];
+    const double* dem_d = r.dem_d;
     double gain = 0.0, gabs = 0.0;
+#pragma unroll 4
     for (int k = threadIdx.x; k < a.K; k += blockDim.x) {
-        const double diff = h64[(int64_t)a.s[k] * a.Kp + k] - h64[(int64_t)a.t[k] * a.Kp + k];
+        const int32_t i = a.s[k], j = a.t[k];
+        const double wi = sizeof(T) == 4 ? r.inv_deg_d[i] : 1.0, wj = sizeof(T) == 4 ? r.inv_deg_d[j] : 1.0;
+        const double diff = h64[(int64_t)i * a.Kp + k] * wi - h64[(int64_t)j * a.Kp + k] * wj;
         gain += dem_d[k] * diff;
         gabs += dem_d[k] * fabs(diff);
     }
@@ -336,9 +460,12 @@ template <typename T>
 cudaError_t launch_residuals(const SweepArgs<T>& a, const ResidIn& r, double* h64, double* part, int32_t grid_v,
                              int32_t grid_e, ResidOut* out, cudaStream_t stream)
 {
-    resid_vertex_kernel<T><<<grid_v, 256, 0, stream>>>(a, r, h64, part);
-    resid_edge_kernel<T><<<grid_e, 256, 0, stream>>>(a, r, h64, part + (int64_t)grid_v * kVParts);
-    resid_final_kernel<T><<<1, 256, 0, stream>>>(a, r.dem_d, h64, part, grid_v, grid_e, out);
+    if constexpr (sizeof(T) == 4) resid_vertex_pair_kernel<<<grid_v, 256, 0, stream>>>(a, r, a.h, h64, part);
+    else resid_vertex_kernel<<<grid_v, 256, 0, stream>>>(a, r, h64, part);
+    const float* h32 = sizeof(T) == 4 ? reinterpret_cast<const float*>(a.h) : nullptr;
+    resid_edge_kernel<T><<<grid_e, 256, 0, stream>>>(a, r, h32, h64, part + (int64_t)grid_v * kVParts);
+    const int longest = a.K > grid_v ? (a.K > grid_e ? a.K : grid_e) : (grid_v > grid_e ? grid_v : grid_e);
+    resid_final_kernel<T><<<1, longest > 256 ? 1024 : 256, 0, stream>>>(a, r, h64, part, grid_v, grid_e, out);
     return cudaGetLastError();
 }
 
