@@ -99,25 +99,15 @@ typedef enum {
 
 typedef struct {
     int32_t precision;  /* pdr_precision (default PDR_PREC_FP32) */
-    int32_t use_graph;  /* sweep-loop engine.  1: the loop runs on the device as one CUDA graph with
-                           a conditional while node (default).  0: the same kernels are launched
-                           from a host loop that reads the stop flag between chunks of sweeps.
-                           2: one persistent cooperative kernel runs the excess pass and the edge
-                           QPs of every sweep, separated by grid barriers, for 1024 sweeps per
-                           launch (PDR_ALGO_ESO with a lane-group edge variant, K <= 1024 in FP32
-                           or 512 in FP64; otherwise 1 is used); a barrier that waits more than
-                           about a second ends the solve with PDR_ERR_TIMEOUT.
-                           3: one thread-block cluster (1-8 blocks) runs the whole solve --
-                           excess pass, objective and stop test, edge QPs, separated by
-                           cluster barriers -- for 2048 sweeps per launch, as the batched
-                           form does for its small instances (PDR_ALGO_ESO or PDR_ALGO_CK,
-                           m x K <= 2^18 and a lane-group edge variant of at most 4 vectors
-                           per lane; otherwise 1 is used).  An instance that one block solves
-                           and whose arrays fit in 100 KB of shared memory (flows, heights,
-                           roots, partials, state and the read-only arrays of a sweep) is
-                           solved there, copied in and out once per launch.  FP64 sweeps
-                           (PDR_PREC_FP64 and the FP64 tail) run on engine 1: one block has
-                           one SM's FP64 rate.  Same flows and sweeps as 1. */
+    int32_t use_graph;  /* sweep-loop engine.  1: the loop runs on the device, as one CUDA graph with
+                           a conditional while node, or -- FP32 sweeps of Alg. 1 and Program (6)
+                           on an instance that fits in the shared memory of a thread-block
+                           cluster, with excess_variant < 0 -- on one cluster of 1-8 blocks
+                           (default); 0: a host loop launches the same kernels (profiling); 2:
+                           one persistent cooperative kernel (small instances; the graph where
+                           it does not apply); 3: the cluster whatever excess_variant is (the
+                           graph where it does not apply).  Per element the arithmetic is the
+                           same in all of them (bit-identical flows); z agrees to rounding. */
     double eps_obj;     /* Alg. 1 stop rule, absolute; <= 0 disables (default 1e-6, Section 7) */
     double resid_tol;   /* residual stop and feasibility tolerance; <= 0 disables the stop (default 1e-6) */
     double eps_rel;     /* relative objective-change stop; <= 0 disables (default 0) */
@@ -477,18 +467,18 @@ typedef struct {
  * with the options opt shared by all).  Every instance gets its own context
  * on `stream`; an autotuner then times the edge-kernel variants that fit each
  * instance's row length (lanes per edge, vectors per lane, block size) on
- * that instance and keeps the fastest; opt->edge_variant >= 0 fixes the
- * variant for every instance instead.  Errors: PDR_ERR_INVALID_ARG (count <
+ * that instance and keeps the fastest; an instance that a cluster solves
+ * keeps the smallest lane group that holds its rows, and opt->edge_variant
+ * >= 0 fixes the variant for every instance instead.  Errors: PDR_ERR_INVALID_ARG (count <
  * 1, NULL, or an instance rejected by pdr_create: the message names it),
  * PDR_ERR_OOM, PDR_ERR_CUDA, PDR_ERR_UNSUPPORTED. */
 pdr_status pdr_batch_create(int32_t count, const pdr_instance *inst, const pdr_options *opt, void *stream,
                             pdr_batch **out);
 
-/* Solves every instance from its current state.  Small instances (m x K <=
- * 2^18 on a lane-group variant of at most 4 vectors per lane, Alg. 1 or
- * Program (6)) run their FP32 sweeps on one thread-block cluster each, in
- * shared launches of the cluster kernel (engine 3 of pdr_options.use_graph,
- * with its shared-memory form for the instances that fit).  The others, and
+/* Solves every instance from its current state.  Instances that fit in the
+ * shared memory of a thread-block cluster (on a lane-group variant of at most
+ * 4 vectors per lane, Alg. 1 or Program (6)) run their FP32 sweeps on one
+ * cluster each, in shared launches (see pdr_options.use_graph).  The others, and
  * every FP64 sweep (one block has only one SM's FP64 rate), run in one CUDA
  * graph launch: a conditional while loop whose body holds one chain of
  * sweeps per instance; the chains are independent, so the instances run

@@ -13,12 +13,14 @@
 #include "pdr.h"
 #include "pdr_internal.cuh"
 
+#include <algorithm>
 #include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <tuple>
 #include <vector>
 
 using namespace pdr;
@@ -186,7 +188,13 @@ struct pdr_ctx {
     long long barrier_ns = kBarrierNs;
     int hold_barrier = 0;
     int64_t t_widen = -1;  // t at which the FP64 tail of the last solve began (-1: none)
-    unsigned char* cl_args = nullptr;  // the cluster engine's arguments and instance id (device)
+    // cluster engine: the vertex split for clusters of 1, 2, 4 and 8 blocks
+    // (cl_split: their csize + 1 first vertices one after the other, on the
+    // device) and the largest share of any block; max_m < 0: no split
+    int32_t* cl_split = nullptr;
+    struct {
+        int32_t max_n = 0, max_m = -1, max_chunks = 0;
+    } cl[4];
     // reverse-mode workspace (pdr_backward: checkpoints, segment states,
     // cotangents), kept for later calls: the i-th buffer a call asks for is
     // reused when it is large enough, so calls with the same T, checkpoint
@@ -776,74 +784,131 @@ pdr_status widen_to_fp64(pdr_ctx* ctx)
 }
 
 constexpr int64_t kPersistChunk = 1024;  // sweeps per persistent launch (even)
-constexpr int64_t kBlockElems = int64_t(1) << 18;  // m x Kp up to which one cluster solves an instance
-constexpr int64_t kBlockChunk = 2048;              // sweeps per launch of the cluster kernel
+constexpr int kClusterChunk = 8192;  // sweeps per launch of the cluster engine
 
-// Blocks of the thread-block cluster that runs an instance's whole solve:
-// enough that each lane group handles at most 16 edges per sweep (1..8).
-int batch_cluster_size(const pdr_ctx* c, int p);
-
-// Shared memory of the one-block engine's shared-memory form for instance c
-// in precision p, or 0 where it does not apply (a cluster of several blocks,
-// or more than kBlockSmemMax bytes).
-int64_t block_smem(const pdr_ctx* c, int p)
+// The vertex splits of the cluster engine (see pdr_ctx::cl): contiguous
+// ranges of about equal out-edges and incidences.  split: 1 + 2 + 4 + 8 + 4
+// entries.  Instances far beyond shared memory keep max_m = -1.
+constexpr int kClusterSplits = 19;
+void plan_clusters(pdr_ctx* ctx, const int64_t* row_ptr, const int32_t* col, std::vector<int32_t>* split)
 {
-    if (batch_cluster_size(c, p) != 1) return 0;
-    const int64_t n_psi = kBatchThreads / 32;
-    const int64_t b = p == Prec<double>::id ? block_smem_bytes<double>(c->n, c->m, c->Kp, n_psi)
-                                         : block_smem_bytes<float>(c->n, c->m, c->Kp, n_psi);
-    return b <= kBlockSmemMax ? b : 0;
+    const int32_t n = ctx->n;
+    const int64_t m = ctx->m;
+    split->assign(kClusterSplits, 0);
+    if (m < 1 || ctx->Kp > 512 || 8 * (m + n) * ctx->Kp > (int64_t)kClusterMax * kClusterSmemMax)
+        return;
+    std::vector<int64_t> in_ptr(n + 1, 0);
+    for (int64_t e = 0; e < m; ++e) ++in_ptr[col[e] + 1];
+    for (int32_t i = 0; i < n; ++i) in_ptr[i + 1] += in_ptr[i];
+    std::vector<int64_t> chunks(n + 1, 0);  // fours of incident rows of vertices 0 .. i - 1
+    for (int32_t i = 0; i < n; ++i)
+        chunks[i + 1] = chunks[i] + (in_ptr[i + 1] - in_ptr[i] + 3) / 4 + (row_ptr[i + 1] - row_ptr[i] + 3) / 4;
+    auto weight = [&](int64_t i) { return 2 * row_ptr[i] + in_ptr[i] + i; };  // of vertices 0 .. i - 1
+    int at = 0;
+    for (int c = 0; c < 4; ++c) {
+        const int csize = 1 << c;
+        int32_t* v = split->data() + at;
+        at += csize + 1;
+        int32_t i = 0;
+        for (int r = 0; r <= csize; ++r) {
+            while (i < n && weight(i) < weight(n) * r / csize) ++i;
+            v[r] = r == csize ? n : i;
+        }
+        auto& p = ctx->cl[c];
+        p.max_n = p.max_m = p.max_chunks = 0;
+        for (int r = 0; r < csize; ++r) {
+            const int32_t dn = v[r + 1] - v[r];
+            const int32_t dm = (int32_t)(row_ptr[v[r + 1]] - row_ptr[v[r]]);
+            const int32_t dc = (int32_t)(chunks[v[r + 1]] - chunks[v[r]]);
+            if (dn > p.max_n) p.max_n = dn;
+            if (dm > p.max_m) p.max_m = dm;
+            if (dc > p.max_chunks) p.max_chunks = dc;
+        }
+    }
 }
 
-// The cluster engine (use_graph = 3, and the batched form's small
-// instances) applies to Alg. 1 and Program (6) on a small instance whose
-// edge variant is a lane-group form of at most 4 vectors per lane.
-bool cluster_eligible(const pdr_ctx* ctx, int p)
+// A cluster size for the current variant: blocks, threads and shared memory
+// of a block, the shares per lane, and the rounds its lane groups would need
+// over the edges with one share.
+struct ClusterShape {
+    int csize = 0, threads = 0, bytes = 0, shares = 1, rounds = 0;
+};
+bool cluster_shape(const pdr_ctx* ctx, int c, bool shared_sm, ClusterShape* out)
 {
-    const int cfg = ctx->cfg[p];
-    return !is_gd(ctx->opt) && ctx->m > 0 && ctx->m * (int64_t)ctx->Kp <= kBlockElems && batch_block_config(cfg) &&
-           edge_plain_config(cfg) <= 5;
+    const auto& p = ctx->cl[c];
+    if (p.max_m < 0) return false;
+    ClusterShape s;
+    s.csize = 1 << c;
+    s.bytes = cluster_bytes(p.max_n, p.max_m, p.max_chunks, ctx->Kp, s.csize);
+    if (s.bytes > kClusterSmemMax) return false;
+    // workers: a lane group per edge or a thread per (vertex, vector), whichever
+    // is more.  In a batch two blocks share an SM below 112 KB.
+    const int64_t edge_lanes = (int64_t)p.max_m * edge_group_lanes(ctx->cfg[0]);
+    const int64_t lanes = std::max<int64_t>(std::max<int64_t>(edge_lanes, (int64_t)p.max_n * (ctx->Kp / 4)), 32);
+    const int most = shared_sm && s.bytes <= 112 * 1024 ? 512 : 1024, dec = most - cluster_workers(most);
+    s.threads = (int)std::min<int64_t>(most, (lanes + 31) / 32 * 32 + dec);
+    s.rounds = (int)((edge_lanes + s.threads - dec - 1) / (s.threads - dec));
+    s.shares = cluster_shares(ctx->cfg[0], s.rounds <= 1 ? 1 : s.rounds <= 6 ? 2 : 4);
+    *out = s;
+    return true;
 }
 
-// Alg. 1 by the cluster kernel (use_graph = 3): one thread-block cluster runs
-// the excess pass, the objective and stop test and the edge QPs of every
-// sweep, separated by cluster barriers, for kBlockChunk sweeps per launch
-// until the stop rules fire; the flows start in buffer 0.  The per-element
-// arithmetic is the standalone kernels' (the batched form's engine, with one
-// instance).
-template <typename T>
+// The cluster engine runs FP32 sweeps of Alg. 1 and Program (6) on an
+// instance that fits in a cluster's shared memory and whose variant is a
+// lane-group form of at most 4 vectors per lane.  The engine options: 1 (the
+// default) takes it unless an excess form was asked for, 3 always.
+bool cluster_eligible(const pdr_ctx* ctx)
+{
+    const int cfg = ctx->cfg[0];
+    if (is_gd(ctx->opt) || cfg < 0 || edge_plain_config(cfg) > 5) return false;
+    if (ctx->opt.use_graph != 3 && (ctx->opt.use_graph != 1 || ctx->opt.excess_variant >= 0)) return false;
+    ClusterShape s;
+    return cluster_shape(ctx, 3, false, &s);
+}
+
+// One instance on its own: the smallest cluster whose lane groups take at
+// most kClusterRounds rounds over the edges, or the largest.
+constexpr int kClusterRounds = 2;
+ClusterShape cluster_alone(const pdr_ctx* ctx)
+{
+    ClusterShape s;
+    for (int c = 0; c < 4; ++c)
+        if (cluster_shape(ctx, c, false, &s) && s.rounds <= kClusterRounds) break;
+    return s;
+}
+
+ClusterArgs cluster_args(pdr_ctx* ctx, const ClusterShape& s, int par, bool first)
+{
+    ClusterArgs a{};
+    a.a = make_args<float>(ctx, MODE_SOLVE, 0, 0, par, 0);
+    int c = 0, at = 0;
+    for (; (1 << c) < s.csize; ++c) at += (1 << c) + 1;
+    a.v_start = ctx->cl_split + at;
+    a.max_n = ctx->cl[c].max_n;
+    a.max_m = ctx->cl[c].max_m;
+    a.max_chunks = ctx->cl[c].max_chunks;
+    a.csize = s.csize;
+    a.sweeps = kClusterChunk;
+    a.first = first ? 1 : 0;
+    return a;
+}
+
+// FP32 sweeps by the cluster engine until the stop rules fire, in launches of
+// kClusterChunk sweeps; the flows start in buffer 0.
 pdr_status run_cluster(pdr_ctx* ctx, int64_t t_start)
 {
-    const int p = Prec<T>::id;
-    if (!ctx->cl_args) {
-        pdr_status st = PDR_OK;
-        ctx->cl_args = dalloc<unsigned char>(ctx, sizeof(SweepArgs<double>) + 64, &st);
-        if (!ctx->cl_args) return st;
-    }
-    SweepArgs<T>* dargs = reinterpret_cast<SweepArgs<T>*>(ctx->cl_args);
-    int* dids = reinterpret_cast<int*>(ctx->cl_args + sizeof(SweepArgs<double>) + 32);
-    CK(cudaMemsetAsync(dids, 0, sizeof(int), ctx->stream));  // the instance id: 0, its arguments at dargs[0]
-    const int csize = batch_cluster_size(ctx, p);
+    const ClusterShape s = cluster_alone(ctx);
     for (bool first = true;; first = false) {
         const int par = first ? 0 : (int)((ctx->hst->t - t_start) & 1);
-        SweepArgs<T> a = make_args<T>(ctx, MODE_SOLVE, 0, 0, par, 0);
-        a.excess_form = 0;  // the gather form, run by the cluster's blocks
-        a.grid_v = csize;
-        a.grid_e = csize;
-        a.n_psi = csize * (kBatchThreads / 32);
-        a.pf_edges = 0;
-        a.l2_hints = 0;
-        a.active = nullptr;
-        CK(cudaMemcpyAsync(dargs, &a, sizeof(a), cudaMemcpyHostToDevice, ctx->stream));
-        CK(launch_batch_block<T>(edge_plain_config(ctx->cfg[p]), dargs, dids, 1, csize, kBlockChunk, first ? 1 : 0,
-                                 ctx->stream, block_smem(ctx, p)));
-        const pdr_status s = read_state(ctx);  // synchronises the stream
-        if (s != PDR_OK) return s;
+        CK(launch_cluster(ctx->cfg[0], s.shares, nullptr, nullptr, cluster_args(ctx, s, par, first), 1, s.csize, s.threads, s.bytes,
+                          ctx->stream));
+        const pdr_status st = read_state(ctx);  // synchronises the stream
+        if (st != PDR_OK) return st;
         if (ctx->hst->stop) break;
     }
     ctx->cur = (int)((ctx->hst->t - t_start) & 1);
     // the current flows' congestion partials in the standalone kernels' layout
-    return refresh_psi<T>(ctx, nullptr, true);
+    return refresh_psi<float>(ctx, nullptr, true);
 }
 
 // The persistent engine applies to Alg. 1 with a lane-group variant.
@@ -917,10 +982,10 @@ pdr_status run_phase(pdr_ctx* ctx, int64_t t_start)
     if (s != PDR_OK) return s;
     s = flows_to_buffer0<T>(ctx);
     if (s != PDR_OK) return s;
-    // one instance's FP64 sweeps stay on the graph engine: one block is held
-    // to one SM's FP64 rate, a small fraction of its FP32 rate on this GPU,
-    // and loses to the kernels that spread a sweep over several SMs
-    if (ctx->opt.use_graph == 3 && p == Prec<float>::id && cluster_eligible(ctx, p)) return run_cluster<T>(ctx, t_start);
+    // FP64 sweeps stay on the graph engine: a block is held to one SM's FP64
+    // rate, a small fraction of its FP32 rate on this GPU, and loses to the
+    // kernels that spread a sweep over every SM
+    if (p == Prec<float>::id && cluster_eligible(ctx)) return run_cluster(ctx, t_start);
     if (persistent_ok(ctx, p)) {
         bool ran = false;
         s = run_persistent<T>(ctx, &ran);
@@ -1277,7 +1342,7 @@ void pdr_destroy(pdr_ctx* ctx)
                    ctx->beta_buf[0], ctx->beta_buf[1], ctx->v32[0], ctx->v32[1], ctx->v64[0], ctx->v64[1],
                    ctx->r_h64, ctx->r_part, ctx->r_out, ctx->psi_tmp, ctx->bar, ctx->xv_start[1], ctx->xv_start[2], ctx->xv_start[3],
                    ctx->xv_start[4], ctx->xv_start[5],
-                   ctx->data_err, ctx->cl_args};
+                   ctx->data_err, ctx->cl_split};
     for (void* p : dev)
         if (p) cudaFree(p);
     release_adjoint_workspace(ctx);
@@ -1410,6 +1475,7 @@ pdr_status pdr_create(int32_t n, int64_t m, const int64_t* row_ptr, const int32_
     ALLOC(ctx->r_part, double, resid_part_count(ctx->r_grid_v, ctx->r_grid_e));
     ALLOC(ctx->r_out, ResidOut, 1);
     ALLOC(ctx->psi_tmp, double, m);
+    ALLOC(ctx->cl_split, int32_t, kClusterSplits);
     ALLOC(ctx->data_err, int, 4);  // error word, then the mean positive capacity (8-byte aligned)
     CKC(cudaMallocHost(&ctx->hst, sizeof(DevState)));
     CKC(cudaMallocHost(&ctx->hr_out, sizeof(ResidOut)));
@@ -1450,6 +1516,9 @@ pdr_status pdr_create(int32_t n, int64_t m, const int64_t* row_ptr, const int32_
     CKC(cudaMemcpyAsync(ctx->dem_f, dpf.data(), sizeof(float) * Kp, cudaMemcpyHostToDevice, ctx->stream));
     CKC(cudaMemcpyAsync(ctx->inv_dem_d, idd.data(), sizeof(double) * Kp, cudaMemcpyHostToDevice, ctx->stream));
     CKC(cudaMemcpyAsync(ctx->inv_dem_f, idf.data(), sizeof(float) * Kp, cudaMemcpyHostToDevice, ctx->stream));
+    std::vector<int32_t> split;
+    plan_clusters(ctx, row_ptr, col, &split);
+    CKC(cudaMemcpyAsync(ctx->cl_split, split.data(), sizeof(int32_t) * split.size(), cudaMemcpyHostToDevice, ctx->stream));
     CKC(build_adjacency(n, m, ctx->row_ptr, ctx->col, ctx->src, ctx->in_ptr, ctx->in_eid, ctx->inc_ptr, ctx->inc,
                         ctx->deg, ctx->work, ctx->stream));
     for (int f = 1; f < kExcessForms; ++f)
@@ -2304,10 +2373,10 @@ struct pdr_batch {
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
     std::vector<char> graph_mask[2];
     bool graph_tried[2] = {false, false}, graph_ok[2] = {false, false};
-    // one-block-per-instance engine: the instances one block solves at speed
-    void* bargs[2] = {nullptr, nullptr};  // device SweepArgs<float> / <double> [count]
-    int* bids = nullptr;                  // device instance ids [count], grouped by variant
-    void* hstage = nullptr;               // pinned staging of the arguments and ids
+    // cluster engine
+    void* bargs = nullptr;   // device ClusterArgs [count]
+    int* bids = nullptr;     // device instance ids [count], grouped by launch
+    void* hstage = nullptr;  // pinned staging of the arguments and ids
 };
 
 namespace {
@@ -2472,46 +2541,46 @@ fail:
 
 __global__ void set_counter_kernel(unsigned int* c, unsigned int v) { *c = v; }
 
-// Alg. 1 in precision T for the instances with run[i] set, from the states
-// their callers initialised (instance i's sweep counter starting at
-// t_start[i]); the others keep their stopped state.
-// Blocks of the cluster that solves an instance on the one-cluster-per-
-// instance engine: enough that each lane group of the cluster handles at
-// most about 16 edges per sweep (the edges of a group run one after the
-// other), a power of two up to 8.
-int batch_cluster_size(const pdr_ctx* c, int p)
+// Cluster sizes of a batch: every instance starts at the smallest cluster that
+// holds it, then, while the batch leaves SMs idle, the instances whose lane
+// groups take the most rounds are split further.
+void batch_shapes(const pdr_batch* b, const std::vector<int32_t>& live, std::vector<ClusterShape>* shapes)
 {
-    const int G = edge_group_lanes(c->cfg[p]);
-    const int64_t groups = (int64_t)(kBatchThreads / 32) * (32 / G);
-    const int64_t want = (c->m + groups * 16 - 1) / (groups * 16);
-    int cs = 1;
-    while (cs < want && cs < 8) cs <<= 1;
-    return cs;
+    shapes->assign(b->count, ClusterShape{});
+    std::vector<int> level(b->count, 0);
+    int64_t blocks = 0;
+    for (int32_t i : live) {
+        while (!cluster_shape(b->ctx[i], level[i], true, &(*shapes)[i])) ++level[i];  // 3 fits: cluster_eligible
+        blocks += (*shapes)[i].csize;
+    }
+    const int64_t sms = b->ctx[0]->num_sms;
+    for (;;) {
+        int32_t worst = -1;
+        for (int32_t i : live)
+            if (level[i] < 3 && (*shapes)[i].rounds > kClusterRounds &&
+                (worst < 0 || (*shapes)[i].rounds > (*shapes)[worst].rounds))
+                worst = i;
+        ClusterShape next;
+        if (worst < 0 || blocks + (*shapes)[worst].csize > sms || !cluster_shape(b->ctx[worst], level[worst] + 1, true, &next))
+            return;
+        ++level[worst];
+        blocks += next.csize - (*shapes)[worst].csize;
+        (*shapes)[worst] = next;
+    }
 }
 
-// True if instance i runs on the one-cluster-per-instance engine in
-// precision p (cluster_eligible: a small instance with a lane-group variant
-// of at most 4 vectors per lane; the larger ones spill at the block's
-// register budget).  FP64 sweeps run on the graph: one block has one SM's
-// FP64 rate, and the graph's kernels spread each instance over several SMs.
-bool batch_resident(const pdr_batch* b, int32_t i, int p)
+// The instances of `blk` (set up by batch_run) on the cluster engine:
+// launches of kClusterChunk sweeps, one per (variant, cluster size, threads)
+// on its own stream so that they run side by side, until every instance
+// stopped.  A finished instance's blocks leave and free their SM.
+pdr_status batch_cluster_run(pdr_batch* b, const std::vector<char>& blk, const std::vector<int64_t>& t_start)
 {
-    return p == Prec<float>::id && cluster_eligible(b->ctx[i], p);
-}
-
-// The instances of `blk` (set up by batch_run) on the one-block-per-instance
-// engine: launches of kBlockChunk sweeps, one per edge-kernel variant on its
-// own stream so that they run side by side, until every instance stopped.
-template <typename T>
-pdr_status batch_block_run(pdr_batch* b, const std::vector<char>& blk, const std::vector<int64_t>& t_start)
-{
-    const int p = Prec<T>::id;
     std::vector<int32_t> live;
     for (int32_t i = 0; i < b->count; ++i)
         if (blk[i]) live.push_back(i);
-    SweepArgs<T>* hargs = static_cast<SweepArgs<T>*>(b->hstage);
+    ClusterArgs* hargs = static_cast<ClusterArgs*>(b->hstage);
     int* hids = reinterpret_cast<int*>(hargs + b->count);
-    SweepArgs<T>* dargs = static_cast<SweepArgs<T>*>(b->bargs[p]);
+    ClusterArgs* dargs = static_cast<ClusterArgs*>(b->bargs);
     std::vector<cudaEvent_t> ev;
     auto done = [&](pdr_status st) {
         for (cudaEvent_t e : ev) cudaEventDestroy(e);
@@ -2520,85 +2589,63 @@ pdr_status batch_block_run(pdr_batch* b, const std::vector<char>& blk, const std
     auto cuda_err = [&](const char* what, cudaError_t e) {
         return done(batch_fail(PDR_ERR_CUDA, std::string("batch: ") + what + ": " + cudaGetErrorString(e)));
     };
-    for (int q = 0; q < 7; ++q) {  // the fork event and one per launch group (more on demand)
-        cudaEvent_t e;
-        const cudaError_t er = cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
-        if (er != cudaSuccess) return cuda_err("event", er);
-        ev.push_back(e);
-    }
     bool first = true;
     while (!live.empty()) {
+        std::vector<ClusterShape> shapes;
+        batch_shapes(b, live, &shapes);
         // arguments with the buffer parity of each instance's current flows
         for (int32_t i : live) {
             pdr_ctx* c = b->ctx[i];
-            const int par = first ? 0 : (int)((c->hst->t - t_start[i]) & 1);
-            const int csize = batch_cluster_size(c, p);
-            SweepArgs<T> a = make_args<T>(c, MODE_SOLVE, 0, 0, par, 0);
-            a.excess_form = 0;  // the gather form, run by the cluster's blocks
-            a.grid_v = csize;
-            a.grid_e = csize;
-            a.n_psi = csize * (kBatchThreads / 32);
-            a.pf_edges = 0;
-            a.l2_hints = 0;
-            a.active = nullptr;
-            hargs[i] = a;
+            hargs[i] = cluster_args(c, shapes[i], first ? 0 : (int)((c->hst->t - t_start[i]) & 1), first);
         }
-        // one launch per (lane-group variant, cluster size, form), largest
-        // clusters first; single blocks whose instance fits in shared memory
-        // run the shared-memory form, with the largest of their sizes
-        struct Group {
-            int cfg, csize, off, count;
-            int64_t smem;
+        // groups of one launch, the largest clusters first
+        std::vector<int32_t> order(live);
+        auto key = [&](int32_t i) {
+            return std::make_tuple(-shapes[i].csize, edge_plain_config(b->ctx[i]->cfg[0]), shapes[i].shares, -shapes[i].threads);
         };
-        std::vector<Group> groups;
-        int pos = 0;
-        for (int csize = 8; csize >= 1; csize >>= 1)
-            for (int cfg = 0; cfg <= 5; ++cfg)
-                for (int sm = 0; sm < (csize == 1 ? 2 : 1); ++sm) {
-                    const int off = pos;
-                    int64_t smem = 0;
-                    for (int32_t i : live) {
-                        const pdr_ctx* c = b->ctx[i];
-                        if (edge_plain_config(c->cfg[p]) != cfg || batch_cluster_size(c, p) != csize) continue;
-                        const int64_t need = csize == 1 ? block_smem(c, p) : 0;
-                        if ((need > 0) != (sm == 1)) continue;
-                        hids[pos++] = i;
-                        smem = need > smem ? need : smem;
-                    }
-                    if (pos > off) groups.push_back({cfg, csize, off, pos - off, smem});
-                }
-        cudaError_t e = cudaMemcpyAsync(dargs, hargs, sizeof(SweepArgs<T>) * b->count, cudaMemcpyHostToDevice,
-                                        b->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(b->bids, hids, sizeof(int) * pos, cudaMemcpyHostToDevice, b->stream);
-        if (e == cudaSuccess) e = cudaEventRecord(ev[0], b->stream);
-        for (size_t g = 0; g < groups.size() && e == cudaSuccess; ++g) {
-            while (ev.size() < g + 2) {
+        std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return key(x) < key(y); });
+        cudaError_t e = cudaSuccess;
+        std::copy(order.begin(), order.end(), hids);
+        auto event = [&](size_t k) {  // the k-th event, made on demand
+            while (ev.size() <= k && e == cudaSuccess) {
                 cudaEvent_t x;
                 e = cudaEventCreateWithFlags(&x, cudaEventDisableTiming);
-                if (e != cudaSuccess) break;
-                ev.push_back(x);
+                if (e == cudaSuccess) ev.push_back(x);
             }
-            if (e != cudaSuccess) break;
-            cudaStream_t sg = b->pool[g % b->pool.size()];
+            return e == cudaSuccess;
+        };
+        e = cudaMemcpyAsync(dargs, hargs, sizeof(ClusterArgs) * b->count, cudaMemcpyHostToDevice, b->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(b->bids, hids, sizeof(int) * order.size(), cudaMemcpyHostToDevice, b->stream);
+        if (e == cudaSuccess && event(0)) e = cudaEventRecord(ev[0], b->stream);
+        size_t group = 0;
+        for (size_t at = 0; at < order.size() && e == cudaSuccess; ++group) {
+            size_t end = at;
+            int bytes = 0;
+            while (end < order.size() && key(order[end]) == key(order[at])) {
+                bytes = std::max(bytes, shapes[order[end]].bytes);
+                ++end;
+            }
+            const ClusterShape& s = shapes[order[at]];
+            cudaStream_t sg = b->pool[group % b->pool.size()];
+            if (!event(group + 1)) break;
             e = cudaStreamWaitEvent(sg, ev[0], 0);
             if (e == cudaSuccess)
-                e = launch_batch_block<T>(groups[g].cfg, dargs, b->bids + groups[g].off, groups[g].count, groups[g].csize,
-                                          kBlockChunk, first ? 1 : 0, sg, groups[g].smem);
-            if (e == cudaSuccess) e = cudaEventRecord(ev[1 + g], sg);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, ev[1 + g], 0);
+                e = launch_cluster(b->ctx[order[at]]->cfg[0], s.shares, dargs, b->bids + at, ClusterArgs{}, (int)(end - at), s.csize,
+                                   s.threads, bytes, sg);
+            if (e == cudaSuccess) e = cudaEventRecord(ev[1 + group], sg);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, ev[1 + group], 0);
+            at = end;
         }
         for (size_t q = 0; q < live.size() && e == cudaSuccess; ++q) {
             pdr_ctx* c = b->ctx[live[q]];
             e = cudaMemcpyAsync(c->hst, c->st, sizeof(DevState), cudaMemcpyDeviceToHost, b->stream);
         }
         if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-        if (e != cudaSuccess) return cuda_err("one-block-per-instance engine", e);
+        if (e != cudaSuccess) return cuda_err("cluster engine", e);
         std::vector<int32_t> next;
-        for (int32_t i : live) {
-            if (b->ctx[i]->hst->fault)
-                return done(batch_fail(PDR_ERR_TIMEOUT, "instance " + std::to_string(i) + ": a device wait timed out"));
+        for (int32_t i : live)
             if (!b->ctx[i]->hst->stop) next.push_back(i);
-        }
         live.swap(next);
         first = false;
     }
@@ -2607,22 +2654,25 @@ pdr_status batch_block_run(pdr_batch* b, const std::vector<char>& blk, const std
         if (!blk[i]) continue;
         pdr_ctx* c = b->ctx[i];
         c->cur = (int)((c->hst->t - t_start[i]) & 1);
-        const pdr_status st = refresh_psi<T>(c, nullptr, true);
+        const pdr_status st = refresh_psi<float>(c, nullptr, true);
         if (st != PDR_OK) return done(st);
     }
     return done(PDR_OK);
 }
 
+// Alg. 1 in precision T for the instances with run_all[i] set, from the states
+// their callers initialised (instance i's sweep counter starting at
+// t_start[i]); the others keep their stopped state.
 template <typename T>
 pdr_status batch_run(pdr_batch* b, const std::vector<char>& run_all, const std::vector<int64_t>& t_start)
 {
     const int p = Prec<T>::id;
-    // small instances go to the one-block-per-instance engine, the others to the graph
+    // small instances go to the cluster engine, the others to the graph
     std::vector<char> blk(b->count, 0), run(run_all);
     bool any_blk = false;
     const bool use_graph = b->ctx[0]->opt.use_graph != 0;
     for (int32_t i = 0; i < b->count; ++i)
-        if (run_all[i] && use_graph && batch_resident(b, i, p)) {
+        if (run_all[i] && p == Prec<float>::id && cluster_eligible(b->ctx[i])) {
             blk[i] = 1;
             run[i] = 0;
             any_blk = true;
@@ -2638,7 +2688,7 @@ pdr_status batch_run(pdr_batch* b, const std::vector<char>& run_all, const std::
         if (run[i]) ++running;
     }
     if (any_blk) {
-        const pdr_status s = batch_block_run<T>(b, blk, t_start);
+        const pdr_status s = batch_cluster_run(b, blk, t_start);
         if (s != PDR_OK) return s;
     }
     if (running == 0) return PDR_OK;
@@ -2735,19 +2785,17 @@ pdr_status pdr_batch_create(int32_t count, const pdr_instance* inst, const pdr_o
     }
     b->tuned_cfg.assign(count, -1);
     b->tuned_us.assign(count, -1.0);
-    for (int p = 0; p < 2; ++p)
-        if (cudaMalloc(&b->bargs[p], sizeof(SweepArgs<double>) * count) != cudaSuccess) {
-            cudaGetLastError();
-            return give_up(PDR_ERR_OOM, "batch: argument table allocation failed");
-        }
-    if (cudaMalloc(&b->bids, sizeof(int) * count) != cudaSuccess ||
-        cudaMallocHost(&b->hstage, (sizeof(SweepArgs<double>) + sizeof(int)) * count) != cudaSuccess) {
+    if (cudaMalloc(&b->bargs, sizeof(ClusterArgs) * count) != cudaSuccess ||
+        cudaMalloc(&b->bids, sizeof(int) * count) != cudaSuccess ||
+        cudaMallocHost(&b->hstage, (sizeof(ClusterArgs) + sizeof(int)) * count) != cudaSuccess) {
         cudaGetLastError();
         return give_up(PDR_ERR_OOM, "batch: argument table allocation failed");
     }
     for (int32_t i = 0; i < count; ++i) {
         pdr_ctx* c = b->ctx[i];
-        if (o.edge_variant >= 0) {  // the caller's variant: no tuning
+        // the caller's variant, or the cluster engine (whose smallest lane group
+        // costs the fewest shuffles): no tuning
+        if (o.edge_variant >= 0 || (c->cur_prec == 0 && cluster_eligible(c))) {
             b->tuned_cfg[i] = c->cfg[c->cur_prec];
             continue;
         }
@@ -2867,8 +2915,7 @@ void pdr_batch_destroy(pdr_batch* b)
     for (cudaStream_t s : b->pool) cudaStreamDestroy(s);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
     if (b->active) cudaFree(b->active);
-    for (void* q : b->bargs)
-        if (q) cudaFree(q);
+    if (b->bargs) cudaFree(b->bargs);
     if (b->bids) cudaFree(b->bids);
     if (b->hstage) cudaFreeHost(b->hstage);
     cudaGetLastError();

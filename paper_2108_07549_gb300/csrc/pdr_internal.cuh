@@ -22,7 +22,6 @@
 namespace pdr {
 
 constexpr int kThreads = 256;  // block size of every sweep kernel
-constexpr int kBatchThreads = 512;  // block size of the one-block-per-instance batch kernel
 constexpr int kExcessForms = 6;     // excess kernel forms: 0 gathers, 1..5 bulk copies
 // Resident blocks per SM that the block forms of the edge kernels are
 // compiled for (the register cap that follows from it: 65,536 / (B x that)).
@@ -199,23 +198,30 @@ int excess_grid(int32_t n, int Kp, int vec, int num_sms, int resident_blocks);
 // of Alg. 1 or until the stop rules fire.  Only the lane-group variants.
 template <typename T>
 int persistent_grid(int cfg, int64_t m, int32_t n, int Kp, int num_sms);  // 0: not available
-// Batched form, one thread-block cluster of csize blocks (1, 2, 4 or 8) per
-// instance: instances ids[0..count) of args run up to `sweeps` sweeps each
-// with the lane-group variant cfg (true for batch_block_config);
-// psi_prologue: first launch of a solve.  smem > 0 (csize = 1 only, at most
-// kBlockSmemMax): the shared-memory form, each block holding its instance's
-// flows, heights, roots, partials and state in smem bytes of shared memory
-// (the largest block_smem_bytes of the instances launched).
-template <typename T>
-cudaError_t launch_batch_block(int cfg, const SweepArgs<T>* args, const int* ids, int count, int csize, int64_t sweeps,
-                               int psi_prologue, cudaStream_t stream, int64_t smem = 0);
-bool batch_block_config(int cfg);
-// Shared memory of the one-block form for an instance of n vertices, m edges,
-// rows of Kp values and n_psi edge partials, in bytes.
-template <typename T>
-int64_t block_smem_bytes(int64_t n, int64_t m, int64_t Kp, int64_t n_psi);
-// Largest shared-memory form: two blocks of it fit on one SM.
-constexpr int64_t kBlockSmemMax = 100 * 1024;
+// Cluster engine (cluster.cu): FP32 sweeps of Alg. 1 (or its capacity-kept
+// form) of a small instance in the shared memory of one thread-block cluster.
+constexpr int kClusterMax = 8;                    // blocks per cluster (the portable limit)
+constexpr int kClusterSmemMax = 224 * 1024;       // dynamic shared memory of a block
+struct ClusterArgs {
+    SweepArgs<float> a;      // f, theta_in: the buffers of the flows at the launch's start
+    const int32_t* v_start;  // [csize + 1] first vertex of each block (device)
+    // largest share of any block: vertices, out-edges, fours of incident rows
+    // (each vertex's in-edges and its out-edges rounded up apart)
+    int32_t max_n, max_m, max_chunks;
+    int32_t csize;
+    int32_t sweeps;          // at most this many in the launch (>= 1)
+    int32_t first;           // 1: the first launch of a solve
+};
+// Dynamic shared memory of a block, or more than kClusterSmemMax.
+int cluster_bytes(int max_n, int max_m, int max_chunks, int Kp, int csize);
+int cluster_workers(int threads);  // threads of a block that do sweep work
+// `count` clusters: instances table[ids[0..count)], or `one` where table is
+// NULL (count 1), all of csize blocks and the lane-group variant cfg
+// (edge_plain_config <= 5), whose lane groups run on 1 / shares of their lanes
+// (cluster_shares).
+int cluster_shares(int cfg, int want);
+cudaError_t launch_cluster(int cfg, int shares, const ClusterArgs* table, const int* ids, const ClusterArgs& one, int count,
+                           int csize, int threads, int bytes, cudaStream_t stream);
 
 // Packs and widens m padded rows into dst[rows*K] (double), dst writable by the GPU.
 template <typename T>

@@ -93,7 +93,6 @@ struct PairSum {
         two_sum(hi, x, hi, e);
         lo = __fadd_rn(lo, e);
     }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
 // Four consecutive elements of a padded row as doubles.

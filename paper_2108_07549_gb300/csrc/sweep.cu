@@ -24,7 +24,7 @@
 // active-set iteration of Michelot 1986 for projections onto a simplex,
 // applied to this problem).  Each round is one group-wide sum and count held
 // in registers, so no row is sorted or re-read.
-#include "sweep_common.cuh"
+#include "edge_root.cuh"
 #include "widen.cuh"
 
 namespace pdr {
@@ -38,14 +38,13 @@ __global__ void __launch_bounds__(kThreads) finalize_kernel(SweepArgs<T> a)
 
 // ------------------------------------------------------------------ excess and heights
 
-template <typename T, bool SH = false>
+template <typename T>
 __device__ __forceinline__ void excess_tail(const SweepArgs<T>& a, int block, int nblocks,
                                             typename Acc<T>::V zacc, T cons);
 
 // Body of one excess pass run by block `block` of `nblocks` (the standalone
-// kernel passes its own grid; the persistent kernel its whole grid).  SH:
-// the objective partials live in shared memory (the one-block engine).
-template <typename T, bool SH = false>
+// kernel passes its own grid; the persistent kernel its whole grid).
+template <typename T>
 __device__ __forceinline__ void excess_body(const SweepArgs<T>& a, int block, int nblocks)
 {
     using VT = typename VecOf<T>::type;
@@ -136,26 +135,26 @@ __device__ __forceinline__ void excess_body(const SweepArgs<T>& a, int block, in
         }
         zacc = A::add(zacc, zt);
     }
-    excess_tail<T, SH>(a, block, nblocks, zacc, cons);
+    excess_tail<T>(a, block, nblocks, zacc, cons);
 }
 
 // End of an excess pass in every block: add this block's fixed slice of the
 // edge kernel's psi partials and write the block's three partials.  Every
 // thread of the block calls it.
-template <typename T, bool SH>
+template <typename T>
 __device__ __forceinline__ void excess_tail(const SweepArgs<T>& a, int block, int nblocks,
                                             typename Acc<T>::V zacc, T cons)
 {
     using A = Acc<T>;
     T capb = T(0);
     {
-        // the block's slice [lo, hi) of the edge partials (SH: the one block takes all)
-        const int64_t lo = SH ? 0 : (int64_t)block * a.n_psi / nblocks;
-        const int64_t hi = SH ? a.n_psi : (int64_t)(block + 1) * a.n_psi / nblocks;
+        // the block's slice [lo, hi) of the edge partials
+        const int64_t lo = (int64_t)block * a.n_psi / nblocks;
+        const int64_t hi = (int64_t)(block + 1) * a.n_psi / nblocks;
         const typename A::S* pp = reinterpret_cast<const typename A::S*>(a.part_psi);
         for (int64_t b = lo + threadIdx.x; b < hi; b += blockDim.x) {
-            zacc = A::add(zacc, A::unstore(ld_part<SH>(pp + b)));
-            const T c = ld_part<SH>(a.part_cap + b);
+            zacc = A::add(zacc, A::load(pp + b));
+            const T c = __ldcg(a.part_cap + b);
             capb = c > capb ? c : capb;
         }
     }
@@ -470,136 +469,6 @@ __global__ void excess_split_kernel(const int64_t* inc_ptr, int32_t n, int grid,
     xv_start[b] = lo;
 }
 
-// ------------------------------------------------------------------ the root search of Alg. 2
-//
-// Every pass over a row returns three group-wide values for a threshold w:
-// S(w) = sum of the c_k > w, n(w) = their number and m(w) = the smallest of
-// them.  theta = (S(w) - u)/(2 + n(w)) is the root of the active set
-// A = {c > w}; if m(w) > theta, no element of A falls at or below theta, so A
-// is the active set of its own root and the search ends without another
-// pass.  Otherwise the elements c <= theta leave (Michelot's step) and the
-// next pass starts at theta.  In a converged solve the warm start w lies just
-// below the root with no element in between, so one pass decides the edge.
-
-template <int G, typename X>
-__device__ __forceinline__ X group_min(X x)
-{
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) {
-        const X y = __shfl_xor_sync(kFull, x, o);
-        x = y < x ? y : x;
-    }
-    return x;
-}
-
-template <typename T, int G, int V, int N>
-__device__ __forceinline__ void above(const T (&c)[V][N], T w, T& S, int& n, T& mn)
-{
-    T sl = T(0), ml = T(INFINITY);
-    int nl = 0;
-#pragma unroll
-    for (int q = 0; q < V; ++q)
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-            const T x = c[q][j];
-            if (x > w) {
-                sl += x;
-                ++nl;
-                ml = x < ml ? x : ml;
-            }
-        }
-    S = group_sum<G>(sl);
-    if constexpr (G == 32 && sizeof(T) == 4) {
-        // whole-warp groups: one redux each for the count and the minimum
-        // (every counted x exceeds w >= 0, so ml is positive or +inf and its
-        // bit pattern orders as an unsigned integer)
-        n = (int)__reduce_add_sync(kFull, (unsigned)nl);
-        mn = __uint_as_float(__reduce_min_sync(kFull, __float_as_uint(ml)));
-    } else {
-        n = group_sum<G>(nl);
-        mn = group_min<G>(ml);
-    }
-}
-
-// Case decision and root from the sums above a threshold w >= 0 that is known
-// to lie at or below the root (w = 0, or g(w) >= 0 certified).  den = 2 for
-// Alg. 2 (the congestion term of eq. (10) gives theta = (S_A - u)/(2 + |A|));
-// den = 0 with the capacity kept (Program (6): sum_A (c - theta) = u).
-template <typename T>
-__device__ __forceinline__ void start_root(T S, int n, T mn, T ue, int den, T& theta, int& nA, bool& done)
-{
-    if (S <= ue) {  // Case 1 of Alg. 2: nothing to shed
-        theta = T(0);
-        done = true;
-    } else {  // Case 2 (S > u >= 0, so n >= 1)
-        theta = (S - ue) / T(den + n);
-        nA = n;
-        done = mn > theta;
-    }
-}
-
-// theta = psi'/2 for the row c (all lanes of the warp call it; `valid` is
-// uniform over the lane group).  w0 is the warm start (>= 0).
-template <typename T, int G, int V, int N>
-__device__ __forceinline__ T qp_root_group(const T (&c)[V][N], T ue, T w0, bool valid, int Kp, int den)
-{
-    T S, mn, theta = T(0);
-    int n, nA = 0;
-    bool done = !valid, cold = false;
-    above<T, G, V, N>(c, w0, S, n, mn);
-    if (valid) {
-        if (w0 <= T(0)) start_root(S, n, mn, ue, den, theta, nA, done);
-        else if (n > 0 && S - T(n) * w0 - ue - T(den) * w0 >= T(0)) {
-            // g(w0) = sum max(0, c - w0) - u - den w0 >= 0: w0 <= root, Case 2
-            theta = (S - ue) / T(den + n);
-            nA = n;
-            done = mn > theta;
-        } else {
-            cold = true;  // the root dropped below the warm start
-        }
-    }
-    if (__any_sync(kFull, cold)) {
-        T S0, m0;
-        int n0;
-        above<T, G, V, N>(c, T(0), S0, n0, m0);
-        if (cold) start_root(S0, n0, m0, ue, den, theta, nA, done);
-    }
-    for (int it = 0; __any_sync(kFull, !done); ++it) {
-        T S2, m2;
-        int n2;
-        above<T, G, V, N>(c, theta, S2, n2, m2);
-        if (!done) {
-            if (n2 >= nA || n2 == 0) done = true;  // no element left: keep theta
-            else {
-                nA = n2;
-                theta = (S2 - ue) / T(den + n2);
-                done = m2 > theta;
-            }
-        }
-        if (it > Kp + 2) break;  // unreachable: nA drops every round
-    }
-    // A Case 2 root below 0 can only come from rounding in sums that put
-    // s = sum max(0, c) within rounding of u: that edge is in Case 1 (root 0).
-    // Without the clamp, f' = max(0, c - theta) would lift every c <= 0 --
-    // the zero padding included -- to -theta.
-    return theta > T(0) ? theta : T(0);
-}
-
-// Warm start of the next sweep's root search from this sweep's root theta
-// and the previous one, prev.  A root that rose is expected to stay at or
-// above theta; one that fell is expected to fall by about as much again.
-// Starting the search at the previous root itself leaves out the many
-// entries whose flows have decayed to zero, which sit just above it (c_k =
-// theta + f'_k): one pass decides almost every edge.  A start above the
-// new root is detected by its certificate g(w) < 0 and costs a cold pass.
-template <typename T>
-__device__ __forceinline__ T next_warm_start(T theta, T prev)
-{
-    if (theta > prev) return theta;
-    const T w = T(0.999) * theta + T(2) * (theta - prev);
-    return w > T(0) ? w : T(0);
-}
-
 // ------------------------------------------------------------------ edge QP, lane-group form
 
 // One aligned group of G lanes per edge; each lane keeps V vectors of the
@@ -861,6 +730,7 @@ __global__ void __launch_bounds__(kThreads, 2) edge_pipe_kernel(SweepArgs<T> a)
 template <typename T, int V, int N>
 __device__ __forceinline__ void block_above(const T (&c)[V][N], T w, T& S, int& n, T& mn, T* sa, int* sb, T* sm)
 {
+    __syncwarp();  // a branch of thread 0 alone may lie just before
     T sl = T(0), ml = T(INFINITY);
     int nl = 0;
 #pragma unroll
@@ -963,29 +833,16 @@ __global__ void __launch_bounds__(B, block_min_blocks(B, V)) edge_block_kernel(S
         T psi;
         if (!psi_only) {
             // the lane-group search with block-wide sums, counts and minima
-            const T w0 = a.theta_in[a.m + e];
             const int den = a.ck ? 0 : 2;
-            T S, mn, theta = T(0);
-            int n, nA = 0;
-            bool done = false;
-            block_above<T, V, N>(c, w0, S, n, mn, sa_buf, sb_buf, sm_buf);
-            if (w0 <= T(0)) start_root(S, n, mn, ue, den, theta, nA, done);
-            else if (n > 0 && S - T(n) * w0 - ue - T(den) * w0 >= T(0)) {
-                theta = (S - ue) / T(den + n);
-                nA = n;
-                done = mn > theta;
-            } else {
-                block_above<T, V, N>(c, T(0), S, n, mn, sa_buf, sb_buf, sm_buf);
-                start_root(S, n, mn, ue, den, theta, nA, done);
-            }
-            for (int it = 0; !done && it <= a.Kp + 2; ++it) {  // block-uniform
-                block_above<T, V, N>(c, theta, S, n, mn, sa_buf, sb_buf, sm_buf);
-                if (n >= nA || n == 0) break;
-                nA = n;
-                theta = (S - ue) / T(den + n);
-                done = mn > theta;
-            }
-            if (theta < T(0)) theta = T(0);  // a root below 0 is rounding at s = u: Case 1 (as qp_root_group)
+            RootSearch<T> rs(a.theta_in[a.m + e], true);
+            int it = 0;
+            do {  // block-uniform
+                T S, mn;
+                int n;
+                block_above<T, V, N>(c, rs.w, S, n, mn, sa_buf, sb_buf, sm_buf);
+                rs.step(S, n, mn, ue, den);
+            } while (!rs.done && ++it <= a.Kp + 4);
+            const T theta = rs.root();
             if (threadIdx.x == 0) {
                 a.theta[a.m + e] = next_warm_start(theta, a.theta_in[e]);
                 a.theta[e] = theta;
@@ -1229,32 +1086,20 @@ __global__ void __launch_bounds__(B, 1) edge_staged_kernel(SweepArgs<T> a)
         }
         __syncthreads();  // every row is in registers: the staging buffer is free
         if (threadIdx.x == 0 && e + nb < a.m) stage(e + nb);
+        __syncwarp();  // thread 0 back with its warp before the search's barriers
         T* orow = a.f_out + e * a.Kp;
         T psi;
         if (!psi_only) {
-            const T w0 = a.theta_in[a.m + e];
             const int den = a.ck ? 0 : 2;
-            T S, mn, theta = T(0);
-            int n, nA = 0;
-            bool done = false;
-            block_above<T, V, N>(c, w0, S, n, mn, sa_buf, sb_buf, sm_buf);
-            if (w0 <= T(0)) start_root(S, n, mn, ue, den, theta, nA, done);
-            else if (n > 0 && S - T(n) * w0 - ue - T(den) * w0 >= T(0)) {
-                theta = (S - ue) / T(den + n);
-                nA = n;
-                done = mn > theta;
-            } else {
-                block_above<T, V, N>(c, T(0), S, n, mn, sa_buf, sb_buf, sm_buf);
-                start_root(S, n, mn, ue, den, theta, nA, done);
-            }
-            for (int it = 0; !done && it <= a.Kp + 2; ++it) {  // block-uniform
-                block_above<T, V, N>(c, theta, S, n, mn, sa_buf, sb_buf, sm_buf);
-                if (n >= nA || n == 0) break;
-                nA = n;
-                theta = (S - ue) / T(den + n);
-                done = mn > theta;
-            }
-            if (theta < T(0)) theta = T(0);  // a root below 0 is rounding at s = u: Case 1
+            RootSearch<T> rs(a.theta_in[a.m + e], true);
+            int it = 0;
+            do {  // block-uniform
+                T S, mn;
+                int n;
+                block_above<T, V, N>(c, rs.w, S, n, mn, sa_buf, sb_buf, sm_buf);
+                rs.step(S, n, mn, ue, den);
+            } while (!rs.done && ++it <= a.Kp + 4);
+            const T theta = rs.root();
             if (threadIdx.x == 0) {
                 a.theta[a.m + e] = next_warm_start(theta, a.theta_in[e]);
                 a.theta[e] = theta;
@@ -1292,210 +1137,6 @@ __global__ void __launch_bounds__(B, 1) edge_staged_kernel(SweepArgs<T> a)
     if (threadIdx.x == 0) {
         reinterpret_cast<typename A::S*>(a.part_psi)[blockIdx.x] = A::store(zpsi);
         a.part_cap[blockIdx.x] = capmax;
-    }
-}
-
-// ------------------------------------------------------------------ batched form: one cluster per instance
-//
-// For a batch of small instances one launch runs every instance's solve: the
-// csize consecutive blocks of a thread-block cluster own instance
-// ids[blockIdx.x / csize] and run Alg. 1 sweep after sweep -- the excess
-// pass, the objective and stop test, then (unless it stopped) the edge QPs --
-// separated only by cluster barriers (block barriers for csize = 1), until
-// its own stop rule fires or `sweeps` sweeps are done.  A finished instance's
-// blocks leave and free their SM slots, which is the per-instance
-// convergence mask.  Per element the arithmetic and its order are those of
-// the standalone kernels with the same lane-group variant, so the flows equal
-// theirs bit for bit; the objective's partials are grouped per block (z
-// agrees to rounding).  The flows start in the buffer args[i] names and every
-// applied sweep swaps the buffers.
-
-// All threads of the cluster; release/acquire at cluster scope orders the
-// global-memory writes of one phase before the reads of the next.
-__device__ __forceinline__ void cluster_sync_all()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// Shared-memory form (SM, one block per instance): the block copies the
-// instance's mutable arrays -- both flow buffers, the heights, both root
-// buffers, the objective partials -- and its solver state into shared
-// memory, with the read-only arrays the sweep reads (incidence lists,
-// commodities, capacities, endpoints, scales), runs its sweeps there, and
-// copies the mutable ones back before it returns.  The phases then pass
-// their data through shared memory instead of L2, whose latency is what a
-// sweep of a small instance waits on.  The arithmetic and the order of
-// every reduction are unchanged, so flows, roots, z and the stop sweep
-// equal the global-memory form's bit for bit.  Layout (each part 16-byte
-// aligned): f buffer 0 and 1 [m][Kp], h [n][Kp], roots 0 and 1 [2m], psi
-// partials [n_psi] (stored pairs) and [n_psi], excess partials (one each),
-// then inc_ptr [n+1], inc [2m], s, t, dem, 1/d [Kp], u, src, col,
-// 1/scale [m], 1/delta [n].
-template <typename T>
-struct BlockSmem {
-    int64_t f0, f1, h, th0, th1, ppsi, pcap, ph, pcons, pcapb;
-    int64_t incp, inc, s, t, dem, idem, u, src, col, isc, ideg, bytes;
-};
-
-template <typename T>
-__host__ __device__ inline BlockSmem<T> block_smem_layout(int64_t n, int64_t m, int64_t Kp, int64_t n_psi)
-{
-    auto up = [](int64_t x) { return (x + 15) & ~int64_t(15); };
-    BlockSmem<T> L{};
-    int64_t o = 0;
-    L.f0 = o;    o = up(o + m * Kp * (int64_t)sizeof(T));
-    L.f1 = o;    o = up(o + m * Kp * (int64_t)sizeof(T));
-    L.h = o;     o = up(o + n * Kp * (int64_t)sizeof(T));
-    L.th0 = o;   o = up(o + 2 * m * (int64_t)sizeof(T));
-    L.th1 = o;   o = up(o + 2 * m * (int64_t)sizeof(T));
-    L.ppsi = o;  o = up(o + n_psi * (int64_t)sizeof(typename Acc<T>::S));
-    L.pcap = o;  o = up(o + n_psi * (int64_t)sizeof(T));
-    L.ph = o;    o = up(o + (int64_t)sizeof(double));
-    L.pcons = o; o = up(o + (int64_t)sizeof(T));
-    L.pcapb = o; o = up(o + (int64_t)sizeof(T));
-    L.incp = o;  o = up(o + (n + 1) * (int64_t)sizeof(int64_t));
-    L.inc = o;   o = up(o + 2 * m * (int64_t)sizeof(int32_t));
-    L.s = o;     o = up(o + Kp * (int64_t)sizeof(int32_t));
-    L.t = o;     o = up(o + Kp * (int64_t)sizeof(int32_t));
-    L.dem = o;   o = up(o + Kp * (int64_t)sizeof(T));
-    L.idem = o;  o = up(o + Kp * (int64_t)sizeof(T));
-    L.u = o;     o = up(o + m * (int64_t)sizeof(T));
-    L.src = o;   o = up(o + m * (int64_t)sizeof(int32_t));
-    L.col = o;   o = up(o + m * (int64_t)sizeof(int32_t));
-    L.isc = o;   o = up(o + m * (int64_t)sizeof(T));
-    L.ideg = o;  o = up(o + n * (int64_t)sizeof(T));
-    L.bytes = o;
-    return L;
-}
-
-// count elements of X from src to dst by the whole block
-template <typename X>
-__device__ __forceinline__ void block_copy(X* __restrict__ dst, const X* __restrict__ src, int64_t count)
-{
-    for (int64_t q = threadIdx.x; q < count; q += blockDim.x) dst[q] = src[q];
-}
-
-template <typename T, int G, int V, bool SM>
-__global__ void __launch_bounds__(kBatchThreads, 2)
-    batch_block_kernel(const SweepArgs<T>* __restrict__ args, const int* __restrict__ ids, int csize,
-                       int64_t sweeps, int psi_prologue)
-{
-    using VT = typename VecOf<T>::type;
-    using S = typename Acc<T>::S;
-    // the instance's arguments live in shared memory (not in every thread's
-    // registers); thread 0 of every block swaps its buffers between sweeps
-    __shared__ SweepArgs<T> sa;
-    __shared__ int stop;
-    __shared__ DevState sst;  // SM: the solver state while the block runs
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int rank = (int)(blockIdx.x % (unsigned)csize);
-    auto sync = [csize]() {
-        if (csize > 1) cluster_sync_all();
-        else __syncthreads();
-    };
-    if (threadIdx.x == 0) {
-        sa = args[ids[blockIdx.x / (unsigned)csize]];
-        stop = reinterpret_cast<volatile DevState*>(sa.st)->stop;
-        if (psi_prologue) sa.mode = MODE_PSI;
-    }
-    __syncthreads();
-    if (stop) return;  // the same value in every block of the cluster (no block of it has run yet)
-    // SM: the global buffers, to which the shared copies return at the end
-    T* const gf0 = sa.f;
-    T* const gf1 = sa.f_out;
-    T* const gh = sa.h;
-    T* const gth0 = const_cast<T*>(sa.theta_in);
-    T* const gth1 = sa.theta;
-    S* const gpsi = reinterpret_cast<S*>(sa.part_psi);
-    T* const gcap = sa.part_cap;
-    DevState* const gst = sa.st;
-    const BlockSmem<T> L = block_smem_layout<T>(sa.n, sa.m, sa.Kp, sa.n_psi);
-    if constexpr (SM) {
-        const int64_t rowv = sa.m * sa.Kp / VecOf<T>::N;
-        block_copy(reinterpret_cast<VT*>(smem + L.f0), reinterpret_cast<const VT*>(gf0), rowv);
-        block_copy(reinterpret_cast<VT*>(smem + L.f1), reinterpret_cast<const VT*>(gf1), rowv);
-        block_copy(reinterpret_cast<VT*>(smem + L.h), reinterpret_cast<const VT*>(gh),
-                   (int64_t)sa.n * sa.Kp / VecOf<T>::N);
-        block_copy(reinterpret_cast<T*>(smem + L.th0), gth0, 2 * sa.m);
-        block_copy(reinterpret_cast<T*>(smem + L.th1), gth1, 2 * sa.m);
-        block_copy(reinterpret_cast<S*>(smem + L.ppsi), gpsi, sa.n_psi);
-        block_copy(reinterpret_cast<T*>(smem + L.pcap), gcap, sa.n_psi);
-        block_copy(reinterpret_cast<int64_t*>(smem + L.incp), sa.inc_ptr, (int64_t)sa.n + 1);
-        block_copy(reinterpret_cast<int32_t*>(smem + L.inc), sa.inc, 2 * sa.m);
-        block_copy(reinterpret_cast<int32_t*>(smem + L.s), sa.s, (int64_t)sa.Kp);
-        block_copy(reinterpret_cast<int32_t*>(smem + L.t), sa.t, (int64_t)sa.Kp);
-        block_copy(reinterpret_cast<T*>(smem + L.dem), sa.dem, (int64_t)sa.Kp);
-        block_copy(reinterpret_cast<T*>(smem + L.idem), sa.inv_dem, (int64_t)sa.Kp);
-        block_copy(reinterpret_cast<T*>(smem + L.u), sa.u, sa.m);
-        block_copy(reinterpret_cast<int32_t*>(smem + L.src), sa.src, sa.m);
-        block_copy(reinterpret_cast<int32_t*>(smem + L.col), sa.col, sa.m);
-        block_copy(reinterpret_cast<T*>(smem + L.isc), sa.inv_scale_t, sa.m);
-        block_copy(reinterpret_cast<T*>(smem + L.ideg), sa.inv_deg, (int64_t)sa.n);
-        __syncthreads();  // every thread has read sa's global pointers
-        if (threadIdx.x == 0) {
-            sst = *gst;
-            sa.f = reinterpret_cast<T*>(smem + L.f0);
-            sa.f_out = reinterpret_cast<T*>(smem + L.f1);
-            sa.h = reinterpret_cast<T*>(smem + L.h);
-            sa.theta_in = reinterpret_cast<const T*>(smem + L.th0);
-            sa.theta = reinterpret_cast<T*>(smem + L.th1);
-            sa.part_psi = smem + L.ppsi;
-            sa.part_cap = reinterpret_cast<T*>(smem + L.pcap);
-            sa.part_h = reinterpret_cast<double*>(smem + L.ph);
-            sa.part_cons = reinterpret_cast<T*>(smem + L.pcons);
-            sa.part_capb = reinterpret_cast<T*>(smem + L.pcapb);
-            sa.inc_ptr = reinterpret_cast<const int64_t*>(smem + L.incp);
-            sa.inc = reinterpret_cast<const int32_t*>(smem + L.inc);
-            sa.s = reinterpret_cast<const int32_t*>(smem + L.s);
-            sa.t = reinterpret_cast<const int32_t*>(smem + L.t);
-            sa.dem = reinterpret_cast<const T*>(smem + L.dem);
-            sa.inv_dem = reinterpret_cast<const T*>(smem + L.idem);
-            sa.u = reinterpret_cast<const T*>(smem + L.u);
-            sa.src = reinterpret_cast<const int32_t*>(smem + L.src);
-            sa.col = reinterpret_cast<const int32_t*>(smem + L.col);
-            sa.inv_scale_t = reinterpret_cast<const T*>(smem + L.isc);
-            sa.inv_deg = reinterpret_cast<const T*>(smem + L.ideg);
-            sa.st = &sst;
-        }
-        __syncthreads();
-    }
-    if (psi_prologue) {  // congestion partials of the starting flows, in this kernel's layout
-        edge_group_body<T, G, V, true>(sa, rank, csize);
-        sync();
-        if (threadIdx.x == 0) sa.mode = MODE_SOLVE;
-        __syncthreads();
-    }
-    for (int64_t q = 0; q < sweeps; ++q) {
-        excess_body<T, SM>(sa, rank, csize);
-        sync();
-        if (rank == 0) reduce_and_finalize<T, SM>(sa);
-        sync();
-        if (threadIdx.x == 0) stop = reinterpret_cast<volatile DevState*>(sa.st)->stop;
-        __syncthreads();
-        if (stop) break;  // f^(t) stays in sa.f
-        edge_group_body<T, G, V, true>(sa, rank, csize);
-        sync();
-        if (threadIdx.x == 0) {  // f^(t+1) becomes the current flows
-            T* f = sa.f;
-            sa.f = sa.f_out;
-            sa.f_out = f;
-            const T* th = sa.theta_in;
-            sa.theta_in = sa.theta;
-            sa.theta = const_cast<T*>(th);
-        }
-        __syncthreads();
-    }
-    if constexpr (SM) {  // every buffer back to its global counterpart
-        const int64_t rowv = sa.m * sa.Kp / VecOf<T>::N;
-        block_copy(reinterpret_cast<VT*>(gf0), reinterpret_cast<const VT*>(smem + L.f0), rowv);
-        block_copy(reinterpret_cast<VT*>(gf1), reinterpret_cast<const VT*>(smem + L.f1), rowv);
-        block_copy(reinterpret_cast<VT*>(gh), reinterpret_cast<const VT*>(smem + L.h),
-                   (int64_t)sa.n * sa.Kp / VecOf<T>::N);
-        block_copy(gth0, reinterpret_cast<const T*>(smem + L.th0), 2 * sa.m);
-        block_copy(gth1, reinterpret_cast<const T*>(smem + L.th1), 2 * sa.m);
-        block_copy(gpsi, reinterpret_cast<const S*>(smem + L.ppsi), sa.n_psi);
-        block_copy(gcap, reinterpret_cast<const T*>(smem + L.pcap), sa.n_psi);
-        if (threadIdx.x == 0) *gst = sst;
     }
 }
 
@@ -1861,67 +1502,6 @@ int persistent_grid(int cfg, int64_t m, int32_t n, int Kp, int num_sms)
     const int64_t cap = (int64_t)num_sms * per_sm;
     if (g > cap) g = cap;
     return g < 2 ? 2 : (int)g;
-}
-
-template <typename T, int G, int V>
-cudaError_t launch_batch_block_gv(const SweepArgs<T>* args, const int* ids, int count, int csize, int64_t sweeps,
-                                  int psi_prologue, cudaStream_t stream, int64_t smem)
-{
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(count * csize));
-    cfg.blockDim = dim3(kBatchThreads);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = (unsigned)csize;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = csize > 1 ? 1 : 0;
-    if (smem > 0) {
-        const cudaError_t e = cudaFuncSetAttribute(batch_block_kernel<T, G, V, true>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        cfg.dynamicSmemBytes = (size_t)smem;
-        return cudaLaunchKernelEx(&cfg, batch_block_kernel<T, G, V, true>, args, ids, csize, sweeps, psi_prologue);
-    }
-    return cudaLaunchKernelEx(&cfg, batch_block_kernel<T, G, V, false>, args, ids, csize, sweeps, psi_prologue);
-}
-
-template <typename T>
-cudaError_t launch_batch_block(int cfg, const SweepArgs<T>* args, const int* ids, int count, int csize, int64_t sweeps,
-                               int psi_prologue, cudaStream_t stream, int64_t smem)
-{
-    if (count <= 0) return cudaSuccess;
-    if (csize < 1 || csize > 8 || (csize & (csize - 1))) return cudaErrorInvalidValue;
-    if (smem < 0 || smem > kBlockSmemMax || (smem > 0 && csize != 1)) return cudaErrorInvalidValue;
-    switch (edge_plain_config(cfg)) {
-    case 0: return launch_batch_block_gv<T, 4, 1>(args, ids, count, csize, sweeps, psi_prologue, stream, smem);
-    case 1: return launch_batch_block_gv<T, 8, 1>(args, ids, count, csize, sweeps, psi_prologue, stream, smem);
-    case 2: return launch_batch_block_gv<T, 16, 1>(args, ids, count, csize, sweeps, psi_prologue, stream, smem);
-    case 3: return launch_batch_block_gv<T, 32, 1>(args, ids, count, csize, sweeps, psi_prologue, stream, smem);
-    case 4: return launch_batch_block_gv<T, 32, 2>(args, ids, count, csize, sweeps, psi_prologue, stream, smem);
-    case 5: return launch_batch_block_gv<T, 32, 4>(args, ids, count, csize, sweeps, psi_prologue, stream, smem);
-    default: return cudaErrorInvalidValue;
-    }
-}
-template cudaError_t launch_batch_block<float>(int, const SweepArgs<float>*, const int*, int, int, int64_t, int,
-                                               cudaStream_t, int64_t);
-template cudaError_t launch_batch_block<double>(int, const SweepArgs<double>*, const int*, int, int, int64_t, int,
-                                                cudaStream_t, int64_t);
-
-template <typename T>
-int64_t block_smem_bytes(int64_t n, int64_t m, int64_t Kp, int64_t n_psi)
-{
-    return block_smem_layout<T>(n, m, Kp, n_psi).bytes;
-}
-template int64_t block_smem_bytes<float>(int64_t, int64_t, int64_t, int64_t);
-template int64_t block_smem_bytes<double>(int64_t, int64_t, int64_t, int64_t);
-
-bool batch_block_config(int cfg)
-{
-    const int c = edge_plain_config(cfg);
-    return c >= 0 && c < kNumCfg && kCfg[c].G > 0;
 }
 
 template <typename T>

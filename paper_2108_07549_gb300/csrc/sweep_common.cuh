@@ -308,7 +308,6 @@ struct Acc<float> {
     }
     static __device__ __forceinline__ S store(V a) { return make_float2(a.hi, a.lo); }
     static __device__ __forceinline__ V load(const S* p) { const float2 x = __ldcg(p); return {x.x, x.y}; }
-    static __device__ __forceinline__ V unstore(S x) { return {x.x, x.y}; }
     static __device__ __forceinline__ bool nonzero(V a) { return a.hi != 0.f || a.lo != 0.f; }
     static __device__ __forceinline__ double to_double(V a) { return (double)a.hi + (double)a.lo; }
 };
@@ -322,7 +321,6 @@ struct Acc<double> {
     static __device__ __forceinline__ V shfl(V a, int o) { return __shfl_xor_sync(kFull, a, o); }
     static __device__ __forceinline__ S store(V a) { return a; }
     static __device__ __forceinline__ V load(const S* p) { return __ldcg(p); }
-    static __device__ __forceinline__ V unstore(S x) { return x; }
     static __device__ __forceinline__ bool nonzero(V a) { return a != 0.0; }
     static __device__ __forceinline__ double to_double(V a) { return a; }
 };
@@ -437,111 +435,104 @@ __device__ void stop_from_kernel(const SweepArgs<T>& a)
     if (a.use_cond && last) cudaGraphSetConditional(a.cond, 0);
 }
 
-// Alg. 1: z = 1/2 sum psi^2 + 1/2 sum delta h^2 and the stop test, run by one
-// thread after every partial of this sweep is final.
-template <typename T>
-__device__ void finalize(const SweepArgs<T>& a, double zsum, double cons, double cap)
+// Alg. 1: z = 1/2 sum psi^2 + 1/2 sum delta h^2 and the stop test of a sweep
+// of a solve, on the solver state `st` (in memory, or a thread's own copy).
+// True if the solve stops at this sweep; otherwise t and z_prev advance.
+__device__ __forceinline__ bool apply_stop_rules(DevState& st, int mode, double* trace, double z, double cons, double cap)
 {
-    DevState* st = a.st;
-    const double z = 0.5 * zsum;
-    st->z = z;
-    st->cap_rel = cap;
-    st->cons_rel = cons;
-    if (a.mode == MODE_EVAL) return;
-    const double dz = z - st->z_prev;
-    st->dz = dz;
-    if (a.trace && st->evals < st->trace_len) a.trace[st->evals] = z;
-    st->evals += 1;
+    st.z = z;
+    st.cap_rel = cap;
+    st.cons_rel = cons;
+    const double dz = z - st.z_prev;
+    st.dz = dz;
+    if (trace && st.evals < st.trace_len) trace[st.evals] = z;
+    st.evals += 1;
     int stop = 0, reason = STOP_MAX_SWEEPS;
-    if (a.mode == MODE_SOLVE) {
+    if (mode == MODE_SOLVE) {
         if (!isfinite(z)) {
             stop = 1;
             reason = STOP_NUMERIC;
-        } else if (st->t >= st->max_sweeps) {
+        } else if (st.t >= st.max_sweeps) {
             stop = 1;
             reason = STOP_MAX_SWEEPS;
-        } else if (st->eps_obj > 0.0 && fabs(dz) < st->eps_obj) {
+        } else if (st.eps_obj > 0.0 && fabs(dz) < st.eps_obj) {
             stop = 1;
             reason = STOP_OBJECTIVE;
-        } else if (st->resid_tol > 0.0 && cap <= st->resid_tol && cons <= st->resid_tol) {
+        } else if (st.resid_tol > 0.0 && cap <= st.resid_tol && cons <= st.resid_tol) {
             stop = 1;
             reason = STOP_RESIDUAL;
-        } else if (st->eps_rel > 0.0 && fabs(dz) <= st->eps_rel * z) {
+        } else if (st.eps_rel > 0.0 && fabs(dz) <= st.eps_rel * z) {
             stop = 1;
             reason = STOP_RELATIVE;
-        } else if (st->stop_on_rise && dz >= 0.0) {
+        } else if (st.stop_on_rise && dz >= 0.0) {
             // the Section 4 theorem makes z non-increasing in exact arithmetic,
             // so a rise means rounding now dominates the progress
             stop = 1;
             reason = STOP_STALL;
-        } else if (st->plat_window > 0) {
+        } else if (st.plat_window > 0) {
             // residual plateau: the best r = max(cap_rel, cons_rel) of a window of
             // sweeps improves on the previous window's best by less than
             // kPlateauGain -- the FP32 rounding floor, not a slow descent (which
             // still improves every window)
             const double r = fmax(cap, cons);
-            if (r < st->plat_cur) st->plat_cur = r;
-            if (st->t - st->plat_t0 + 1 >= st->plat_window) {
+            if (r < st.plat_cur) st.plat_cur = r;
+            if (st.t - st.plat_t0 + 1 >= st.plat_window) {
                 // only near the target, where FP32 rounding can be the limit: a
                 // stall far above it is the method's own slow phase
-                const double ceiling = kPlateauCeiling * (st->resid_tol > 0.0 ? st->resid_tol : 1e-6);
-                if (st->plat_cur <= ceiling && st->plat_cur > (1.0 - kPlateauGain) * st->plat_prev) {
+                const double ceiling = kPlateauCeiling * (st.resid_tol > 0.0 ? st.resid_tol : 1e-6);
+                if (st.plat_cur <= ceiling && st.plat_cur > (1.0 - kPlateauGain) * st.plat_prev) {
                     stop = 1;
                     reason = STOP_PLATEAU;
                 }
-                st->plat_prev = st->plat_cur;
-                st->plat_cur = INFINITY;
-                st->plat_t0 = st->t + 1;
+                st.plat_prev = st.plat_cur;
+                st.plat_cur = INFINITY;
+                st.plat_t0 = st.t + 1;
             }
         }
     }
     if (stop) {
-        st->stop = 1;
-        st->reason = reason;
+        st.stop = 1;
+        st.reason = reason;
+    } else {
+        st.z_prev = z;
+        st.t += 1;
+    }
+    return stop != 0;
+}
+
+// The decision of one sweep, run by one thread after every partial of the
+// sweep is final.
+template <typename T>
+__device__ void finalize(const SweepArgs<T>& a, double zsum, double cons, double cap)
+{
+    DevState* st = a.st;
+    const double z = 0.5 * zsum;
+    if (a.mode == MODE_EVAL) {
+        st->z = z;
+        st->cap_rel = cap;
+        st->cons_rel = cons;
+        return;
+    }
+    if (apply_stop_rules(*st, a.mode, a.trace, z, cons, cap)) {
         // one instance: its stop ends the loop; a batch ends with its last instance
         const bool last = a.active ? atomicSub(a.active, 1u) == 1u : true;
         if (a.use_cond && last) cudaGraphSetConditional(a.cond, 0);
-    } else {
-        st->z_prev = z;
-        st->t += 1;
     }
-}
-
-// Load of an objective partial that another block of the same launch may
-// have written: at L2 (coherent) from global memory; SH = true when the
-// partials live in the block's shared memory (the one-block engine), where
-// a plain load is the coherent one.
-template <bool SH, typename X>
-__device__ __forceinline__ X ld_part(const X* p)
-{
-    if constexpr (SH) return *p;
-    else return __ldcg(p);
 }
 
 // FP64 reduction of the excess blocks' partials in a fixed order, then the
 // objective and the stop test.  Run by one whole block.
-template <typename T, bool SH = false>
+template <typename T>
 __device__ void reduce_and_finalize(const SweepArgs<T>& a)
 {
-    if (SH && a.grid_v == 1) {
-        // one partial of each kind: the block reduction below would add and
-        // compare only zeros to thread 0's values, so thread 0 forms the
-        // same result directly
-        if (threadIdx.x == 0) {
-            const double zs = 0.0 + ld_part<SH>(a.part_h);
-            const T c1 = ld_part<SH>(a.part_cons), c2 = ld_part<SH>(a.part_capb);
-            finalize(a, zs, (double)(c1 > T(0) ? c1 : T(0)), (double)(c2 > T(0) ? c2 : T(0)));
-        }
-        return;
-    }
     __shared__ double sz[32];
     __shared__ T sm1[32], sm2[32];
     double zs = 0.0;
     T cm = T(0), cp = T(0);
     for (int b = threadIdx.x; b < a.grid_v; b += blockDim.x) {
-        zs += ld_part<SH>(a.part_h + b);
-        const T c1 = ld_part<SH>(a.part_cons + b);
-        const T c2 = ld_part<SH>(a.part_capb + b);
+        zs += __ldcg(a.part_h + b);
+        const T c1 = __ldcg(a.part_cons + b);
+        const T c2 = __ldcg(a.part_capb + b);
         cm = c1 > cm ? c1 : cm;
         cp = c2 > cp ? c2 : cp;
     }
