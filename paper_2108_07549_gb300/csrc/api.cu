@@ -157,6 +157,8 @@ struct pdr_ctx {
     GridBarrier* bar = nullptr;    // its grid barrier
     DevState* st = nullptr;
     DevState* hst = nullptr;  // pinned mirror
+    bool owns_state = true;   // false: st, hst, r_out and hr_out are slices of a batch's arrays
+    bool psi_stale = false;   // the congestion partials are not those of the current flows (cluster engine)
     double* trace = nullptr;
     int64_t trace_cap = 0;
     // residuals
@@ -427,7 +429,7 @@ pdr_status ensure_velocity(pdr_ctx* ctx)
 template <typename T>
 pdr_status init_gd_state(pdr_ctx* ctx)
 {
-    if (ctx->m == 0) return PDR_OK;
+    if (ctx->m == 0 || !is_gd(ctx->opt)) return PDR_OK;
     std::vector<T> b(ctx->m, (T)ctx->g_beta_init);
     CK(cudaMemcpyAsync(ctx->beta_buf[0], b.data(), sizeof(T) * ctx->m, cudaMemcpyHostToDevice, ctx->stream));
     if (ctx->opt.algo == PDR_ALGO_GDM) {
@@ -451,7 +453,7 @@ pdr_status flows_to_buffer0(pdr_ctx* ctx)
     if (ctx->cur == 0) return PDR_OK;
     const size_t bytes = sizeof(T) * (size_t)ctx->m * ctx->Kp;
     if (bytes) CK(cudaMemcpyAsync(Prec<T>::f(ctx, 0), Prec<T>::f(ctx, 1), bytes, cudaMemcpyDeviceToDevice, ctx->stream));
-    if (ctx->m > 0)
+    if (ctx->m > 0 && is_gd(ctx->opt))
         CK(cudaMemcpyAsync(ctx->beta_buf[0], ctx->beta_buf[1], sizeof(T) * ctx->m, cudaMemcpyDeviceToDevice,
                            ctx->stream));
     if (ctx->opt.algo == PDR_ALGO_GDM && bytes && Prec<T>::v(ctx, 1))
@@ -481,6 +483,7 @@ pdr_status refresh_psi(pdr_ctx* ctx, T* psi_out = nullptr, bool keep_theta = fal
     }
     SweepArgs<T> a = make_args<T>(ctx, MODE_PSI);
     a.psi_out = psi_out;
+    ctx->psi_stale = false;
     if (ctx->m > 0) {
         CK(launch_edge<T>(a, ctx->cfg[Prec<T>::id], ctx->stream));
     } else {
@@ -493,6 +496,14 @@ pdr_status refresh_psi(pdr_ctx* ctx, T* psi_out = nullptr, bool keep_theta = fal
 pdr_status refresh_psi_current(pdr_ctx* ctx)
 {
     return ctx->cur_prec ? refresh_psi<double>(ctx) : refresh_psi<float>(ctx);
+}
+
+// Before a kernel that reads the congestion partials: the cluster engine, which
+// keeps its own, leaves them behind.
+pdr_status ensure_psi(pdr_ctx* ctx)
+{
+    if (!ctx->psi_stale) return PDR_OK;
+    return ctx->cur_prec ? refresh_psi<double>(ctx, nullptr, true) : refresh_psi<float>(ctx, nullptr, true);
 }
 
 template <typename T>
@@ -652,7 +663,7 @@ cudaError_t launch_set_data(int64_t m, int K, int Kp, const double* u, const dou
     return cudaGetLastError();
 }
 
-pdr_status init_state(pdr_ctx* ctx, bool fresh, int stop_on_rise, bool keep_zprev = false)
+DevState make_state(pdr_ctx* ctx, bool fresh, int stop_on_rise, bool keep_zprev = false)
 {
     if (fresh) ctx->resume_pending = false;
     DevState v{};
@@ -675,8 +686,59 @@ pdr_status init_state(pdr_ctx* ctx, bool fresh, int stop_on_rise, bool keep_zpre
     v.plat_t0 = keep_zprev ? ctx->hst->plat_t0 : v.t;  // a resumed solve keeps its windows
     v.plat_cur = keep_zprev ? ctx->hst->plat_cur : INFINITY;
     v.plat_prev = keep_zprev ? ctx->hst->plat_prev : INFINITY;
-    set_state_kernel<<<1, 1, 0, ctx->stream>>>(ctx->st, v);
+    return v;
+}
+
+pdr_status init_state(pdr_ctx* ctx, bool fresh, int stop_on_rise, bool keep_zprev = false)
+{
+    set_state_kernel<<<1, 1, 0, ctx->stream>>>(ctx->st, make_state(ctx, fresh, stop_on_rise, keep_zprev));
     CK(cudaGetLastError());
+    return PDR_OK;
+}
+
+// f = 0: flows, roots, warm starts, congestion partials (those of f = 0 are
+// 0), Alg. 3/4 rates and velocities, and the solver state, in one launch.
+// Everything but the rates is zeroed in 16-byte words.
+struct ResetSpans {
+    uint4* at[6];
+    int64_t words[6];
+};
+template <typename T>
+__global__ void __launch_bounds__(256) reset_kernel(ResetSpans z, T* beta, int64_t m, T beta_init, DevState* st, DevState v)
+{
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        for (int64_t q = first; q < z.words[k]; q += step) z.at[k][q] = make_uint4(0u, 0u, 0u, 0u);
+    if (beta)
+        for (int64_t e = first; e < m; e += step) beta[e] = beta_init;
+    if (first == 0) *st = v;
+}
+template <typename T>
+pdr_status zero_flows(pdr_ctx* ctx)
+{
+    const int64_t m = ctx->m > 0 ? ctx->m : 1, rows = (int64_t)ctx->m * ctx->Kp * (int64_t)sizeof(T) / 16;
+    const int64_t parts = (ctx->n_psi[Prec<T>::id] + 1) / 2;  // 8 bytes each; the arrays hold an even count
+    const bool gd = is_gd(ctx->opt) && ctx->m > 0;
+    ResetSpans z{};
+    auto span = [&](int k, void* p, int64_t words) { z.at[k] = static_cast<uint4*>(p), z.words[k] = words; };
+    span(0, Prec<T>::f(ctx, 0), rows);
+    span(1, ctx->theta[0], m);  // [2 m] doubles
+    span(2, ctx->theta[1], m);
+    span(3, ctx->part_psi, parts);
+    span(4, ctx->part_cap, parts);
+    if (gd && ctx->opt.algo == PDR_ALGO_GDM) {
+        const pdr_status s = ensure_velocity<T>(ctx);
+        if (s != PDR_OK) return s;
+        span(5, Prec<T>::v(ctx, 0), rows);
+    }
+    const DevState v = make_state(ctx, true, 0);
+    const int64_t want = ((rows > m ? rows : m) + 1023) / 1024, cap = (int64_t)ctx->num_sms * 8;
+    reset_kernel<T><<<(int)(want < 1 ? 1 : want < cap ? want : cap), 256, 0, ctx->stream>>>(
+        z, gd ? reinterpret_cast<T*>(ctx->beta_buf[0]) : nullptr, ctx->m, (T)ctx->g_beta_init, ctx->st, v);
+    CK(cudaGetLastError());
+    *ctx->hst = v;
+    ctx->psi_stale = false;
     return PDR_OK;
 }
 
@@ -907,8 +969,8 @@ pdr_status run_cluster(pdr_ctx* ctx, int64_t t_start)
         if (ctx->hst->stop) break;
     }
     ctx->cur = (int)((ctx->hst->t - t_start) & 1);
-    // the current flows' congestion partials in the standalone kernels' layout
-    return refresh_psi<float>(ctx, nullptr, true);
+    ctx->psi_stale = true;
+    return PDR_OK;
 }
 
 // The persistent engine applies to Alg. 1 with a lane-group variant.
@@ -986,6 +1048,8 @@ pdr_status run_phase(pdr_ctx* ctx, int64_t t_start)
     // rate, a small fraction of its FP32 rate on this GPU, and loses to the
     // kernels that spread a sweep over every SM
     if (p == Prec<float>::id && cluster_eligible(ctx)) return run_cluster(ctx, t_start);
+    s = ensure_psi(ctx);
+    if (s != PDR_OK) return s;
     if (persistent_ok(ctx, p)) {
         bool ran = false;
         s = run_persistent<T>(ctx, &ran);
@@ -1027,20 +1091,32 @@ pdr_status run_phase(pdr_ctx* ctx, int64_t t_start)
 }
 
 template <typename T>
+ResidTask<T> resid_task(pdr_ctx* ctx)
+{
+    ResidTask<T> k{};
+    k.a = make_args<T>(ctx, MODE_EVAL);
+    k.r = ResidIn{ctx->u_d, ctx->dem_d, ctx->inv_deg_d, ctx->inv_dem_f};
+    k.h64 = ctx->r_h64;
+    k.part = ctx->r_part;
+    k.out = ctx->r_out;
+    k.grid_v = ctx->r_grid_v;
+    k.grid_e = ctx->r_grid_e;
+    return k;
+}
+
+template <typename T>
 pdr_status residuals_T(pdr_ctx* ctx)
 {
-    SweepArgs<T> a = make_args<T>(ctx, MODE_EVAL);
-    const ResidIn r{ctx->u_d, ctx->dem_d, ctx->inv_deg_d, ctx->inv_dem_f};
-    CK(launch_residuals<T>(a, r, ctx->r_h64, ctx->r_part, ctx->r_grid_v, ctx->r_grid_e, ctx->r_out, ctx->stream));
+    const ResidTask<T> k = resid_task<T>(ctx);
+    CK(launch_residuals<T>(nullptr, &k, 1, ctx->stream));
     CK(cudaMemcpyAsync(ctx->hr_out, ctx->r_out, sizeof(ResidOut), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     return PDR_OK;
 }
 
-pdr_status residuals_into(pdr_ctx* ctx, pdr_result* r)
+// The result of a residual pass (in hr_out) and the verdict.
+void residuals_out(pdr_ctx* ctx, pdr_result* r)
 {
-    pdr_status s = ctx->cur_prec ? residuals_T<double>(ctx) : residuals_T<float>(ctx);
-    if (s != PDR_OK) return s;
     const ResidOut& o = *ctx->hr_out;
     r->z = o.z;
     r->cap_abs = o.cap_abs;
@@ -1054,6 +1130,13 @@ pdr_status residuals_into(pdr_ctx* ctx, pdr_result* r)
     if (ctx->isolated || o.margin > 1e-9 * o.margin_scale) r->verdict = PDR_VERDICT_INFEASIBLE;
     else if (o.cap_rel <= tol && o.cons_rel <= tol) r->verdict = PDR_VERDICT_FEASIBLE;
     else r->verdict = PDR_VERDICT_UNKNOWN;
+}
+
+pdr_status residuals_into(pdr_ctx* ctx, pdr_result* r)
+{
+    const pdr_status s = ctx->cur_prec ? residuals_T<double>(ctx) : residuals_T<float>(ctx);
+    if (s != PDR_OK) return s;
+    residuals_out(ctx, r);
     return PDR_OK;
 }
 
@@ -1337,17 +1420,18 @@ void pdr_destroy(pdr_ctx* ctx)
     void* dev[] = {ctx->row_ptr, ctx->in_ptr, ctx->inc_ptr, ctx->inc, ctx->work, ctx->col, ctx->src, ctx->in_eid,
                    ctx->deg, ctx->s, ctx->t,
                    ctx->u_d, ctx->dem_d, ctx->inv_scale, ctx->u_f, ctx->dem_f, ctx->inv_dem_f, ctx->inv_dem_d,
-                   ctx->f32[0], ctx->f32[1], ctx->h32, ctx->f64[0], ctx->f64[1], ctx->h64, ctx->part_h, ctx->part_cons, ctx->part_capb, ctx->part_psi, ctx->part_cap, ctx->st,
+                   ctx->f32[0], ctx->f32[1], ctx->h32, ctx->f64[0], ctx->f64[1], ctx->h64, ctx->part_h, ctx->part_cons, ctx->part_capb, ctx->part_psi, ctx->part_cap,
+                   ctx->owns_state ? ctx->st : nullptr,
                    ctx->trace, ctx->inv_scale_f, ctx->inv_deg_f, ctx->inv_deg_d, ctx->theta[0], ctx->theta[1],
                    ctx->beta_buf[0], ctx->beta_buf[1], ctx->v32[0], ctx->v32[1], ctx->v64[0], ctx->v64[1],
-                   ctx->r_h64, ctx->r_part, ctx->r_out, ctx->psi_tmp, ctx->bar, ctx->xv_start[1], ctx->xv_start[2], ctx->xv_start[3],
+                   ctx->r_h64, ctx->r_part, ctx->owns_state ? ctx->r_out : nullptr, ctx->psi_tmp, ctx->bar, ctx->xv_start[1], ctx->xv_start[2], ctx->xv_start[3],
                    ctx->xv_start[4], ctx->xv_start[5],
                    ctx->data_err, ctx->cl_split};
     for (void* p : dev)
         if (p) cudaFree(p);
     release_adjoint_workspace(ctx);
-    if (ctx->hst) cudaFreeHost(ctx->hst);
-    if (ctx->hr_out) cudaFreeHost(ctx->hr_out);
+    if (ctx->hst && ctx->owns_state) cudaFreeHost(ctx->hst);
+    if (ctx->hr_out && ctx->owns_state) cudaFreeHost(ctx->hr_out);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     cudaGetLastError();
     delete ctx;
@@ -1462,6 +1546,7 @@ pdr_status pdr_create(int32_t n, int64_t m, const int64_t* row_ptr, const int32_
     // partial per block and per warp
     if (gv < 8 * ctx->num_sms) gv = 8 * ctx->num_sms;
     if (np < 64 * (int64_t)ctx->num_sms) np = 64 * (int64_t)ctx->num_sms;
+    np += np & 1;  // zeroed in 16-byte words
     ALLOC(ctx->part_h, double, gv);
     ALLOC(ctx->part_cons, double, gv);
     ALLOC(ctx->part_capb, double, gv);
@@ -1623,17 +1708,8 @@ pdr_status pdr_reset(pdr_ctx* ctx)
     ctx->cur_prec = start_prec(ctx->opt);
     pdr_status s = ctx->cur_prec ? ensure_fp64(ctx) : ensure_fp32(ctx);
     if (s != PDR_OK) return s;
-    const size_t fm = (size_t)ctx->m * ctx->Kp;
     ctx->cur = 0;
-    if (ctx->cur_prec) CK(cudaMemsetAsync(ctx->f64[0], 0, sizeof(double) * (fm ? fm : 1), ctx->stream));
-    else CK(cudaMemsetAsync(ctx->f32[0], 0, sizeof(float) * (fm ? fm : 1), ctx->stream));
-    s = init_gd_state_current(ctx);
-    if (s != PDR_OK) return s;
-    s = refresh_psi_current(ctx);
-    if (s != PDR_OK) return s;
-    s = init_state(ctx, true, 0);
-    if (s != PDR_OK) return s;
-    return read_state(ctx);
+    return ctx->cur_prec ? zero_flows<double>(ctx) : zero_flows<float>(ctx);
 }
 
 pdr_status pdr_set_flows(pdr_ctx* ctx, const double* f)
@@ -2088,6 +2164,8 @@ pdr_status pdr_congestion(pdr_ctx* ctx, double* psi)
 pdr_status pdr_objective(pdr_ctx* ctx, double* z)
 {
     if (!ctx || !z) return ctx ? ctx->fail(PDR_ERR_INVALID_ARG, "z is NULL") : PDR_ERR_INVALID_ARG;
+    pdr_status s = ensure_psi(ctx);
+    if (s != PDR_OK) return s;
     if (ctx->cur_prec) {
         CK(launch_excess<double>(make_args<double>(ctx, MODE_EVAL), ctx->stream));
         CK(launch_finalize<double>(make_args<double>(ctx, MODE_EVAL), ctx->stream));
@@ -2095,7 +2173,7 @@ pdr_status pdr_objective(pdr_ctx* ctx, double* z)
         CK(launch_excess<float>(make_args<float>(ctx, MODE_EVAL), ctx->stream));
         CK(launch_finalize<float>(make_args<float>(ctx, MODE_EVAL), ctx->stream));
     }
-    pdr_status s = read_state(ctx);
+    s = read_state(ctx);
     if (s != PDR_OK) return s;
     *z = ctx->hst->z;
     return PDR_OK;
@@ -2119,6 +2197,8 @@ pdr_status pdr_sweeps(pdr_ctx* ctx, int64_t count)
     pdr_status s = read_state(ctx);
     if (s != PDR_OK) return s;
     s = init_state(ctx, false, 0);  // t continues (it drives the Alg. 3 / Alg. 4 schedule)
+    if (s != PDR_OK) return s;
+    s = ensure_psi(ctx);
     if (s != PDR_OK) return s;
     s = ctx->cur_prec ? ensure_velocity<double>(ctx) : ensure_velocity<float>(ctx);
     if (s != PDR_OK) return s;
@@ -2148,6 +2228,8 @@ pdr_status pdr_time_sweeps(pdr_ctx* ctx, int64_t count, double* ms_excess, doubl
     pdr_status s = read_state(ctx);
     if (s != PDR_OK) return s;
     s = init_state(ctx, false, 0);
+    if (s != PDR_OK) return s;
+    s = ensure_psi(ctx);
     if (s != PDR_OK) return s;
     s = ctx->cur_prec ? ensure_velocity<double>(ctx) : ensure_velocity<float>(ctx);
     if (s != PDR_OK) return s;
@@ -2377,6 +2459,11 @@ struct pdr_batch {
     void* bargs = nullptr;   // device ClusterArgs [count]
     int* bids = nullptr;     // device instance ids [count], grouped by launch
     void* hstage = nullptr;  // pinned staging of the arguments and ids
+    // the contexts' solver states and residual results, side by side, so that
+    // one copy moves them all, and the residual pass's table
+    DevState *st = nullptr, *hst = nullptr;
+    ResidOut *r_out = nullptr, *hr_out = nullptr;
+    void *tasks = nullptr, *htasks = nullptr;  // ResidTask<double> [count], room for either precision
 };
 
 namespace {
@@ -2637,10 +2724,8 @@ pdr_status batch_cluster_run(pdr_batch* b, const std::vector<char>& blk, const s
             if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, ev[1 + group], 0);
             at = end;
         }
-        for (size_t q = 0; q < live.size() && e == cudaSuccess; ++q) {
-            pdr_ctx* c = b->ctx[live[q]];
-            e = cudaMemcpyAsync(c->hst, c->st, sizeof(DevState), cudaMemcpyDeviceToHost, b->stream);
-        }
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(b->hst, b->st, sizeof(DevState) * b->count, cudaMemcpyDeviceToHost, b->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
         if (e != cudaSuccess) return cuda_err("cluster engine", e);
         std::vector<int32_t> next;
@@ -2649,13 +2734,11 @@ pdr_status batch_cluster_run(pdr_batch* b, const std::vector<char>& blk, const s
         live.swap(next);
         first = false;
     }
-    // current flows, and the congestion partials in the standalone kernels' layout
     for (int32_t i = 0; i < b->count; ++i) {
         if (!blk[i]) continue;
         pdr_ctx* c = b->ctx[i];
         c->cur = (int)((c->hst->t - t_start[i]) & 1);
-        const pdr_status st = refresh_psi<float>(c, nullptr, true);
-        if (st != PDR_OK) return done(st);
+        c->psi_stale = true;
     }
     return done(PDR_OK);
 }
@@ -2663,6 +2746,35 @@ pdr_status batch_cluster_run(pdr_batch* b, const std::vector<char>& blk, const s
 // Alg. 1 in precision T for the instances with run_all[i] set, from the states
 // their callers initialised (instance i's sweep counter starting at
 // t_start[i]); the others keep their stopped state.
+// Every instance's solver state, in one copy.
+pdr_status batch_read_states(pdr_batch* b)
+{
+    cudaError_t e = cudaMemcpyAsync(b->hst, b->st, sizeof(DevState) * b->count, cudaMemcpyDeviceToHost, b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    if (e != cudaSuccess) return batch_fail(PDR_ERR_CUDA, std::string("batch: ") + cudaGetErrorString(e));
+    for (int32_t i = 0; i < b->count; ++i)
+        if (b->hst[i].fault) return batch_fail(PDR_ERR_TIMEOUT, "instance " + std::to_string(i) + ": a device wait timed out");
+    return PDR_OK;
+}
+
+// The residual pass of the instances whose flows are of type T, in three launches.
+template <typename T>
+pdr_status batch_residuals(pdr_batch* b)
+{
+    ResidTask<T>* host = static_cast<ResidTask<T>*>(b->htasks);
+    int count = 0;
+    for (pdr_ctx* c : b->ctx)
+        if (c->cur_prec == Prec<T>::id) host[count++] = resid_task<T>(c);
+    if (count == 0) return PDR_OK;
+    cudaError_t e = cudaMemcpyAsync(b->tasks, host, sizeof(ResidTask<T>) * count, cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) e = launch_residuals<T>(static_cast<const ResidTask<T>*>(b->tasks), host, count, b->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->hr_out, b->r_out, sizeof(ResidOut) * b->count, cudaMemcpyDeviceToHost, b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    if (e != cudaSuccess) return batch_fail(PDR_ERR_CUDA, std::string("batch residuals: ") + cudaGetErrorString(e));
+    return PDR_OK;
+}
+
 template <typename T>
 pdr_status batch_run(pdr_batch* b, const std::vector<char>& run_all, const std::vector<int64_t>& t_start)
 {
@@ -2685,7 +2797,11 @@ pdr_status batch_run(pdr_batch* b, const std::vector<char>& run_all, const std::
         if (s != PDR_OK) return s;
         s = flows_to_buffer0<T>(c);
         if (s != PDR_OK) return s;
-        if (run[i]) ++running;
+        if (run[i]) {
+            s = ensure_psi(c);
+            if (s != PDR_OK) return s;
+            ++running;
+        }
     }
     if (any_blk) {
         const pdr_status s = batch_cluster_run(b, blk, t_start);
@@ -2720,13 +2836,10 @@ pdr_status batch_run(pdr_batch* b, const std::vector<char>& run_all, const std::
             if (left == 0) break;
         }
     }
-    for (int32_t i = 0; i < b->count; ++i) {
-        if (!run[i]) continue;
-        pdr_ctx* c = b->ctx[i];
-        pdr_status s = read_state(c);
-        if (s != PDR_OK) return s;
-        c->cur = (int)((c->hst->t - t_start[i]) & 1);
-    }
+    const pdr_status s = batch_read_states(b);
+    if (s != PDR_OK) return s;
+    for (int32_t i = 0; i < b->count; ++i)
+        if (run[i]) b->ctx[i]->cur = (int)((b->ctx[i]->hst->t - t_start[i]) & 1);
     return PDR_OK;
 }
 
@@ -2783,6 +2896,31 @@ pdr_status pdr_batch_create(int32_t count, const pdr_instance* inst, const pdr_o
         }
         b->ctx.push_back(c);
     }
+    // the contexts' states and results move into shared arrays
+    if (cudaMalloc(&b->st, sizeof(DevState) * count) != cudaSuccess ||
+        cudaMalloc(&b->r_out, sizeof(ResidOut) * count) != cudaSuccess ||
+        cudaMalloc(&b->tasks, sizeof(ResidTask<double>) * count) != cudaSuccess ||
+        cudaMallocHost(&b->hst, sizeof(DevState) * count) != cudaSuccess ||
+        cudaMallocHost(&b->hr_out, sizeof(ResidOut) * count) != cudaSuccess ||
+        cudaMallocHost(&b->htasks, sizeof(ResidTask<double>) * count) != cudaSuccess) {
+        cudaGetLastError();
+        return give_up(PDR_ERR_OOM, "batch: state table allocation failed");
+    }
+    for (int32_t i = 0; i < count; ++i) {
+        pdr_ctx* c = b->ctx[i];
+        b->hst[i] = *c->hst;
+        cudaFree(c->st);
+        cudaFree(c->r_out);
+        cudaFreeHost(c->hst);
+        cudaFreeHost(c->hr_out);
+        c->st = b->st + i;
+        c->hst = b->hst + i;
+        c->r_out = b->r_out + i;
+        c->hr_out = b->hr_out + i;
+        c->owns_state = false;
+        const pdr_status s = init_state(c, true, 0);
+        if (s != PDR_OK) return give_up(s, "instance " + std::to_string(i) + ": " + c->err);
+    }
     b->tuned_cfg.assign(count, -1);
     b->tuned_us.assign(count, -1.0);
     if (cudaMalloc(&b->bargs, sizeof(ClusterArgs) * count) != cudaSuccess ||
@@ -2820,10 +2958,12 @@ pdr_status pdr_batch_solve(pdr_batch* b, pdr_result* results)
     // every instance starts a fresh solve from its current flows, as pdr_solve
     for (int32_t i = 0; i < B; ++i) {
         pdr_ctx* c = b->ctx[i];
-        s = init_state(c, true, (tail && c->cur_prec == 0) ? 1 : 0);
-        if (s != PDR_OK) return s;
+        *c->hst = make_state(c, true, (tail && c->cur_prec == 0) ? 1 : 0);
         (c->cur_prec ? run64 : run32)[i] = 1;
     }
+    cudaError_t e = cudaMemcpyAsync(b->st, b->hst, sizeof(DevState) * B, cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // the mirror is a copy's target below
+    if (e != cudaSuccess) return batch_fail(PDR_ERR_CUDA, std::string("batch: ") + cudaGetErrorString(e));
     s = batch_run<float>(b, run32, t_start);
     if (s != PDR_OK) return s;
     if (tail) {
@@ -2832,8 +2972,6 @@ pdr_status pdr_batch_solve(pdr_batch* b, pdr_result* results)
         for (int32_t i = 0; i < B; ++i) {
             pdr_ctx* c = b->ctx[i];
             if (!run32[i]) continue;
-            s = read_state(c);
-            if (s != PDR_OK) return s;
             sweeps32[i] = c->hst->t;
             reason32[i] = c->hst->reason;
             if (needs_fp64_tail(c->hst->reason)) {
@@ -2857,18 +2995,18 @@ pdr_status pdr_batch_solve(pdr_batch* b, pdr_result* results)
     if (s != PDR_OK) return s;
     const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     bool numeric = false;
+    s = batch_residuals<float>(b);
+    if (s == PDR_OK) s = batch_residuals<double>(b);
+    if (s != PDR_OK) return s;
     for (int32_t i = 0; i < b->count; ++i) {
         pdr_ctx* c = b->ctx[i];
-        s = read_state(c);
-        if (s != PDR_OK) return s;
         pdr_result r{};
         r.sweeps = c->hst->t;
         r.sweeps_fp64 = c->cur_prec ? c->hst->t - sweeps32[i] : 0;
         r.dz = c->hst->dz;
         r.stop_reason = c->hst->reason;
         r.stop_reason_fp32 = tail ? reason32[i] : -1;
-        s = residuals_into(c, &r);
-        if (s != PDR_OK) return batch_fail(s, "instance " + std::to_string(i) + ": " + c->err);
+        residuals_out(c, &r);
         r.ms_total = ms;
         c->last = r;
         if (results) results[i] = r;
@@ -2915,7 +3053,10 @@ void pdr_batch_destroy(pdr_batch* b)
     for (cudaStream_t s : b->pool) cudaStreamDestroy(s);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
     if (b->active) cudaFree(b->active);
-    if (b->bargs) cudaFree(b->bargs);
+    for (void* q : {b->bargs, static_cast<void*>(b->st), static_cast<void*>(b->r_out), b->tasks})
+        if (q) cudaFree(q);
+    for (void* q : {static_cast<void*>(b->hst), static_cast<void*>(b->hr_out), b->htasks})
+        if (q) cudaFreeHost(q);
     if (b->bids) cudaFree(b->bids);
     if (b->hstage) cudaFreeHost(b->hstage);
     cudaGetLastError();

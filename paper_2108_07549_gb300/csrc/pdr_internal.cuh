@@ -277,8 +277,17 @@ struct ResidIn {
 };
 
 template <typename T>
-cudaError_t launch_residuals(const SweepArgs<T>& a, const ResidIn& r, double* h64, double* part, int32_t grid_v,
-                             int32_t grid_e, ResidOut* out, cudaStream_t stream);
+struct ResidTask {
+    SweepArgs<T> a;  // f: the flows; h: FP32 heights (overwritten, FP32 flows only)
+    ResidIn r;
+    double *h64, *part;  // scratch: [n][Kp], [resid_part_count]
+    ResidOut* out;
+    int32_t grid_v, grid_e;
+};
+// `count` instances: tasks on the device and the same on the host, or tasks
+// NULL and one on the host.
+template <typename T>
+cudaError_t launch_residuals(const ResidTask<T>* tasks, const ResidTask<T>* host, int count, cudaStream_t stream);
 int resid_part_count(int32_t grid_v, int32_t grid_e);
 
 // Message returned by pdr_last_error(NULL) on the calling thread (api.cu).

@@ -20,6 +20,12 @@
 //   sum_k d_k (pi_{s_k,k} - pi_{t_k,k}) = sum_{e,k} f_e,k (pi_ik - pi_jk)
 //                                      <= sum_e l_e sum_k f_e,k <= sum_e u_e l_e,
 // so margin > 0 proves that eq. (1) has no solution.
+//
+// The kernels take one instance, or a table of them (a batch: blockIdx.y, in
+// the final pass blockIdx.x, is the instance), so that a batch's pass is three
+// launches and not three per instance.  One instance's arguments come from
+// the constant bank: through the table's pointer the edge pass took 931 us
+// against 681 us at m = 39,600, K = 10,000.
 #include "widen.cuh"
 
 #include <math.h>
@@ -130,42 +136,56 @@ constexpr float kHeightSlack = 4.76837158e-7f;  // 2^-21
 // and 1/delta_i is applied once per four squares.  The three kernels of a
 // residual pass at n = 10,000, m = 39,600, K = 10,000: 5.0 ms before, 2.04 ms
 // now (vertex 1.31 ms, edge 0.68 ms).
-__global__ void __launch_bounds__(256) resid_vertex_pair_kernel(SweepArgs<float> a, ResidIn r, float* __restrict__ h32,
-                                                                double* __restrict__ delta, double* __restrict__ part)
+template <bool TABLE>
+__global__ void __launch_bounds__(256)
+    resid_vertex_pair_kernel(const ResidTask<float>* __restrict__ tasks, const __grid_constant__ ResidTask<float> one)
 {
+    const ResidTask<float>& task = TABLE ? tasks[blockIdx.y] : one;
+    const int nblocks = task.grid_v;
+    if ((int)blockIdx.x >= nblocks) return;
+    const SweepArgs<float>& a = task.a;
+    const ResidIn r = task.r;
+    float* const h32 = a.h;
+    double* const delta = task.h64;
+    double* const part = task.part;
     __shared__ double smem[5][32];
-    const uint32_t nvec = (uint32_t)(a.Kp / 4);
+    const int K = a.K;
+    const int64_t Kp = a.Kp;
+    const float* const f = a.f;
+    const int64_t* const inc_ptr = a.inc_ptr;
+    const int32_t* const inc = a.inc;
+    const uint32_t nvec = (uint32_t)(Kp / 4);
     const uint64_t total = (uint64_t)a.n * nvec;
     double zsum = 0.0, cabs = 0.0, crel = 0.0;
     float cabs32 = 0.f, crel32 = 0.f;  // FP32 estimates of the elements behind cabs, crel
     for (uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (uint64_t)gridDim.x * blockDim.x) {
+         idx += (uint64_t)nblocks * blockDim.x) {
         const uint32_t i = total <= 0xffffffffull ? (uint32_t)idx / nvec : (uint32_t)(idx / nvec);
         const uint32_t v = (uint32_t)(idx - (uint64_t)i * nvec);
         const int k0 = 4 * (int)v;
         PairSum acc[4];
-        const int64_t q0 = a.inc_ptr[i], q1 = a.inc_ptr[i + 1];
+        const int64_t q0 = inc_ptr[i], q1 = inc_ptr[i + 1];
         auto add = [&](int32_t ev, const float4& x) {
             const float sg = ev >= 0 ? 1.f : -1.f;  // in-edges e, then out-edges ~e
             acc[0].add(sg * x.x), acc[1].add(sg * x.y), acc[2].add(sg * x.z), acc[3].add(sg * x.w);
         };
         auto row = [&](int32_t ev) {
             const int64_t e = ev >= 0 ? ev : ~ev;
-            return __ldg(reinterpret_cast<const float4*>(a.f + e * a.Kp) + v);
+            return __ldg(reinterpret_cast<const float4*>(f + e * Kp) + v);
         };
         int64_t q = q0;
         for (; q + 4 <= q1; q += 4) {  // four rows in flight
             int32_t ev[4];
             float4 x[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) ev[u] = a.inc[q + u];
+            for (int u = 0; u < 4; ++u) ev[u] = inc[q + u];
 #pragma unroll
             for (int u = 0; u < 4; ++u) x[u] = row(ev[u]);
 #pragma unroll
             for (int u = 0; u < 4; ++u) add(ev[u], x[u]);
         }
         for (; q < q1; ++q) {
-            const int32_t ev = a.inc[q];
+            const int32_t ev = inc[q];
             add(ev, row(ev));
         }
         const int4 sv = __ldg(reinterpret_cast<const int4*>(a.s + k0));
@@ -181,7 +201,7 @@ __global__ void __launch_bounds__(256) resid_vertex_pair_kernel(SweepArgs<float>
             const int k = k0 + j;
             D[j] = widen(acc[j].hi) + widen(acc[j].lo);
             float D32 = __fadd_rn(acc[j].hi, acc[j].lo);
-            if (k >= a.K) D[j] = 0.0, D32 = 0.f;  // the padding carries no commodity
+            if (k >= K) D[j] = 0.0, D32 = 0.f;  // the padding carries no commodity
             if (ss[j] == (int)i || tt[j] == (int)i) {  // padding has s = t = -1
                 D[j] += ss[j] == (int)i ? r.dem_d[k] : -r.dem_d[k];
                 D32 = (float)D[j];
@@ -202,10 +222,10 @@ __global__ void __launch_bounds__(256) resid_vertex_pair_kernel(SweepArgs<float>
             }
         }
         zsum = fma(sq, r.inv_deg_d[i], zsum);  // delta_i h^2 = Delta^2 / delta_i
-        double2* dp = reinterpret_cast<double2*>(delta + (int64_t)i * a.Kp + k0);
+        double2* dp = reinterpret_cast<double2*>(delta + (int64_t)i * Kp + k0);
         dp[0] = make_double2(D[0], D[1]);
         dp[1] = make_double2(D[2], D[3]);
-        *reinterpret_cast<float4*>(h32 + (int64_t)i * a.Kp + k0) = make_float4(hf[0], hf[1], hf[2], hf[3]);
+        *reinterpret_cast<float4*>(h32 + (int64_t)i * Kp + k0) = make_float4(hf[0], hf[1], hf[2], hf[3]);
     }
     double v[3] = {zsum, cabs, crel};
     const int op[3] = {0, 1, 1};
@@ -216,13 +236,21 @@ __global__ void __launch_bounds__(256) resid_vertex_pair_kernel(SweepArgs<float>
 
 // Vertex pass, FP64 flows: one warp per vertex, each lane four commodities at
 // a time; h = Delta / delta_i stored in FP64.
-__global__ void __launch_bounds__(256) resid_vertex_kernel(SweepArgs<double> a, ResidIn r, double* __restrict__ h64,
-                                                           double* __restrict__ part)
+template <bool TABLE>
+__global__ void __launch_bounds__(256)
+    resid_vertex_kernel(const ResidTask<double>* __restrict__ tasks, const __grid_constant__ ResidTask<double> one)
 {
+    const ResidTask<double>& task = TABLE ? tasks[blockIdx.y] : one;
+    const int nblocks = task.grid_v;
+    if ((int)blockIdx.x >= nblocks) return;
+    const SweepArgs<double>& a = task.a;
+    const ResidIn r = task.r;
+    double* const h64 = task.h64;
+    double* const part = task.part;
     __shared__ double smem[5][32];
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t nwarps = ((int64_t)nblocks * blockDim.x) >> 5;
     const int nvec = a.Kp / 4;
     double zsum = 0.0, cabs = 0.0, crel = 0.0;
     float cabs32 = 0.f, crel32 = 0.f;  // FP32 estimates of the elements behind cabs, crel
@@ -293,20 +321,33 @@ __global__ void __launch_bounds__(256) resid_vertex_kernel(SweepArgs<double> a, 
 // elements need their FP64 difference, so a row costs 12 bytes per element
 // and FP64 only at its few candidates (both height rows in FP64 made the
 // FP64 pipe the bound: 559 us at m = 39,600, K = 2,500).
-template <typename T>
-__global__ void __launch_bounds__(256) resid_edge_kernel(SweepArgs<T> a, ResidIn r, const float* __restrict__ h32,
-                                                         const double* __restrict__ h64, double* __restrict__ part)
+template <typename T, bool TABLE>
+__global__ void __launch_bounds__(256)
+    resid_edge_kernel(const ResidTask<T>* __restrict__ tasks, const __grid_constant__ ResidTask<T> one)
 {
+    const ResidTask<T>& task = TABLE ? tasks[blockIdx.y] : one;
+    const int nblocks = task.grid_e;
+    if ((int)blockIdx.x >= nblocks) return;
+    const SweepArgs<T>& a = task.a;
+    const ResidIn r = task.r;
+    const float* const h32 = sizeof(T) == 4 ? reinterpret_cast<const float*>(a.h) : nullptr;
+    const double* const h64 = task.h64;
+    double* const part = task.part + (int64_t)task.grid_v * kVParts;
     __shared__ double smem[5][32];
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t nwarps = ((int64_t)nblocks * blockDim.x) >> 5;
+    const int K = a.K;
+    const int64_t Kp = a.Kp, m = a.m;
+    const T* const f = a.f;
+    const int32_t* const src = a.src;
+    const int32_t* const col = a.col;
     const int nvec = a.Kp / 4;
     double psi2 = 0.0, capa = 0.0, capr = 0.0, cost = 0.0, fmn = INFINITY;
-    for (int64_t e = warp; e < a.m; e += nwarps) {
+    for (int64_t e = warp; e < m; e += nwarps) {
         const double ue = r.u_d[e];
         const bool need_l = ue > 0.0;
-        const int64_t ro = (int64_t)a.src[e] * a.Kp, co = (int64_t)a.col[e] * a.Kp;
+        const int64_t ro = (int64_t)src[e] * Kp, co = (int64_t)col[e] * Kp;
         double tot = 0.0, l = 0.0, mn = INFINITY;
         if constexpr (sizeof(T) == 4) {
             PairSum acc;
@@ -315,13 +356,13 @@ __global__ void __launch_bounds__(256) resid_edge_kernel(SweepArgs<T> a, ResidIn
             // bound of the lane's other elements
             float mn32 = INFINITY, lb = 0.f, best = 0.f, up = 0.f, up2 = 0.f;
             int at = -1;
-            const float4* fr = reinterpret_cast<const float4*>(a.f + e * a.Kp);
+            const float4* fr = reinterpret_cast<const float4*>(f + e * Kp);
             const float4* hi = reinterpret_cast<const float4*>(h32 + ro);
             const float4* hj = reinterpret_cast<const float4*>(h32 + co);
             double wi = 0.0, wj = 0.0;
             if (need_l) {
-                wi = r.inv_deg_d[a.src[e]];
-                wj = r.inv_deg_d[a.col[e]];
+                wi = r.inv_deg_d[src[e]];
+                wj = r.inv_deg_d[col[e]];
             }
 #pragma unroll 4
             for (int v = lane; v < nvec; v += 32) {
@@ -336,7 +377,7 @@ __global__ void __launch_bounds__(256) resid_edge_kernel(SweepArgs<T> a, ResidIn
                 }
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    if (k0 + j >= a.K) continue;  // the padding carries no commodity
+                    if (k0 + j >= K) continue;  // the padding carries no commodity
                     acc.add(xs[j]);
                     mn32 = fminf(mn32, xs[j]);
                     const float x0 = p[j] - q[j], sl = kHeightSlack * (fabsf(p[j]) + fabsf(q[j]));
@@ -356,7 +397,7 @@ __global__ void __launch_bounds__(256) resid_edge_kernel(SweepArgs<T> a, ResidIn
                 if (__any_sync(0xffffffffu, up2 > 0.f && up2 >= low)) {  // a lane holds several such elements
                     const float* si = h32 + ro;
                     const float* sj = h32 + co;
-                    for (int k = lane; k < a.K; k += 32) {
+                    for (int k = lane; k < K; k += 32) {
                         const float x0 = si[k] - sj[k], sl = kHeightSlack * (fabsf(si[k]) + fabsf(sj[k]));
                         if (x0 + sl > 0.f && x0 + sl >= low) l = fmax(l, h64[ro + k] * wi - h64[co + k] * wj);
                     }
@@ -366,8 +407,8 @@ __global__ void __launch_bounds__(256) resid_edge_kernel(SweepArgs<T> a, ResidIn
             for (int v = lane; v < nvec; v += 32) {
                 const int k0 = 4 * v;
                 double x[4];
-                load4(reinterpret_cast<const double*>(a.f) + e * a.Kp + k0, x);
-                const int nk = a.K - k0 < 4 ? a.K - k0 : 4;  // the padding carries no commodity
+                load4(reinterpret_cast<const double*>(f) + e * Kp + k0, x);
+                const int nk = K - k0 < 4 ? K - k0 : 4;  // the padding carries no commodity
                 for (int j = 0; j < nk; ++j) {
                     tot += x[j];
                     mn = fmin(mn, x[j]);
@@ -402,11 +443,17 @@ __global__ void __launch_bounds__(256) resid_edge_kernel(SweepArgs<T> a, ResidIn
 
 // One block; its time is the latency of the K gathers and of the partials, so
 // every thread keeps several of them in flight.  FP32 flows: h64 holds Delta.
-template <typename T>
-__global__ void __launch_bounds__(1024) resid_final_kernel(SweepArgs<T> a, ResidIn r, const double* __restrict__ h64,
-                                                           const double* __restrict__ part, int32_t grid_v,
-                                                           int32_t grid_e, ResidOut* __restrict__ out)
+template <typename T, bool TABLE>
+__global__ void __launch_bounds__(1024)
+    resid_final_kernel(const ResidTask<T>* __restrict__ tasks, const __grid_constant__ ResidTask<T> one)
 {
+    const ResidTask<T>& task = TABLE ? tasks[blockIdx.x] : one;
+    const SweepArgs<T>& a = task.a;
+    const ResidIn r = task.r;
+    const double* const h64 = task.h64;
+    const double* const part = task.part;
+    const int grid_v = task.grid_v, grid_e = task.grid_e;
+    ResidOut* const out = task.out;
     __shared__ double smem[5][32];
     const double* dem_d = r.dem_d;
     double gain = 0.0, gabs = 0.0;
@@ -455,22 +502,32 @@ __global__ void __launch_bounds__(1024) resid_final_kernel(SweepArgs<T> a, Resid
 
 int resid_part_count(int32_t grid_v, int32_t grid_e) { return grid_v * kVParts + grid_e * kEParts; }
 
-template <typename T>
-cudaError_t launch_residuals(const SweepArgs<T>& a, const ResidIn& r, double* h64, double* part, int32_t grid_v,
-                             int32_t grid_e, ResidOut* out, cudaStream_t stream)
+template <typename T, bool TABLE>
+void launch_passes(const ResidTask<T>* tasks, const ResidTask<T>& one, int count, int gv, int ge, int longest, cudaStream_t stream)
 {
-    if constexpr (sizeof(T) == 4) resid_vertex_pair_kernel<<<grid_v, 256, 0, stream>>>(a, r, a.h, h64, part);
-    else resid_vertex_kernel<<<grid_v, 256, 0, stream>>>(a, r, h64, part);
-    const float* h32 = sizeof(T) == 4 ? reinterpret_cast<const float*>(a.h) : nullptr;
-    resid_edge_kernel<T><<<grid_e, 256, 0, stream>>>(a, r, h32, h64, part + (int64_t)grid_v * kVParts);
-    const int longest = a.K > grid_v ? (a.K > grid_e ? a.K : grid_e) : (grid_v > grid_e ? grid_v : grid_e);
-    resid_final_kernel<T><<<1, longest > 256 ? 1024 : 256, 0, stream>>>(a, r, h64, part, grid_v, grid_e, out);
+    if constexpr (sizeof(T) == 4) resid_vertex_pair_kernel<TABLE><<<dim3(gv, count), 256, 0, stream>>>(tasks, one);
+    else resid_vertex_kernel<TABLE><<<dim3(gv, count), 256, 0, stream>>>(tasks, one);
+    resid_edge_kernel<T, TABLE><<<dim3(ge, count), 256, 0, stream>>>(tasks, one);
+    resid_final_kernel<T, TABLE><<<count, longest > 256 ? 1024 : 256, 0, stream>>>(tasks, one);
+}
+
+template <typename T>
+cudaError_t launch_residuals(const ResidTask<T>* tasks, const ResidTask<T>* host, int count, cudaStream_t stream)
+{
+    int gv = 1, ge = 1, longest = 1;
+    for (int i = 0; i < count; ++i) {
+        gv = host[i].grid_v > gv ? host[i].grid_v : gv;
+        ge = host[i].grid_e > ge ? host[i].grid_e : ge;
+        longest = host[i].a.K > longest ? host[i].a.K : longest;
+    }
+    longest = gv > longest ? gv : longest;
+    longest = ge > longest ? ge : longest;
+    if (tasks) launch_passes<T, true>(tasks, *host, count, gv, ge, longest, stream);
+    else launch_passes<T, false>(tasks, *host, 1, gv, ge, longest, stream);
     return cudaGetLastError();
 }
 
-template cudaError_t launch_residuals<float>(const SweepArgs<float>&, const ResidIn&, double*, double*, int32_t,
-                                             int32_t, ResidOut*, cudaStream_t);
-template cudaError_t launch_residuals<double>(const SweepArgs<double>&, const ResidIn&, double*, double*, int32_t,
-                                              int32_t, ResidOut*, cudaStream_t);
+template cudaError_t launch_residuals<float>(const ResidTask<float>*, const ResidTask<float>*, int, cudaStream_t);
+template cudaError_t launch_residuals<double>(const ResidTask<double>*, const ResidTask<double>*, int, cudaStream_t);
 
 }  // namespace pdr

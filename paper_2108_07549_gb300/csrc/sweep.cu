@@ -730,7 +730,6 @@ __global__ void __launch_bounds__(kThreads, 2) edge_pipe_kernel(SweepArgs<T> a)
 template <typename T, int V, int N>
 __device__ __forceinline__ void block_above(const T (&c)[V][N], T w, T& S, int& n, T& mn, T* sa, int* sb, T* sm)
 {
-    __syncwarp();  // a branch of thread 0 alone may lie just before
     T sl = T(0), ml = T(INFINITY);
     int nl = 0;
 #pragma unroll
@@ -767,6 +766,47 @@ __device__ __forceinline__ void block_above(const T (&c)[V][N], T w, T& S, int& 
     S = sa[32];
     n = sb[32];
     mn = sm[32];
+}
+
+// The root search over a block's row.  A failed warm start begins again from 0
+// and each pass has its own code: RootSearch's one loop keeps more values live
+// across a pass, and the spills that follow at these register caps cost more
+// than the passes it saves (512 x 5 at n = 10,000, K = 10,000: 672 against 654
+// us; 128 x 4 at n = 20,000, K = 2000: 396 against 376 us).
+template <typename T, int V, int N>
+__device__ __forceinline__ T block_root(const T (&c)[V][N], T ue, T w0, int den, int Kp, T* sa, int* sb, T* sm)
+{
+    T S, mn, theta = T(0);
+    int n, nA = 0;
+    bool done = false;
+    auto start = [&]() {  // w = 0
+        if (S <= ue) {    // Case 1 of Alg. 2: nothing to shed
+            theta = T(0);
+            done = true;
+        } else {  // Case 2 (S > u >= 0, so n >= 1)
+            theta = (S - ue) / T(den + n);
+            nA = n;
+            done = mn > theta;
+        }
+    };
+    block_above<T, V, N>(c, w0, S, n, mn, sa, sb, sm);
+    if (w0 <= T(0)) start();
+    else if (n > 0 && S - T(n) * w0 - ue - T(den) * w0 >= T(0)) {
+        theta = (S - ue) / T(den + n);
+        nA = n;
+        done = mn > theta;
+    } else {
+        block_above<T, V, N>(c, T(0), S, n, mn, sa, sb, sm);
+        start();
+    }
+    for (int it = 0; !done && it <= Kp + 2; ++it) {  // block-uniform
+        block_above<T, V, N>(c, theta, S, n, mn, sa, sb, sm);
+        if (n >= nA || n == 0) break;
+        nA = n;
+        theta = (S - ue) / T(den + n);
+        done = mn > theta;
+    }
+    return theta < T(0) ? T(0) : theta;  // a root below 0 is rounding at s = u: Case 1 (RootSearch::root)
 }
 
 // One block of B threads per edge; thread l keeps row vectors l + q*B.
@@ -834,15 +874,7 @@ __global__ void __launch_bounds__(B, block_min_blocks(B, V)) edge_block_kernel(S
         if (!psi_only) {
             // the lane-group search with block-wide sums, counts and minima
             const int den = a.ck ? 0 : 2;
-            RootSearch<T> rs(a.theta_in[a.m + e], true);
-            int it = 0;
-            do {  // block-uniform
-                T S, mn;
-                int n;
-                block_above<T, V, N>(c, rs.w, S, n, mn, sa_buf, sb_buf, sm_buf);
-                rs.step(S, n, mn, ue, den);
-            } while (!rs.done && ++it <= a.Kp + 4);
-            const T theta = rs.root();
+            const T theta = block_root<T, V, N>(c, ue, a.theta_in[a.m + e], den, a.Kp, sa_buf, sb_buf, sm_buf);
             if (threadIdx.x == 0) {
                 a.theta[a.m + e] = next_warm_start(theta, a.theta_in[e]);
                 a.theta[e] = theta;
@@ -1091,15 +1123,7 @@ __global__ void __launch_bounds__(B, 1) edge_staged_kernel(SweepArgs<T> a)
         T psi;
         if (!psi_only) {
             const int den = a.ck ? 0 : 2;
-            RootSearch<T> rs(a.theta_in[a.m + e], true);
-            int it = 0;
-            do {  // block-uniform
-                T S, mn;
-                int n;
-                block_above<T, V, N>(c, rs.w, S, n, mn, sa_buf, sb_buf, sm_buf);
-                rs.step(S, n, mn, ue, den);
-            } while (!rs.done && ++it <= a.Kp + 4);
-            const T theta = rs.root();
+            const T theta = block_root<T, V, N>(c, ue, a.theta_in[a.m + e], den, a.Kp, sa_buf, sb_buf, sm_buf);
             if (threadIdx.x == 0) {
                 a.theta[a.m + e] = next_warm_start(theta, a.theta_in[e]);
                 a.theta[e] = theta;
