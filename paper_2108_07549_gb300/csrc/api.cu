@@ -153,6 +153,7 @@ struct pdr_ctx {
     int32_t* xv_start[kExcessForms] = {};
     int64_t n_psi[2] = {1, 1};
     int pgrid[2] = {0, 0};         // persistent kernel grid per precision (0: not available)
+    int ring[2] = {0, 0};          // edge kernel: the ring form (per precision)
     int64_t pf[2] = {0, 0};        // edge-kernel L2 prefetch distance per precision (edges)
     GridBarrier* bar = nullptr;    // its grid barrier
     DevState* st = nullptr;
@@ -344,6 +345,7 @@ SweepArgs<T> make_args(pdr_ctx* ctx, int mode, int use_cond = 0, cudaGraphCondit
     a.n_psi = ctx->n_psi[p];
     a.pf_edges = ctx->pf[p];
     a.l2_hints = ctx->pf[p] > 0 ? 1 : 0;
+    a.ring = ctx->ring[p];
     a.psi_out = nullptr;
     a.st = ctx->st;
     a.trace = ctx->trace;
@@ -513,6 +515,17 @@ int64_t prefetch_policy(const pdr_ctx* ctx, int cfg)
     return rows * sizeof(T) > kL2Bytes ? edge_prefetch_distance<T>(cfg, ctx->num_sms) : 0;
 }
 
+// Grid, partials and form (plain or ring) of edge variant cfg.
+template <typename T>
+void set_edge_grid(pdr_ctx* ctx, int cfg, const pdr_options& o)
+{
+    const int p = Prec<T>::id;
+    const int ring = is_gd(o) ? 0 : edge_ring_grid<T>(cfg, ctx->m, ctx->Kp, ctx->num_sms);
+    ctx->ring[p] = ring > 0 ? 1 : 0;
+    ctx->grid_e[p] = ring > 0 ? ring : edge_grid<T>(cfg, ctx->m, ctx->num_sms);
+    ctx->n_psi[p] = edge_parts<T>(cfg, ctx->grid_e[p]);
+}
+
 // The edge-kernel variant of each precision: the caller's (it must hold the
 // rows in every precision the solve uses) or the library's choice.  Sets
 // cfg, grid_e and n_psi; cfg = -1 for a precision whose rows no variant holds.
@@ -537,10 +550,9 @@ pdr_status select_edge_variants(pdr_ctx* ctx, const pdr_options& o)
                          "K = " + std::to_string(ctx->K) + " exceeds the largest edge-kernel row supported by this build");
     ctx->cfg[0] = c32;
     ctx->cfg[1] = c64;
-    ctx->grid_e[0] = edge_grid<float>(c32, ctx->m, ctx->num_sms);
-    ctx->grid_e[1] = c64 >= 0 ? edge_grid<double>(c64, ctx->m, ctx->num_sms) : 1;
-    ctx->n_psi[0] = edge_parts<float>(c32, ctx->grid_e[0]);
-    ctx->n_psi[1] = c64 >= 0 ? edge_parts<double>(c64, ctx->grid_e[1]) : 1;
+    set_edge_grid<float>(ctx, c32, o);
+    if (c64 >= 0) set_edge_grid<double>(ctx, c64, o);
+    else ctx->grid_e[1] = 1, ctx->n_psi[1] = 1, ctx->ring[1] = 0;
     // L2 prefetch of later waves' rows pays only when the rows come from HBM:
     // when both flow buffers and the heights fit in L2 (as they stay across
     // sweeps) the prefetches are pure overhead
@@ -1084,7 +1096,7 @@ pdr_status run_phase(pdr_ctx* ctx, int64_t t_start)
     // The sweep that stopped also ran its edge QPs (their output is
     // discarded) and wrote their congestion partials: recompute those of the
     // returned flows f^(t), keeping the warm starts.  A stop by the sweep cap
-    // skipped those updates (final_evaluation), so its partials are still
+    // skipped those updates (update_skipped), so its partials are still
     // the returned flows'.
     if (ctx->hst->stop && ctx->hst->reason != STOP_MAX_SWEEPS) return refresh_psi<T>(ctx, nullptr, true);
     return PDR_OK;
@@ -1650,7 +1662,7 @@ pdr_status pdr_set_options(pdr_ctx* ctx, const pdr_options* opt)
     if (opt) o = *opt;
     std::string why;
     if (!options_ok(&o, &why)) return ctx->fail(PDR_ERR_INVALID_ARG, why);
-    const bool variant_changed = o.edge_variant != ctx->opt.edge_variant ||
+    const bool variant_changed = o.edge_variant != ctx->opt.edge_variant || is_gd(o) != is_gd(ctx->opt) ||
                                  (o.precision != PDR_PREC_FP32 && ctx->cfg[1] < 0);
     if (variant_changed) {
         const pdr_status vs = select_edge_variants(ctx, o);  // writes nothing on failure
@@ -2506,8 +2518,7 @@ pdr_status autotune(pdr_ctx* ctx, int32_t* best_cfg, double* best_us)
     double best = 1e30;
     for (int c : cand) {
         ctx->cfg[p] = c;
-        ctx->grid_e[p] = edge_grid<T>(c, ctx->m, ctx->num_sms);
-        ctx->n_psi[p] = edge_parts<T>(c, ctx->grid_e[p]);
+        set_edge_grid<T>(ctx, c, ctx->opt);
         ctx->pf[p] = prefetch_policy<T>(ctx, c);
         double tot = 0.0;
         for (int r = 0; r < 4; ++r) {
@@ -2533,8 +2544,7 @@ pdr_status autotune(pdr_ctx* ctx, int32_t* best_cfg, double* best_us)
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     ctx->cfg[p] = *best_cfg;
-    ctx->grid_e[p] = edge_grid<T>(*best_cfg, ctx->m, ctx->num_sms);
-    ctx->n_psi[p] = edge_parts<T>(*best_cfg, ctx->grid_e[p]);
+    set_edge_grid<T>(ctx, *best_cfg, ctx->opt);
     ctx->pf[p] = prefetch_policy<T>(ctx, *best_cfg);
     ctx->pgrid[p] = persistent_grid<T>(*best_cfg, ctx->m, ctx->n, ctx->Kp, ctx->num_sms);
     *best_us = best;

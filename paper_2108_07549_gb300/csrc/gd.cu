@@ -40,12 +40,13 @@ __global__ void __launch_bounds__(kThreads) gd_group_kernel(SweepArgs<T> a)
     constexpr int N = VecOf<T>::N;
     constexpr int GPW = 32 / G;
     volatile DevState* vst = a.st;
-    if (sweep_stopped(a)) return;  // an earlier sweep of this solve stopped
-    if (blockIdx.x == gridDim.x - 1) {               // the decision block
+    const int skip = update_skipped(a);
+    if (skip == 1) return;              // an earlier sweep of this solve stopped
+    if (blockIdx.x == gridDim.x - 1) {  // the decision block
         if (a.mode != MODE_PSI) reduce_and_finalize(a);
         return;
     }
-    if (final_evaluation(a)) return;  // the sweep cap stops this sweep: its output is not used
+    if (skip) return;  // the sweep cap stops this sweep: its output is not used
     const bool grow = (vst->t_sweep % 10) == 0;
     const int lane = threadIdx.x & 31;
     const int gl = lane & (G - 1);
@@ -170,12 +171,13 @@ __global__ void __launch_bounds__(B, gd_min_blocks(B, V)) gd_block_kernel(SweepA
     __shared__ int sb_buf[33];
     __shared__ T sc_buf[33];
     volatile DevState* vst = a.st;
-    if (sweep_stopped(a)) return;  // an earlier sweep of this solve stopped
+    const int skip = update_skipped(a);
+    if (skip == 1) return;  // an earlier sweep of this solve stopped
     if (blockIdx.x == gridDim.x - 1) {
         if (a.mode != MODE_PSI) reduce_and_finalize(a);
         return;
     }
-    if (final_evaluation(a)) return;  // the sweep cap stops this sweep: its output is not used
+    if (skip) return;  // the sweep cap stops this sweep: its output is not used
     const bool grow = (vst->t_sweep % 10) == 0;
     const int vpr = a.Kp / N;
     typename A::V zpsi = A::zero();

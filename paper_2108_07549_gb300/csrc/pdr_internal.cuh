@@ -148,6 +148,7 @@ struct SweepArgs {
     int64_t n_psi;      // number of edge partials
     int64_t pf_edges;   // edge QP: L2 prefetch of the rows of edge e + pf_edges while
                         // edge e is solved (about one wave of resident edges ahead; 0: off)
+    int ring;           // edge QP: 1 = the ring form of a 32-lane variant (grid_e from edge_ring_grid)
     int l2_hints;       // 1: the working set exceeds L2; the edge QP streams flow rows evict-first
     // Alg. 3 / Alg. 4 state (double-buffered like the flows) and parameters
     const T* beta_in;   // [m] learning rates beta_ij of iteration t
@@ -181,6 +182,8 @@ template <typename T>
 int edge_config(int Kp);  // picks the edge-kernel variant for a row length
 template <typename T>
 int edge_grid(int cfg, int64_t m, int num_sms);  // grid size of that variant
+template <typename T>
+int edge_ring_grid(int cfg, int64_t m, int Kp, int num_sms);  // the ring form's, 0 where it does not apply
 template <typename T>
 int64_t edge_parts(int cfg, int grid);  // number of partials that grid writes
 template <typename T>

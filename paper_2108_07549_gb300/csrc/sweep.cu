@@ -596,14 +596,164 @@ template <typename T, int G, int V>
 __global__ void __launch_bounds__(kThreads) edge_group_kernel(SweepArgs<T> a)
 {
     pdl_wait();  // the excess kernel has finished (no-op without PDL)
-    volatile DevState* vst = a.st;
-    if (sweep_stopped(a)) return;  // an earlier sweep of this solve stopped
-    if (blockIdx.x == gridDim.x - 1) {               // the decision block
+    const int skip = update_skipped(a);
+    if (skip == 1) return;              // an earlier sweep of this solve stopped
+    if (blockIdx.x == gridDim.x - 1) {  // the decision block
         if (a.mode != MODE_PSI) reduce_and_finalize(a);
         return;
     }
-    if (final_evaluation(a)) return;  // the sweep cap stops this sweep: its output is not used
+    if (skip) return;  // the sweep cap stops this sweep: its output is not used
     edge_group_body<T, G, V, false>(a, blockIdx.x, gridDim.x - 1);
+}
+
+// ------------------------------------------------------------------ edge QP, ring lane-group form
+//
+// The 32-lane variants when there are more edges than resident warps.  One
+// wave of blocks; each warp walks a stride of edges and has the next edge's
+// three rows on the way into its own slice of shared memory (cp.async.bulk)
+// while it solves the current one from registers.  The plain form's time went
+// into the chain index loads -> row loads -> search, once per edge with
+// nothing in flight meanwhile, and into a last wave that was nearly empty
+// (knn graph with m = 15,000, K = 500: 1876 blocks, 3.1 waves, 46 % of the
+// warps active).  Holding the next rows in registers instead leaves half the
+// warps (edge_pipe_kernel).  Per element the arithmetic is the plain form's,
+// so the flows are bit-identical to it.  Each wait is limited
+// (a.wait_cycles); a warp whose wait runs out records the fault, ends the
+// solve, waits (limited) for its copies and leaves.
+template <typename T>
+__host__ __device__ constexpr size_t ring_stage_bytes(int Kp)  // f, h_i, h_j
+{
+    return 3 * (size_t)Kp * sizeof(T);
+}
+template <typename T>
+size_t ring_smem(int Kp)
+{
+    return (kThreads / 32) * ring_stage_bytes<T>(Kp);
+}
+
+template <typename T, int V>
+__global__ void __launch_bounds__(kThreads) edge_ring_kernel(SweepArgs<T> a)
+{
+    using VT = typename VecOf<T>::type;
+    using A = Acc<T>;
+    constexpr int N = VecOf<T>::N, W = kThreads / 32;
+    extern __shared__ __align__(128) unsigned char rsm[];
+    __shared__ __align__(8) uint64_t full[W];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const bool decision = blockIdx.x == gridDim.x - 1;
+    const int64_t stride = (int64_t)(gridDim.x - 1) * W;
+    int64_t e = (int64_t)blockIdx.x * W + w;
+    const int vpr = a.Kp / N;
+    const uint32_t row_bytes = (uint32_t)a.Kp * (uint32_t)sizeof(T);
+    unsigned char* const slice = rsm + (size_t)w * 3 * row_bytes;
+    const bool hint = a.l2_hints != 0;
+    const uint64_t pol_first = l2_evict_first();
+    // an edge's endpoints and capacity do not change during a solve: read
+    // the first ones before waiting for the previous kernel
+    const bool any = !decision && e < a.m;
+    int32_t si = any ? a.src[e] : 0, sj = any ? a.col[e] : 0;
+    T ue = any ? a.u[e] : T(0);
+    if (lane == 0) {
+        mbar_init(&full[w], 1);
+        mbar_init_fence();
+    }
+    __syncwarp();
+    auto stage = [&](int64_t x, int32_t i, int32_t j) {  // lane 0
+        mbar_arrive_expect_tx(&full[w], 3u * row_bytes);
+        if (hint) bulk_g2s_hint(slice, a.f + x * a.Kp, row_bytes, &full[w], pol_first);
+        else bulk_g2s(slice, a.f + x * a.Kp, row_bytes, &full[w]);
+        bulk_g2s(slice + row_bytes, a.h + (int64_t)i * a.Kp, row_bytes, &full[w]);
+        bulk_g2s(slice + 2 * (size_t)row_bytes, a.h + (int64_t)j * a.Kp, row_bytes, &full[w]);
+    };
+    pdl_wait();     // the excess kernel has finished (no-op without PDL)
+    pdl_trigger();  // one wave
+    if (any && lane == 0) stage(e, si, sj);
+    __syncwarp();
+    const int skip = update_skipped(a);
+    if (decision) {
+        if (skip != 1) reduce_and_finalize(a);
+        return;
+    }
+    if (skip) {  // the first copy, then leave
+        if (any) mbar_wait(&full[w], 0, a.wait_cycles);
+        return;
+    }
+    const int den = a.ck ? 0 : 2;
+    typename A::V zpsi = A::zero();
+    T capmax = T(0);
+    uint32_t phase = 0;
+    for (; e < a.m; e += stride) {
+        const int64_t en = e + stride;
+        const bool more = en < a.m;
+        const T w0 = a.theta_in[a.m + e], prev = a.theta_in[e], isc = a.inv_scale_t[e];
+        T un = T(0);
+        if (more) {
+            si = a.src[en];
+            sj = a.col[en];
+            un = a.u[en];
+        }
+        if (!__all_sync(kFull, mbar_wait(&full[w], phase, a.wait_cycles))) {
+            if (lane == 0) {
+                a.st->fault = 1;
+                stop_from_kernel(a);
+            }
+            __syncwarp();
+            mbar_wait(&full[w], phase, a.wait_cycles);
+            break;
+        }
+        phase ^= 1u;
+        T c[V][N];
+        const VT* sf = reinterpret_cast<const VT*>(slice);
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            const int v = lane + q * 32;
+            if (v < vpr) {
+                T fx[N], ax[N], bx[N];
+                unpack(sf[v], fx);
+                unpack(sf[vpr + v], ax);
+                unpack(sf[2 * vpr + v], bx);
+#pragma unroll
+                for (int j = 0; j < N; ++j) c[q][j] = fma(T(0.5), ax[j] - bx[j], fx[j]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < N; ++j) c[q][j] = T(0);
+            }
+        }
+        __syncwarp();  // the rows are in registers: the slice is free
+        if (more && lane == 0) stage(en, si, sj);
+        __syncwarp();
+        const T theta = qp_root_group<T, 32, V, N>(c, ue, w0, true, a.Kp, den);
+        VT* orow = reinterpret_cast<VT*>(a.f_out + e * a.Kp);
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            const int v = lane + q * 32;
+            T o[N];
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                const T x = c[q][j] - theta;
+                o[j] = x > T(0) ? x : T(0);
+            }
+            if (v < vpr) {
+                if (hint) st_hint(orow + v, pack4(o), pol_first);
+                else orow[v] = pack4(o);
+            }
+        }
+        const T psi = T(den) * theta;  // sum f' - u at the root
+        if (lane == 0) {
+            a.theta[a.m + e] = next_warm_start(theta, prev);
+            a.theta[e] = theta;
+            zpsi = A::add(zpsi, psi * psi);
+            const T cc = psi * isc;
+            capmax = cc > capmax ? cc : capmax;
+        }
+        ue = un;
+    }
+    warp_acc_max<T>(zpsi, capmax);
+    if (lane == 0) {
+        const int64_t part = (int64_t)blockIdx.x * W + w;
+        reinterpret_cast<typename A::S*>(a.part_psi)[part] = A::store(zpsi);
+        a.part_cap[part] = capmax;
+    }
 }
 
 // ------------------------------------------------------------------ edge QP, pipelined lane-group form
@@ -640,13 +790,13 @@ __global__ void __launch_bounds__(kThreads, 2) edge_pipe_kernel(SweepArgs<T> a)
     using VT = typename VecOf<T>::type;
     using A = Acc<T>;
     constexpr int N = VecOf<T>::N;
-    volatile DevState* vst = a.st;
-    if (sweep_stopped(a)) return;  // an earlier sweep of this solve stopped
+    const int skip = update_skipped(a);
+    if (skip == 1) return;  // an earlier sweep of this solve stopped
     if (blockIdx.x == gridDim.x - 1) {
         if (a.mode != MODE_PSI) reduce_and_finalize(a);
         return;
     }
-    if (final_evaluation(a)) return;  // the sweep cap stops this sweep: its output is not used
+    if (skip) return;  // the sweep cap stops this sweep: its output is not used
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)(gridDim.x - 1) * blockDim.x) >> 5;
@@ -820,13 +970,13 @@ __global__ void __launch_bounds__(B, block_min_blocks(B, V)) edge_block_kernel(S
     __shared__ T sa_buf[33];
     __shared__ int sb_buf[33];
     __shared__ T sm_buf[33];
-    volatile DevState* vst = a.st;
-    if (sweep_stopped(a)) return;  // an earlier sweep of this solve stopped
-    if (blockIdx.x == gridDim.x - 1) {               // the decision block
+    const int skip = update_skipped(a);
+    if (skip == 1) return;              // an earlier sweep of this solve stopped
+    if (blockIdx.x == gridDim.x - 1) {  // the decision block
         if (a.mode != MODE_PSI) reduce_and_finalize(a);
         return;
     }
-    if (final_evaluation(a)) return;  // the sweep cap stops this sweep: its output is not used
+    if (skip) return;  // the sweep cap stops this sweep: its output is not used
     const int vpr = a.Kp / N;
     const bool psi_only = (a.mode == MODE_PSI);
     const bool hint = a.l2_hints != 0;
@@ -1050,13 +1200,13 @@ __global__ void __launch_bounds__(B, 1) edge_staged_kernel(SweepArgs<T> a)
     __shared__ T sa_buf[33];
     __shared__ int sb_buf[33];
     __shared__ T sm_buf[33];
-    volatile DevState* vst = a.st;
-    if (sweep_stopped(a)) return;  // an earlier sweep of this solve stopped
+    const int skip = update_skipped(a);
+    if (skip == 1) return;  // an earlier sweep of this solve stopped
     if (blockIdx.x == gridDim.x - 1) {  // the decision block
         if (a.mode != MODE_PSI) reduce_and_finalize(a);
         return;
     }
-    if (final_evaluation(a)) return;  // the sweep cap stops this sweep: its output is not used
+    if (skip) return;  // the sweep cap stops this sweep: its output is not used
     const int nb = gridDim.x - 1;
     const int vpr = a.Kp / N;
     const uint32_t row_bytes = (uint32_t)a.Kp * (uint32_t)sizeof(T);
@@ -1255,6 +1405,8 @@ constexpr EdgeCfg kCfg[] = {
     // rows into shared memory: 3 rows of up to 40 / 64 KB)
     {0, 512, 5, 2}, {0, 512, 8, 2},
 };
+constexpr int kRingSmemMax = 224 * 1024;
+constexpr double kRingWaves = 0.3;
 constexpr int kFirstPipelined = 16;
 constexpr int kFirstStaged = 19;
 constexpr int kNumCfg = sizeof(kCfg) / sizeof(kCfg[0]);
@@ -1466,10 +1618,58 @@ cudaError_t launch_finalize(const SweepArgs<T>& a, cudaStream_t stream)
     return cudaGetLastError();
 }
 
+template <typename T, int V>
+int ring_blocks(int Kp, int num_sms)
+{
+    const size_t smem = ring_smem<T>(Kp);
+    int blocks = 0;
+    if (cudaFuncSetAttribute(edge_ring_kernel<T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingSmemMax) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, edge_ring_kernel<T, V>, kThreads, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return blocks * num_sms;
+}
+
+// Blocks of the ring form (one wave, less the decision block's slot), or 0
+// where it does not apply: FP32, a 32-lane variant, rows that fit, and edges
+// for at least kRingWaves of its resident warps (below, the plain form's
+// direct loads are as fast).  Sweeps in the graph loop, us, plain / ring (n, m,
+// K): 1500, 9000, 120: 14.7 / 11.9; 2500, 15,000, 500: 27.0 / 25.2; 5000,
+// 25,000, 600: 66.8 / 45.2; 12,000, 36,000, 530: 96.0 / 73.5; 20,000, 100,000,
+// 500: 185 / 170; 900, 3480, 501 (0.7 of its warps): 11.6 / 10.8.
+template <typename T>
+int edge_ring_grid(int cfg, int64_t m, int Kp, int num_sms)
+{
+    if (sizeof(T) != 4 || cfg < 3 || cfg > 6 || ring_smem<T>(Kp) > (size_t)kRingSmemMax) return 0;
+    const int blocks = cfg == 3   ? ring_blocks<T, 1>(Kp, num_sms)
+                       : cfg == 4 ? ring_blocks<T, 2>(Kp, num_sms)
+                       : cfg == 5 ? ring_blocks<T, 4>(Kp, num_sms)
+                                  : ring_blocks<T, 8>(Kp, num_sms);
+    const int64_t warps = (int64_t)blocks * (kThreads / 32);
+    if (blocks < 2 || (double)m < kRingWaves * (double)warps) return 0;
+    // the same number of edges for every warp, as nearly as it goes
+    const int64_t rounds = (m + warps - 1) / warps, need = (m + rounds - 1) / rounds;
+    const int64_t g = (need + kThreads / 32 - 1) / (kThreads / 32);
+    return (int)(g < blocks - 1 ? g : blocks - 1);
+}
+template int edge_ring_grid<float>(int, int64_t, int, int);
+template int edge_ring_grid<double>(int, int64_t, int, int);
+
 template <typename T>
 cudaError_t launch_edge(const SweepArgs<T>& a, int cfg, cudaStream_t stream, bool pdl)
 {
     const int g = a.grid_e + 1;  // edge blocks plus the decision block
+    if (a.ring && a.mode != MODE_PSI) {
+        const size_t smem = ring_smem<T>(a.Kp);
+        switch (cfg) {
+        case 3: return launch_one<T>(edge_ring_kernel<T, 1>, g, kThreads, stream, pdl, a, smem);
+        case 4: return launch_one<T>(edge_ring_kernel<T, 2>, g, kThreads, stream, pdl, a, smem);
+        case 5: return launch_one<T>(edge_ring_kernel<T, 4>, g, kThreads, stream, pdl, a, smem);
+        case 6: return launch_one<T>(edge_ring_kernel<T, 8>, g, kThreads, stream, pdl, a, smem);
+        default: return cudaErrorInvalidValue;
+        }
+    }
     switch (cfg) {
     case 0: return launch_one<T>(edge_group_kernel<T, 4, 1>, g, kThreads, stream, pdl, a);
     case 1: return launch_one<T>(edge_group_kernel<T, 8, 1>, g, kThreads, stream, pdl, a);

@@ -404,23 +404,29 @@ __device__ __forceinline__ bool sweep_stopped(const SweepArgs<T>& a)
     return stopped != 0;
 }
 
-// True in an edge kernel's update blocks during a solve's evaluation at
-// t = max_sweeps: that sweep stops by the sweep cap whatever its objective,
-// so its new flows would be discarded and the updates are skipped.  The
-// congestion partials of the returned flows f^(t), written by the previous
-// sweep's edge kernel, then stay in place.  t_sweep is the t of the sweep in
-// flight (written by the excess kernel before this launch may start), so the
-// decision block advancing t in the same launch does not affect the test.
+// Both tests of an update kernel in one read of the state (two dependent reads
+// and barriers cost about a microsecond at the start of every block):
+// 0 go on; 1 an earlier sweep stopped (as sweep_stopped); 2 the final
+// evaluation at t = max_sweeps, which only the decision block takes part in:
+// that sweep stops by the sweep cap whatever its objective, so its new flows
+// would be discarded, and the congestion partials of the returned flows f^(t),
+// written by the previous sweep's update kernel, stay in place.  t_sweep is the
+// t of the sweep in flight (written by the excess kernel before this launch may
+// start), so the decision block advancing t in the same launch does not affect
+// the test.
 template <typename T>
-__device__ __forceinline__ bool final_evaluation(const SweepArgs<T>& a)
+__device__ __forceinline__ int update_skipped(const SweepArgs<T>& a)
 {
-    __shared__ int fin;
+    __shared__ int skip;
     if (threadIdx.x == 0) {
         const volatile DevState* v = a.st;
-        fin = a.mode == MODE_SOLVE && v->t_sweep >= v->max_sweeps;
+        const int stop = v->stop;
+        const long long t = v->t_sweep, most = v->max_sweeps;
+        skip = a.mode != MODE_SOLVE ? 0 : stop ? 1 : t >= most ? 2 : 0;
+        if (skip == 1 && a.use_cond && !a.active && blockIdx.x == 0) cudaGraphSetConditional(a.cond, 0);
     }
     __syncthreads();
-    return fin != 0;
+    return skip;
 }
 
 // Ends this instance's solve from a kernel other than the decision block
