@@ -146,7 +146,7 @@ struct pdr_ctx {
     double* part_h = nullptr;
     // partials typed by the working precision: 8 bytes per entry covers both
     double *part_cons = nullptr, *part_capb = nullptr, *part_psi = nullptr, *part_cap = nullptr;
-    int grid_v[2] = {1, 1}, grid_e[2] = {1, 1}, cfg[2] = {-1, -1};
+    int grid_v[2] = {1, 1}, grid_e[2] = {1, 1}, cfg[2] = {-1, -1}, shares[2] = {1, 1};
     // excess kernel form (0: gathers, 1..3: bulk copies); grid and vertex split of each bulk form
     int xform = 0;
     int xgrid[kExcessForms] = {};
@@ -346,6 +346,7 @@ SweepArgs<T> make_args(pdr_ctx* ctx, int mode, int use_cond = 0, cudaGraphCondit
     a.pf_edges = ctx->pf[p];
     a.l2_hints = ctx->pf[p] > 0 ? 1 : 0;
     a.ring = ctx->ring[p];
+    a.shares = ctx->shares[p];
     a.psi_out = nullptr;
     a.st = ctx->st;
     a.trace = ctx->trace;
@@ -522,8 +523,9 @@ void set_edge_grid(pdr_ctx* ctx, int cfg, const pdr_options& o)
     const int p = Prec<T>::id;
     const int ring = is_gd(o) ? 0 : edge_ring_grid<T>(cfg, ctx->m, ctx->Kp, ctx->num_sms);
     ctx->ring[p] = ring > 0 ? 1 : 0;
-    ctx->grid_e[p] = ring > 0 ? ring : edge_grid<T>(cfg, ctx->m, ctx->num_sms);
-    ctx->n_psi[p] = edge_parts<T>(cfg, ctx->grid_e[p]);
+    ctx->shares[p] = is_gd(o) || ring > 0 ? 1 : edge_shares<T>(cfg, ctx->m, ctx->num_sms);
+    ctx->grid_e[p] = ring > 0 ? ring : edge_grid<T>(cfg, ctx->m, ctx->num_sms, ctx->shares[p]);
+    ctx->n_psi[p] = edge_parts<T>(cfg, ctx->grid_e[p], ctx->shares[p]);
 }
 
 // The edge-kernel variant of each precision: the caller's (it must hold the
@@ -552,7 +554,7 @@ pdr_status select_edge_variants(pdr_ctx* ctx, const pdr_options& o)
     ctx->cfg[1] = c64;
     set_edge_grid<float>(ctx, c32, o);
     if (c64 >= 0) set_edge_grid<double>(ctx, c64, o);
-    else ctx->grid_e[1] = 1, ctx->n_psi[1] = 1, ctx->ring[1] = 0;
+    else ctx->grid_e[1] = 1, ctx->n_psi[1] = 1, ctx->ring[1] = 0, ctx->shares[1] = 1;
     // L2 prefetch of later waves' rows pays only when the rows come from HBM:
     // when both flow buffers and the heights fit in L2 (as they stay across
     // sweeps) the prefetches are pure overhead

@@ -50,10 +50,10 @@ __device__ __forceinline__ void above(const T (&c)[R][V][N], T w, T& S, int& n, 
 #pragma unroll
             for (int j = 0; j < N; ++j) {
                 const T x = c[r][q][j];
-                if (x > w) {
+                if (exceeds(x, w)) {
                     sl[r] += x;
                     ++nl;
-                    ml = x < ml ? x : ml;
+                    ml = min_pos(x, ml);
                 }
             }
     }
@@ -67,10 +67,7 @@ __device__ __forceinline__ void above(const T (&c)[R][V][N], T w, T& S, int& n, 
     } else {
         n = group_sum<P>(nl);
 #pragma unroll
-        for (int o = P / 2; o > 0; o >>= 1) {
-            const T y = __shfl_xor_sync(kFull, ml, o);
-            ml = y < ml ? y : ml;
-        }
+        for (int o = P / 2; o > 0; o >>= 1) ml = min_pos(__shfl_xor_sync(kFull, ml, o), ml);
         mn = ml;
     }
 }

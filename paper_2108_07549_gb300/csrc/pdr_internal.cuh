@@ -22,6 +22,7 @@
 namespace pdr {
 
 constexpr int kThreads = 256;  // block size of every sweep kernel
+constexpr int kShareThreads = 64;  // block size of the lane-group forms with several shares per lane
 constexpr int kExcessForms = 6;     // excess kernel forms: 0 gathers, 1..5 bulk copies
 // Resident blocks per SM that the block forms of the edge kernels are
 // compiled for (the register cap that follows from it: 65,536 / (B x that)).
@@ -149,6 +150,7 @@ struct SweepArgs {
     int64_t pf_edges;   // edge QP: L2 prefetch of the rows of edge e + pf_edges while
                         // edge e is solved (about one wave of resident edges ahead; 0: off)
     int ring;           // edge QP: 1 = the ring form of a 32-lane variant (grid_e from edge_ring_grid)
+    int shares;         // edge QP: shares per lane of a lane-group variant (1: the plain form)
     int l2_hints;       // 1: the working set exceeds L2; the edge QP streams flow rows evict-first
     // Alg. 3 / Alg. 4 state (double-buffered like the flows) and parameters
     const T* beta_in;   // [m] learning rates beta_ij of iteration t
@@ -181,11 +183,13 @@ cudaError_t launch_edge(const SweepArgs<T>& a, int cfg, cudaStream_t stream, boo
 template <typename T>
 int edge_config(int Kp);  // picks the edge-kernel variant for a row length
 template <typename T>
-int edge_grid(int cfg, int64_t m, int num_sms);  // grid size of that variant
+int edge_grid(int cfg, int64_t m, int num_sms, int shares);  // grid size of that variant
+template <typename T>
+int edge_shares(int cfg, int64_t m, int num_sms);  // shares of a lane of that variant (1, 2 or 4)
 template <typename T>
 int edge_ring_grid(int cfg, int64_t m, int Kp, int num_sms);  // the ring form's, 0 where it does not apply
 template <typename T>
-int64_t edge_parts(int cfg, int grid);  // number of partials that grid writes
+int64_t edge_parts(int cfg, int grid, int shares);  // number of partials that grid writes
 template <typename T>
 int edge_capacity(int cfg);             // elements per row a variant holds (-1 if none)
 int num_edge_configs();

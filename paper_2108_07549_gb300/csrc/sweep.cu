@@ -86,7 +86,7 @@ __device__ __forceinline__ void excess_body(const SweepArgs<T>& a, int block, in
 #pragma unroll
             for (int u = 0; u < 8; ++u)
 #pragma unroll
-                for (int j = 0; j < N; ++j) acc[j] = ev[u] >= 0 ? acc[j] + x[u][j] : acc[j] - x[u][j];
+                for (int j = 0; j < N; ++j) acc[j] += ev[u] >= 0 ? x[u][j] : -x[u][j];
         }
         if (q + 4 <= q1) {
             int32_t ev[4];
@@ -101,7 +101,7 @@ __device__ __forceinline__ void excess_body(const SweepArgs<T>& a, int block, in
 #pragma unroll
             for (int u = 0; u < 4; ++u)
 #pragma unroll
-                for (int j = 0; j < N; ++j) acc[j] = ev[u] >= 0 ? acc[j] + x[u][j] : acc[j] - x[u][j];
+                for (int j = 0; j < N; ++j) acc[j] += ev[u] >= 0 ? x[u][j] : -x[u][j];
             q += 4;
         }
         for (; q < q1; ++q) {
@@ -110,7 +110,7 @@ __device__ __forceinline__ void excess_body(const SweepArgs<T>& a, int block, in
             T x[N];
             unpack(reinterpret_cast<const VT*>(a.f + e * a.Kp)[v], x);
 #pragma unroll
-            for (int j = 0; j < N; ++j) acc[j] = ev >= 0 ? acc[j] + x[j] : acc[j] - x[j];
+            for (int j = 0; j < N; ++j) acc[j] += ev >= 0 ? x[j] : -x[j];
         }
         const int k0 = (int)v * N;
 #pragma unroll
@@ -131,7 +131,7 @@ __device__ __forceinline__ void excess_body(const SweepArgs<T>& a, int block, in
         for (int j = 0; j < N; ++j) {
             zt += dgt * hv[j] * hv[j];
             const T r = fabs(acc[j]) * a.inv_dem[k0 + j];
-            cons = r > cons ? r : cons;
+            cons = exceeds(r, cons) ? r : cons;
         }
         zacc = A::add(zacc, zt);
     }
@@ -438,7 +438,7 @@ __global__ void __launch_bounds__(C + 32) excess_bulk_kernel(SweepArgs<T> a)
                 for (int q = 0; q < N; ++q) {
                     zt += dgt * hv[q] * hv[q];
                     const T rr = fabs(acc[q]) * idk[q];
-                    cons = rr > cons ? rr : cons;
+                    cons = exceeds(rr, cons) ? rr : cons;
                 }
                 zacc = A::add(zacc, zt);
             }
@@ -485,17 +485,18 @@ __device__ __forceinline__ X ld_row(const X* p)
 }
 
 // Body of one edge-QP pass of the lane-group form, run by edge block `block`
-// of `nblocks` (the decision block is not counted).
-template <typename T, int G, int V, bool P>
+// of `nblocks` (the decision block is not counted).  The groups of G lanes run
+// on G / R of them, R shares per lane (edge_root.cuh); same results.
+template <typename T, int G, int R, int V, bool P>
 __device__ __forceinline__ void edge_group_body(const SweepArgs<T>& a, int block, int nblocks)
 {
     using VT = typename VecOf<T>::type;
     constexpr int N = VecOf<T>::N;
-    constexpr int GPW = 32 / G;  // groups per warp
+    constexpr int L = G / R, GPW = 32 / L;  // lanes per edge, edges per warp
     using A = Acc<T>;
     const int lane = threadIdx.x & 31;
-    const int gl = lane & (G - 1);
-    const int gw = lane / G;
+    const int gl = lane & (L - 1);
+    const int gw = lane / L;
     const int64_t warp = ((int64_t)block * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)nblocks * blockDim.x) >> 5;
     const int vpr = a.Kp / N;
@@ -506,48 +507,52 @@ __device__ __forceinline__ void edge_group_body(const SweepArgs<T>& a, int block
         const int64_t e = base + gw;
         const bool valid = e < a.m;
         if (a.pf_edges > 0 && valid && e + a.pf_edges < a.m)  // the flow row a later wave reads
-            prefetch_l2(a.f + (e + a.pf_edges) * a.Kp, (int64_t)a.Kp * sizeof(T), gl, G);
+            prefetch_l2(a.f + (e + a.pf_edges) * a.Kp, (int64_t)a.Kp * sizeof(T), gl, L);
         const T ue = valid ? a.u[e] : T(0);
-        T c[V][N];
+        T c[R][V][N];
         const T* frow = a.f + (valid ? e : 0) * a.Kp;
         T* orow = a.f_out + (valid ? e : 0) * a.Kp;
         if (psi_only) {
 #pragma unroll
-            for (int q = 0; q < V; ++q) {
-                const int v = gl + q * G;
-                if (valid && v < vpr) unpack(reinterpret_cast<const VT*>(frow)[v], c[q]);
-                else
+            for (int r = 0; r < R; ++r)
 #pragma unroll
-                    for (int j = 0; j < N; ++j) c[q][j] = T(0);
-            }
+                for (int q = 0; q < V; ++q) {
+                    const int v = gl + r * L + q * G;
+                    if (valid && v < vpr) unpack(reinterpret_cast<const VT*>(frow)[v], c[r][q]);
+                    else
+#pragma unroll
+                        for (int j = 0; j < N; ++j) c[r][q][j] = T(0);
+                }
         } else {
             const int i = valid ? a.src[e] : 0;
             const int jv = valid ? a.col[e] : 0;
             const VT* hi = reinterpret_cast<const VT*>(a.h + (int64_t)i * a.Kp);
             const VT* hj = reinterpret_cast<const VT*>(a.h + (int64_t)jv * a.Kp);
 #pragma unroll
-            for (int q = 0; q < V; ++q) {
-                const int v = gl + q * G;
-                if (valid && v < vpr) {
-                    T fx[N], ax[N], bx[N];
-                    unpack(reinterpret_cast<const VT*>(frow)[v], fx);
-                    unpack(ld_row<P>(hi + v), ax);
-                    unpack(ld_row<P>(hj + v), bx);
-                    // c_k = 1/2 ((h_ik + f_k) - (h_jk - f_k)) = f_k + (h_ik - h_jk)/2
+            for (int r = 0; r < R; ++r)
 #pragma unroll
-                    for (int j = 0; j < N; ++j) c[q][j] = fma(T(0.5), ax[j] - bx[j], fx[j]);
-                } else {
+                for (int q = 0; q < V; ++q) {
+                    const int v = gl + r * L + q * G;
+                    if (valid && v < vpr) {
+                        T fx[N], ax[N], bx[N];
+                        unpack(reinterpret_cast<const VT*>(frow)[v], fx);
+                        unpack(ld_row<P>(hi + v), ax);
+                        unpack(ld_row<P>(hj + v), bx);
+                        // c_k = 1/2 ((h_ik + f_k) - (h_jk - f_k)) = f_k + (h_ik - h_jk)/2
 #pragma unroll
-                    for (int j = 0; j < N; ++j) c[q][j] = T(0);
+                        for (int j = 0; j < N; ++j) c[r][q][j] = fma(T(0.5), ax[j] - bx[j], fx[j]);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < N; ++j) c[r][q][j] = T(0);
+                    }
                 }
-            }
         }
         T psi;
         if (!psi_only) {
             // warm start left by the previous sweep (roots in [0, m), starts in [m, 2m))
             const T w = valid ? a.theta_in[a.m + e] : T(0);
             const int den = a.ck ? 0 : 2;
-            const T theta = qp_root_group<T, G, V, N>(c, ue, w, valid, a.Kp, den);
+            const T theta = qp_root_group<T, L, R, V, N>(c, ue, w, valid, a.Kp, den);
             if (valid && gl == 0) {
                 a.theta[a.m + e] = next_warm_start(theta, a.theta_in[e]);
                 a.theta[e] = theta;
@@ -556,25 +561,31 @@ __device__ __forceinline__ void edge_group_body(const SweepArgs<T>& a, int block
             // congestion of the new flows is psi' = 2 theta for Alg. 2 and 0 with
             // the capacity kept (and 0 in Case 1)
 #pragma unroll
-            for (int q = 0; q < V; ++q) {
-                const int v = gl + q * G;
-                T o[N];
+            for (int r = 0; r < R; ++r)
 #pragma unroll
-                for (int j = 0; j < N; ++j) {
-                    const T x = c[q][j] - theta;
-                    o[j] = x > T(0) ? x : T(0);
+                for (int q = 0; q < V; ++q) {
+                    const int v = gl + r * L + q * G;
+                    T o[N];
+#pragma unroll
+                    for (int j = 0; j < N; ++j) {
+                        const T x = c[r][q][j] - theta;
+                        o[j] = exceeds(x, T(0)) ? x : T(0);
+                    }
+                    if (valid && v < vpr) reinterpret_cast<VT*>(orow)[v] = pack4(o);
                 }
-                if (valid && v < vpr) reinterpret_cast<VT*>(orow)[v] = pack4(o);
-            }
             psi = T(den) * theta;
         } else {
             // congestion of the stored flows
-            T rs = T(0);
+            T part[R];
 #pragma unroll
-            for (int q = 0; q < V; ++q)
+            for (int r = 0; r < R; ++r) {
+                part[r] = T(0);
 #pragma unroll
-                for (int j = 0; j < N; ++j) rs += c[q][j];
-            rs = group_sum<G>(rs);
+                for (int q = 0; q < V; ++q)
+#pragma unroll
+                    for (int j = 0; j < N; ++j) part[r] += c[r][q][j];
+            }
+            const T rs = share_sum<T, L, R>(part);
             psi = rs - ue > T(0) ? rs - ue : T(0);
         }
         if (valid && gl == 0) {
@@ -592,8 +603,12 @@ __device__ __forceinline__ void edge_group_body(const SweepArgs<T>& a, int block
     }
 }
 
-template <typename T, int G, int V>
-__global__ void __launch_bounds__(kThreads) edge_group_kernel(SweepArgs<T> a)
+// R > 1, FP64: the fixed cost of an edge (sums over the group, decisions, the
+// division: about 35 operations per lane and pass) is spent once per warp,
+// which then holds R times the edges.  Blocks of 64 threads, so that a few
+// hundred of these wider warps still spread evenly over the SMs.
+template <typename T, int G, int R, int V>
+__global__ void __launch_bounds__(R > 1 ? kShareThreads : kThreads) edge_group_kernel(SweepArgs<T> a)
 {
     pdl_wait();  // the excess kernel has finished (no-op without PDL)
     const int skip = update_skipped(a);
@@ -603,7 +618,7 @@ __global__ void __launch_bounds__(kThreads) edge_group_kernel(SweepArgs<T> a)
         return;
     }
     if (skip) return;  // the sweep cap stops this sweep: its output is not used
-    edge_group_body<T, G, V, false>(a, blockIdx.x, gridDim.x - 1);
+    edge_group_body<T, G, R, V, false>(a, blockIdx.x, gridDim.x - 1);
 }
 
 // ------------------------------------------------------------------ edge QP, ring lane-group form
@@ -731,7 +746,7 @@ __global__ void __launch_bounds__(kThreads) edge_ring_kernel(SweepArgs<T> a)
 #pragma unroll
             for (int j = 0; j < N; ++j) {
                 const T x = c[q][j] - theta;
-                o[j] = x > T(0) ? x : T(0);
+                o[j] = exceeds(x, T(0)) ? x : T(0);
             }
             if (v < vpr) {
                 if (hint) st_hint(orow + v, pack4(o), pol_first);
@@ -841,7 +856,7 @@ __global__ void __launch_bounds__(kThreads, 2) edge_pipe_kernel(SweepArgs<T> a)
 #pragma unroll
                 for (int j = 0; j < N; ++j) {
                     const T x = c[q][j] - theta;
-                    o[j] = x > T(0) ? x : T(0);
+                    o[j] = exceeds(x, T(0)) ? x : T(0);
                 }
                 if (v < vpr) reinterpret_cast<VT*>(orow)[v] = pack4(o);
             }
@@ -887,10 +902,10 @@ __device__ __forceinline__ void block_above(const T (&c)[V][N], T w, T& S, int& 
 #pragma unroll
         for (int j = 0; j < N; ++j) {
             const T x = c[q][j];
-            if (x > w) {
+            if (exceeds(x, w)) {
                 sl += x;
                 ++nl;
-                ml = x < ml ? x : ml;
+                ml = min_pos(x, ml);
             }
         }
     warp_sum_count_min(sl, nl, ml);
@@ -1040,7 +1055,7 @@ __global__ void __launch_bounds__(B, block_min_blocks(B, V)) edge_block_kernel(S
 #pragma unroll
                 for (int j = 0; j < N; ++j) {
                     const T x = c[q][j] - theta;
-                    o[j] = x > T(0) ? x : T(0);
+                    o[j] = exceeds(x, T(0)) ? x : T(0);
                 }
                 if (v < vpr) {
                     if (hint) st_hint(reinterpret_cast<VT*>(orow) + v, pack4(o), pol_first);
@@ -1154,7 +1169,7 @@ __global__ void __launch_bounds__(kThreads, (V <= 4 ? 4 : 3))
     if (psi_prologue) {
         SweepArgs<T> b = a;
         b.mode = MODE_PSI;
-        if ((int)blockIdx.x < nb) edge_group_body<T, G, V, true>(b, blockIdx.x, nb);
+        if ((int)blockIdx.x < nb) edge_group_body<T, G, 1, V, true>(b, blockIdx.x, nb);
         if (!grid_sync(bar, a.barrier_ns, hold)) return;
     }
     for (int64_t q = 0; q < sweeps; ++q) {
@@ -1169,7 +1184,7 @@ __global__ void __launch_bounds__(kThreads, (V <= 4 ? 4 : 3))
         excess_body<T>(b, blockIdx.x, gridDim.x);
         if (!grid_sync(bar, a.barrier_ns, hold)) return;
         if ((int)blockIdx.x == nb) reduce_and_finalize(b);
-        else edge_group_body<T, G, V, true>(b, blockIdx.x, nb);
+        else edge_group_body<T, G, 1, V, true>(b, blockIdx.x, nb);
         if (!grid_sync(bar, a.barrier_ns, hold)) return;
     }
 }
@@ -1285,7 +1300,7 @@ __global__ void __launch_bounds__(B, 1) edge_staged_kernel(SweepArgs<T> a)
 #pragma unroll
                 for (int j = 0; j < N; ++j) {
                     const T x = c[q][j] - theta;
-                    o[j] = x > T(0) ? x : T(0);
+                    o[j] = exceeds(x, T(0)) ? x : T(0);
                 }
                 if (v < vpr) st_hint(reinterpret_cast<VT*>(orow) + v, pack4(o), pol_first);
             }
@@ -1461,7 +1476,7 @@ void staged_setup(int cfg)
 }
 
 template <typename T>
-int edge_grid(int cfg, int64_t m, int num_sms)
+int edge_grid(int cfg, int64_t m, int num_sms, int shares)
 {
     const EdgeCfg& c = kCfg[cfg];
     int64_t want, cap;
@@ -1481,7 +1496,7 @@ int edge_grid(int cfg, int64_t m, int num_sms)
         return (int)(g < 1 ? 1 : g);
     }
     if (c.G) {
-        const int64_t per_block = kThreads / c.G;
+        const int64_t per_block = shares > 1 ? (int64_t)kShareThreads * shares / c.G : kThreads / c.G;
         want = (m + per_block - 1) / per_block;
     } else {
         want = m;
@@ -1500,9 +1515,9 @@ int edge_capacity(int cfg)
 int num_edge_configs() { return kNumCfg; }
 
 template <typename T>
-int64_t edge_parts(int cfg, int grid)
+int64_t edge_parts(int cfg, int grid, int shares)
 {
-    return kCfg[cfg].G ? (int64_t)grid * (kThreads / 32) : (int64_t)grid;
+    return kCfg[cfg].G ? (int64_t)grid * ((shares > 1 ? kShareThreads : kThreads) / 32) : (int64_t)grid;
 }
 
 // One wave of resident blocks (or fewer if the rows are fewer): the grid-
@@ -1656,6 +1671,38 @@ int edge_ring_grid(int cfg, int64_t m, int Kp, int num_sms)
 template int edge_ring_grid<float>(int, int64_t, int, int);
 template int edge_ring_grid<double>(int, int64_t, int, int);
 
+// Shares built for a lane-group variant: at most 16 row elements per lane.
+constexpr int share_limit(int G, int V) { return V >= 8 ? 1 : V >= 4 ? 2 : 4; }
+
+// Lanes' shares of variant cfg for m edges (1: the plain form): FP64 only, the
+// most that leave a warp to each of the SMs' four schedulers.  (FP32 has its
+// ring form, and its fixed cost per edge is on pipes that are not the bound.)
+// Bound: the FP64 pipe, two operations per clock and SM.  Together with the
+// comparisons made on bit patterns (exceeds), n 500, m 3000, K 100: 41 us per
+// sweep (about 100 FP64 warp instructions per edge) to 23.
+template <typename T>
+int edge_shares(int cfg, int64_t m, int num_sms)
+{
+    if (sizeof(T) != 8 || cfg < 0 || cfg >= kNumCfg || !kCfg[cfg].G || kCfg[cfg].P) return 1;
+    int r = share_limit(kCfg[cfg].G, kCfg[cfg].V);
+    while (r > 1 && m * kCfg[cfg].G < (int64_t)num_sms * 4 * 32 * r) r >>= 1;
+    return r;
+}
+template int edge_shares<float>(int, int64_t, int);
+template int edge_shares<double>(int, int64_t, int);
+
+template <typename T, int G, int V>
+cudaError_t launch_group(const SweepArgs<T>& a, int g, cudaStream_t stream, bool pdl)
+{
+    if constexpr (sizeof(T) == 8) {
+        if constexpr (share_limit(G, V) >= 4)
+            if (a.shares == 4) return launch_one<T>(edge_group_kernel<T, G, 4, V>, g, kShareThreads, stream, pdl, a);
+        if constexpr (share_limit(G, V) >= 2)
+            if (a.shares == 2) return launch_one<T>(edge_group_kernel<T, G, 2, V>, g, kShareThreads, stream, pdl, a);
+    }
+    return launch_one<T>(edge_group_kernel<T, G, 1, V>, g, kThreads, stream, pdl, a);
+}
+
 template <typename T>
 cudaError_t launch_edge(const SweepArgs<T>& a, int cfg, cudaStream_t stream, bool pdl)
 {
@@ -1671,13 +1718,13 @@ cudaError_t launch_edge(const SweepArgs<T>& a, int cfg, cudaStream_t stream, boo
         }
     }
     switch (cfg) {
-    case 0: return launch_one<T>(edge_group_kernel<T, 4, 1>, g, kThreads, stream, pdl, a);
-    case 1: return launch_one<T>(edge_group_kernel<T, 8, 1>, g, kThreads, stream, pdl, a);
-    case 2: return launch_one<T>(edge_group_kernel<T, 16, 1>, g, kThreads, stream, pdl, a);
-    case 3: return launch_one<T>(edge_group_kernel<T, 32, 1>, g, kThreads, stream, pdl, a);
-    case 4: return launch_one<T>(edge_group_kernel<T, 32, 2>, g, kThreads, stream, pdl, a);
-    case 5: return launch_one<T>(edge_group_kernel<T, 32, 4>, g, kThreads, stream, pdl, a);
-    case 6: return launch_one<T>(edge_group_kernel<T, 32, 8>, g, kThreads, stream, pdl, a);
+    case 0: return launch_group<T, 4, 1>(a, g, stream, pdl);
+    case 1: return launch_group<T, 8, 1>(a, g, stream, pdl);
+    case 2: return launch_group<T, 16, 1>(a, g, stream, pdl);
+    case 3: return launch_group<T, 32, 1>(a, g, stream, pdl);
+    case 4: return launch_group<T, 32, 2>(a, g, stream, pdl);
+    case 5: return launch_group<T, 32, 4>(a, g, stream, pdl);
+    case 6: return launch_group<T, 32, 8>(a, g, stream, pdl);
     case 7: return launch_one<T>(edge_block_kernel<T, 128, 4>, g, 128, stream, pdl, a);
     case 8: return launch_one<T>(edge_block_kernel<T, 256, 2>, g, 256, stream, pdl, a);
     case 9: return launch_one<T>(edge_block_kernel<T, 512, 2>, g, 512, stream, pdl, a);
@@ -1780,13 +1827,13 @@ int64_t edge_prefetch_distance(int cfg, int num_sms)
     int per_sm = 0;
     cudaError_t e = cudaSuccess;
     switch (cfg) {
-    case 0: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_group_kernel<T, 4, 1>, kThreads, 0); break;
-    case 1: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_group_kernel<T, 8, 1>, kThreads, 0); break;
-    case 2: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_group_kernel<T, 16, 1>, kThreads, 0); break;
-    case 3: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_group_kernel<T, 32, 1>, kThreads, 0); break;
-    case 4: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_group_kernel<T, 32, 2>, kThreads, 0); break;
-    case 5: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_group_kernel<T, 32, 4>, kThreads, 0); break;
-    case 6: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_group_kernel<T, 32, 8>, kThreads, 0); break;
+    case 0: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_group_kernel<T, 4, 1, 1>, kThreads, 0); break;
+    case 1: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_group_kernel<T, 8, 1, 1>, kThreads, 0); break;
+    case 2: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_group_kernel<T, 16, 1, 1>, kThreads, 0); break;
+    case 3: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_group_kernel<T, 32, 1, 1>, kThreads, 0); break;
+    case 4: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_group_kernel<T, 32, 1, 2>, kThreads, 0); break;
+    case 5: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_group_kernel<T, 32, 1, 4>, kThreads, 0); break;
+    case 6: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_group_kernel<T, 32, 1, 8>, kThreads, 0); break;
     case 7: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_block_kernel<T, 128, 4>, 128, 0); break;
     case 8: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_block_kernel<T, 256, 2>, 256, 0); break;
     case 9: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, edge_block_kernel<T, 512, 2>, 512, 0); break;
@@ -1836,12 +1883,12 @@ cudaError_t launch_convert_f32_to_f64(const float* a, double* b, int64_t count, 
 
 template int edge_config<float>(int);
 template int edge_config<double>(int);
-template int edge_grid<float>(int, int64_t, int);
-template int64_t edge_parts<float>(int, int);
+template int edge_grid<float>(int, int64_t, int, int);
+template int64_t edge_parts<float>(int, int, int);
 template int edge_capacity<float>(int);
 template int edge_capacity<double>(int);
-template int64_t edge_parts<double>(int, int);
-template int edge_grid<double>(int, int64_t, int);
+template int64_t edge_parts<double>(int, int, int);
+template int edge_grid<double>(int, int64_t, int, int);
 template cudaError_t launch_excess<float>(const SweepArgs<float>&, cudaStream_t, bool);
 template cudaError_t launch_excess<double>(const SweepArgs<double>&, cudaStream_t, bool);
 template cudaError_t launch_edge<float>(const SweepArgs<float>&, int, cudaStream_t, bool);

@@ -158,6 +158,23 @@ __device__ __forceinline__ void bulk_g2s_hint(void* dst, const void* src, uint32
         : "memory");
 }
 
+// x > w for w >= 0 (not -0), and the smaller of two positive values.  The FP64
+// pipe, two operations per clock and SM, also runs FP64 comparisons: those of
+// FP64 values are made on their bit patterns, which order as signed integers
+// where one side is not negative.  NaN exceeds nothing, as in a comparison of
+// floats; +inf does.
+__device__ __forceinline__ bool exceeds(float x, float w) { return x > w; }
+__device__ __forceinline__ bool exceeds(double x, double w)
+{
+    const long long b = __double_as_longlong(x);
+    return b > __double_as_longlong(w) && b <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ float min_pos(float x, float y) { return x < y ? x : y; }
+__device__ __forceinline__ double min_pos(double x, double y)
+{
+    return __double_as_longlong(x) < __double_as_longlong(y) ? x : y;
+}
+
 // Sum over the G lanes of an aligned lane group (xor offsets below G stay
 // inside the group).  Every lane of the warp must call it.  IEEE addition is
 // commutative, so every lane of the group ends with the same value.
@@ -169,13 +186,14 @@ __device__ __forceinline__ X group_sum(X x)
     return x;
 }
 
+// of values that are not negative
 template <typename X>
 __device__ __forceinline__ X warp_max(X x)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const X y = __shfl_xor_sync(kFull, x, o);
-        x = y > x ? y : x;
+        x = exceeds(y, x) ? y : x;
     }
     return x;
 }
@@ -196,8 +214,7 @@ __device__ __forceinline__ void warp_sum_count_min(T& s, int& n, T& mn)
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             n += __shfl_xor_sync(kFull, n, o);
-            const T y = __shfl_xor_sync(kFull, mn, o);
-            mn = y < mn ? y : mn;
+            mn = min_pos(__shfl_xor_sync(kFull, mn, o), mn);
         }
     }
 }
