@@ -128,7 +128,7 @@ typedef struct {
     int32_t edge_variant;
     /* Kernel form of the excess pass (eq. (2), (3); a tuning choice, every form
      * gives bit-identical heights).  -1 (default): the library's choice
-     * (form 2 where it can be resident, else 0).
+     * (2 for long rows and many vertices, else 0).
      * 0: one thread per (vertex, 4 values) gathers the incident flow rows.
      * 1..5: per block, one warp brings the incident row segments of a
      * contiguous range of vertices into shared memory with bulk copies

@@ -993,15 +993,30 @@ bool persistent_ok(const pdr_ctx* ctx, int p)
     return ctx->opt.use_graph == 2 && !is_gd(ctx->opt) && ctx->pgrid[p] >= 2;
 }
 
-// Excess kernel form from the options: -1 takes the default, 0..3 that
+// Excess kernel form from the options: -1 takes the default, 0..5 that
 // form; a bulk-copy form that cannot be resident on this device is refused.
-// The default is bulk-copy form 2 (two stages of eight row segments, six
-// blocks per SM on GB300), the fastest form measured on the grid, k-NN and
-// random-digraph workloads; the gathers where it cannot be resident.
+// The default is the gathers, whose index loads do not wait for the previous
+// kernel, or bulk-copy form 2 (two stages of eight row segments, six blocks per
+// SM on GB300), which keeps more bytes in flight:
+// - FP32: bulk copies once a row fills its 2 KB segment and there are vertices
+//   for the blocks.  Sweep, us, gathers / bulk (n, m, K): 500, 3000, 100: 8.0 /
+//   9.6; 20,000, 100,000, 40: 38 / 60; 20,000, 100,000, 200: 77 / 92; 10,000,
+//   39,600, 300: 42 / 47; 8000, 40,000, 400: 52.7 / 52.9; 8000, 40,000, 500:
+//   60.9 / 56.9; 10,000, 39,600, 600: 74 / 64; 625, 2400, 4000: 38.7 / 44.3;
+//   20,000, 100,000, 2000: 699 / 651.
+// - FP64, bound by its pipe: bulk copies once the gathers need several rounds of
+//   their resident threads.  500, 3000, 100: 20.2 / 23.7; 900, 3480, 500: 58.9 /
+//   67.5; 2000, 8000, 200: 67.2 / 68.6; 10,000, 40,000, 200: 280 / 266; 20,000,
+//   60,000, 50: 143 / 133.
 constexpr int kDefaultExcessForm = 2;
+constexpr int kBulkRowBytes = 1800, kBulkVerticesPerSm = 5, kBulkRounds = 4;
 pdr_status select_excess_form(pdr_ctx* ctx, const pdr_options& o)
 {
-    const int v = o.excess_variant >= 0 ? o.excess_variant : (ctx->xgrid[kDefaultExcessForm] > 0 ? kDefaultExcessForm : 0);
+    const bool bulk = o.precision == PDR_PREC_FP64
+                          ? (int64_t)ctx->n * (ctx->Kp / 2) > (int64_t)kBulkRounds * ctx->grid_v[1] * kGatherThreads
+                          : ctx->Kp * 4 >= kBulkRowBytes && ctx->n >= kBulkVerticesPerSm * ctx->num_sms;
+    const int v = o.excess_variant >= 0 ? o.excess_variant
+                  : bulk && ctx->xgrid[kDefaultExcessForm] > 0 ? kDefaultExcessForm : 0;
     if (v > 0 && ctx->xgrid[v] <= 0)
         return ctx->fail(PDR_ERR_INVALID_ARG, "excess_variant " + std::to_string(v) + " cannot run on this device");
     ctx->xform = v;
@@ -1499,9 +1514,9 @@ pdr_status pdr_create(int32_t n, int64_t m, const int64_t* row_ptr, const int32_
         const pdr_status vs = select_edge_variants(ctx, o);
         if (vs != PDR_OK) return give_up(vs);
     }
-    ctx->grid_v[0] = excess_grid(n, Kp, 4, ctx->num_sms, excess_resident_blocks<float>());
-    ctx->grid_v[1] = excess_grid(n, Kp, 2, ctx->num_sms, excess_resident_blocks<double>());
-    ctx->r_grid_v = excess_grid(n, Kp, 1, ctx->num_sms, 8);
+    ctx->grid_v[0] = excess_grid(n, Kp, 4, ctx->num_sms, excess_resident_blocks<float>(), kGatherThreads);
+    ctx->grid_v[1] = excess_grid(n, Kp, 2, ctx->num_sms, excess_resident_blocks<double>(), kGatherThreads);
+    ctx->r_grid_v = excess_grid(n, Kp, 1, ctx->num_sms, 8, kThreads);
     for (int f = 1; f < kExcessForms; ++f) {
         const int r32 = excess_bulk_resident_blocks<float>(f), r64 = excess_bulk_resident_blocks<double>(f);
         const int64_t r = r32 < r64 ? r32 : r64;
@@ -1683,7 +1698,7 @@ pdr_status pdr_set_options(pdr_ctx* ctx, const pdr_options* opt)
                             o.beta_min != ctx->opt.beta_min || o.beta_max != ctx->opt.beta_max ||
                             o.alpha_inc != ctx->opt.alpha_inc || o.alpha_dec != ctx->opt.alpha_dec ||
                             o.gamma != ctx->opt.gamma;
-    if (o.excess_variant != ctx->opt.excess_variant) {
+    if (o.excess_variant != ctx->opt.excess_variant || o.precision != ctx->opt.precision) {
         const pdr_status xs = select_excess_form(ctx, o);
         if (xs != PDR_OK) return xs;
         destroy_graphs(ctx);

@@ -22,6 +22,7 @@
 namespace pdr {
 
 constexpr int kThreads = 256;  // block size of every sweep kernel
+constexpr int kGatherThreads = 64;  // gather form of the excess pass: small blocks spread a few hundred vertices over the SMs
 constexpr int kShareThreads = 64;  // block size of the lane-group forms with several shares per lane
 constexpr int kExcessForms = 6;     // excess kernel forms: 0 gathers, 1..5 bulk copies
 // Resident blocks per SM that the block forms of the edge kernels are
@@ -199,7 +200,7 @@ template <typename T>
 int64_t edge_prefetch_distance(int cfg, int num_sms);  // edges solved by one wave of resident blocks
 bool edge_config_pipelined(int cfg);
 bool edge_config_staged(int cfg);       // the bulk-copy staged block forms
-int excess_grid(int32_t n, int Kp, int vec, int num_sms, int resident_blocks);
+int excess_grid(int32_t n, int Kp, int vec, int num_sms, int resident_blocks, int threads);
 // Persistent sweep kernel (sweep.cu): excess and edge QP of every sweep in one
 // cooperative launch, separated by grid barriers; runs up to `sweeps` sweeps
 // of Alg. 1 or until the stop rules fire.  Only the lane-group variants.

@@ -38,14 +38,96 @@ __global__ void __launch_bounds__(kThreads) finalize_kernel(SweepArgs<T> a)
 
 // ------------------------------------------------------------------ excess and heights
 
+// Block `block`'s slice of the edge kernel's psi partials: this thread's first
+// one, loaded before the rows arrive.
 template <typename T>
-__device__ __forceinline__ void excess_tail(const SweepArgs<T>& a, int block, int nblocks,
-                                            typename Acc<T>::V zacc, T cons);
+struct TailPart {
+    int64_t at, hi;
+    typename Acc<T>::V z = Acc<T>::zero();
+    T cap = T(0);
+    __device__ __forceinline__ TailPart(const SweepArgs<T>& a, int block, int nblocks)
+    {
+        at = (int64_t)block * a.n_psi / nblocks + threadIdx.x;
+        hi = (int64_t)(block + 1) * a.n_psi / nblocks;
+        load(a);
+    }
+    __device__ __forceinline__ void load(const SweepArgs<T>& a)
+    {
+        if (at >= hi) return;
+        z = Acc<T>::load(reinterpret_cast<const typename Acc<T>::S*>(a.part_psi) + at);
+        cap = __ldcg(a.part_cap + at);
+    }
+};
+
+template <typename T>
+__device__ __forceinline__ void excess_tail(const SweepArgs<T>& a, int block, int nblocks, typename Acc<T>::V zacc, T cons,
+                                            TailPart<T> part);
+
+// The gather form: one thread per (vertex, vector).  Its time on a small
+// instance is a chain of dependent loads (list bounds -> list -> rows), so the
+// first item's lists, which do not change during a solve, are read before the
+// wait for the previous kernel, and its rows together with the stop flag.
+constexpr int kGather = 8;            // rows in flight per thread
+constexpr int kGatherPersistent = 4;  // in the persistent kernel, capped at 64 registers
+template <int W>
+struct ExcessItem {
+    uint32_t i, v;             // vertex, vector of its row
+    int64_t q0, q1;            // its incidence list
+    int32_t ev[W];             // the list's first entries
+};
+
+// commodity endpoints of vector v (of four or two values)
+__device__ __forceinline__ void load_ends(const int32_t* p, uint32_t v, int (&x)[4])
+{
+    const int4 y = reinterpret_cast<const int4*>(p)[v];
+    x[0] = y.x, x[1] = y.y, x[2] = y.z, x[3] = y.w;
+}
+__device__ __forceinline__ void load_ends(const int32_t* p, uint32_t v, int (&x)[2])
+{
+    const int2 y = reinterpret_cast<const int2*>(p)[v];
+    x[0] = y.x, x[1] = y.y;
+}
+template <int W>
+__device__ __forceinline__ void load_list(const int32_t* inc, int64_t q0, int64_t q1, int32_t (&ev)[W])
+{
+#pragma unroll
+    for (int u = 0; u < W; ++u) ev[u] = q0 + u < q1 ? inc[q0 + u] : 0;
+}
+
+template <typename T, int W>
+__device__ __forceinline__ void load_item(const SweepArgs<T>& a, uint64_t idx, uint64_t total, uint32_t vpr,
+                                          ExcessItem<W>& it)
+{
+    if (total <= 0xffffffffull) {
+        it.i = (uint32_t)idx / vpr;
+        it.v = (uint32_t)idx - it.i * vpr;
+    } else {
+        it.i = (uint32_t)(idx / vpr);
+        it.v = (uint32_t)(idx - (uint64_t)it.i * vpr);
+    }
+    it.q0 = a.inc_ptr[it.i];
+    it.q1 = a.inc_ptr[it.i + 1];
+    load_list(a.inc, it.q0, it.q1, it.ev);
+}
+
+// vector v of the rows ev[u] of list positions q0 + u below q1, zeros past it
+template <typename T, typename VT, int W>
+__device__ __forceinline__ void load_rows(const SweepArgs<T>& a, const int32_t (&ev)[W], int64_t q0, int64_t q1,
+                                          uint32_t v, VT (&x)[W])
+{
+#pragma unroll
+    for (int u = 0; u < W; ++u) {
+        x[u] = VT{};
+        if (q0 + u < q1) x[u] = reinterpret_cast<const VT*>(a.f + (int64_t)(ev[u] >= 0 ? ev[u] : ~ev[u]) * a.Kp)[v];
+    }
+}
 
 // Body of one excess pass run by block `block` of `nblocks` (the standalone
-// kernel passes its own grid; the persistent kernel its whole grid).
-template <typename T>
-__device__ __forceinline__ void excess_body(const SweepArgs<T>& a, int block, int nblocks)
+// kernel passes its own grid; the persistent kernel its whole grid), after
+// `it` and `x` were loaded for the thread's first item.
+template <typename T, int W>
+__device__ __forceinline__ void excess_body(const SweepArgs<T>& a, int block, int nblocks, ExcessItem<W>& it,
+                                            typename VecOf<T>::type (&x)[W])
 {
     using VT = typename VecOf<T>::type;
     using A = Acc<T>;
@@ -57,70 +139,45 @@ __device__ __forceinline__ void excess_body(const SweepArgs<T>& a, int block, in
     const uint64_t stride = (uint64_t)nblocks * blockDim.x;
     typename A::V zacc = A::zero();
     T cons = T(0);
-    for (uint64_t idx = (uint64_t)block * blockDim.x + threadIdx.x; idx < total; idx += stride) {
-        uint32_t i, v;
-        if (total <= 0xffffffffull) {
-            i = (uint32_t)idx / vpr;
-            v = (uint32_t)idx - i * vpr;
-        } else {
-            i = (uint32_t)(idx / vpr);
-            v = (uint32_t)(idx - (uint64_t)i * vpr);
-        }
-        T acc[N];
+    const TailPart<T> first(a, block, nblocks);
+    for (uint64_t idx = (uint64_t)block * blockDim.x + threadIdx.x; idx < total;) {
+        const uint32_t i = it.i, v = it.v;
+        const int64_t q1 = it.q1, count = q1 - it.q0;
+        // the commodities of the vector and the vertex's scale, on their way with the rows
+        int sk[N], tk[N];
+        T dk[N], idk[N], acc[N];
+        load_ends(a.s, v, sk);
+        load_ends(a.t, v, tk);
+        unpack(reinterpret_cast<const VT*>(a.dem)[v], dk);
+        unpack(reinterpret_cast<const VT*>(a.inv_dem)[v], idk);
+        const T idg = a.inv_deg[i];
 #pragma unroll
         for (int j = 0; j < N; ++j) acc[j] = T(0);
         // incidence list: in-edges e (added), then out-edges ~e (subtracted),
-        // up to eight rows in flight; the additions keep list order
-        const int64_t q0 = a.inc_ptr[i], q1 = a.inc_ptr[i + 1];
-        int64_t q = q0;
-        for (; q + 8 <= q1; q += 8) {
-            int32_t ev[8];
-            T x[8][N];
+        // in list order; the zeros past its end change nothing (acc is never -0)
+        for (int64_t q = it.q0;;) {
+            const int64_t next = q + W;
+            int32_t ev[W];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) ev[u] = a.inc[q + u];
+            for (int u = 0; u < W; ++u) ev[u] = it.ev[u];
+            if (next < q1) load_list(a.inc, next, q1, it.ev);
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int64_t e = ev[u] >= 0 ? ev[u] : ~ev[u];
-                unpack(reinterpret_cast<const VT*>(a.f + e * a.Kp)[v], x[u]);
+            for (int u = 0; u < W; ++u) {
+                T xu[N];
+                unpack(x[u], xu);
+#pragma unroll
+                for (int j = 0; j < N; ++j) acc[j] += ev[u] >= 0 ? xu[j] : -xu[j];
             }
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-#pragma unroll
-                for (int j = 0; j < N; ++j) acc[j] += ev[u] >= 0 ? x[u][j] : -x[u][j];
+            if (next >= q1) break;
+            q = next;
+            load_rows<T, VT>(a, it.ev, q, q1, v, x);
         }
-        if (q + 4 <= q1) {
-            int32_t ev[4];
-            T x[4][N];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) ev[u] = a.inc[q + u];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int64_t e = ev[u] >= 0 ? ev[u] : ~ev[u];
-                unpack(reinterpret_cast<const VT*>(a.f + e * a.Kp)[v], x[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int j = 0; j < N; ++j) acc[j] += ev[u] >= 0 ? x[u][j] : -x[u][j];
-            q += 4;
-        }
-        for (; q < q1; ++q) {
-            const int32_t ev = a.inc[q];
-            const int64_t e = ev >= 0 ? ev : ~ev;
-            T x[N];
-            unpack(reinterpret_cast<const VT*>(a.f + e * a.Kp)[v], x);
-#pragma unroll
-            for (int j = 0; j < N; ++j) acc[j] += ev >= 0 ? x[j] : -x[j];
-        }
-        const int k0 = (int)v * N;
 #pragma unroll
         for (int j = 0; j < N; ++j) {
-            const int k = k0 + j;
-            if (a.s[k] == (int)i) acc[j] += a.dem[k];
-            else if (a.t[k] == (int)i) acc[j] -= a.dem[k];
+            if (sk[j] == (int)i) acc[j] += dk[j];
+            else if (tk[j] == (int)i) acc[j] -= dk[j];
         }
-        const T dgt = T((int)(q1 - q0));  // delta_i < 2^31: a 32-bit conversion
-        const T idg = a.inv_deg[i];
+        const T dgt = T((int)count);  // delta_i < 2^31: a 32-bit conversion
         T hv[N];
 #pragma unroll
         for (int j = 0; j < N; ++j) hv[j] = acc[j] * idg;
@@ -130,33 +187,31 @@ __device__ __forceinline__ void excess_body(const SweepArgs<T>& a, int block, in
 #pragma unroll
         for (int j = 0; j < N; ++j) {
             zt += dgt * hv[j] * hv[j];
-            const T r = fabs(acc[j]) * a.inv_dem[k0 + j];
+            const T r = fabs(acc[j]) * idk[j];
             cons = exceeds(r, cons) ? r : cons;
         }
         zacc = A::add(zacc, zt);
+        idx += stride;
+        if (idx < total) {
+            load_item(a, idx, total, vpr, it);
+            load_rows<T, VT>(a, it.ev, it.q0, it.q1, it.v, x);
+        }
     }
-    excess_tail<T>(a, block, nblocks, zacc, cons);
+    excess_tail<T>(a, block, nblocks, zacc, cons, first);
 }
 
 // End of an excess pass in every block: add this block's fixed slice of the
 // edge kernel's psi partials and write the block's three partials.  Every
 // thread of the block calls it.
 template <typename T>
-__device__ __forceinline__ void excess_tail(const SweepArgs<T>& a, int block, int nblocks,
-                                            typename Acc<T>::V zacc, T cons)
+__device__ __forceinline__ void excess_tail(const SweepArgs<T>& a, int block, int nblocks, typename Acc<T>::V zacc, T cons,
+                                            TailPart<T> part)
 {
     using A = Acc<T>;
     T capb = T(0);
-    {
-        // the block's slice [lo, hi) of the edge partials
-        const int64_t lo = (int64_t)block * a.n_psi / nblocks;
-        const int64_t hi = (int64_t)(block + 1) * a.n_psi / nblocks;
-        const typename A::S* pp = reinterpret_cast<const typename A::S*>(a.part_psi);
-        for (int64_t b = lo + threadIdx.x; b < hi; b += blockDim.x) {
-            zacc = A::add(zacc, A::load(pp + b));
-            const T c = __ldcg(a.part_cap + b);
-            capb = c > capb ? c : capb;
-        }
+    for (; part.at < part.hi; part.at += blockDim.x, part.load(a)) {
+        zacc = A::add(zacc, part.z);
+        capb = part.cap > capb ? part.cap : capb;
     }
     block_acc_max2<T>(zacc, cons, capb);
     if (threadIdx.x == 0) {
@@ -166,14 +221,21 @@ __device__ __forceinline__ void excess_tail(const SweepArgs<T>& a, int block, in
     }
 }
 
+// (Ten blocks per SM: a cap of 96 registers, which the eight rows in flight need.)
 template <typename T>
-__global__ void __launch_bounds__(kThreads) excess_kernel(SweepArgs<T> a)
+__global__ void __launch_bounds__(kGatherThreads, 10) excess_kernel(SweepArgs<T> a)
 {
+    using VT = typename VecOf<T>::type;
+    const uint32_t vpr = (uint32_t)(a.Kp / VecOf<T>::N);
+    const uint64_t total = (uint64_t)a.n * vpr, idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    ExcessItem<kGather> it{};
+    VT x[kGather];
+    if (idx < total) load_item(a, idx, total, vpr, it);
     pdl_wait();     // the previous sweep's edge kernel has finished (no-op without PDL)
     pdl_trigger();  // one wave: the edge kernel's blocks may queue behind this one's
-    volatile DevState* vst = a.st;
+    if (idx < total) load_rows<T, VT>(a, it.ev, it.q0, it.q1, it.v, x);
     if (sweep_stopped(a)) return;  // an earlier sweep of this solve stopped
-    excess_body<T>(a, blockIdx.x, gridDim.x);
+    excess_body<T>(a, blockIdx.x, gridDim.x, it, x);
 }
 
 // ------------------------------------------------------------------ excess by bulk copies
@@ -415,7 +477,7 @@ __global__ void __launch_bounds__(C + 32) excess_bulk_kernel(SweepArgs<T> a)
                     unpack(rows[r * (kXSegBytes / 16)], x);
                     const bool add = (d.sign >> r) & 1u;
 #pragma unroll
-                    for (int q = 0; q < N; ++q) acc[q] = add ? acc[q] + x[q] : acc[q] - x[q];
+                    for (int q = 0; q < N; ++q) acc[q] += add ? x[q] : -x[q];
                 }
             }
             __syncwarp();
@@ -450,7 +512,7 @@ __global__ void __launch_bounds__(C + 32) excess_bulk_kernel(SweepArgs<T> a)
             stop_from_kernel(a);
         }
     }
-    excess_tail<T>(a, block, gridDim.x, zacc, cons);
+    excess_tail<T>(a, block, gridDim.x, zacc, cons, TailPart<T>(a, block, gridDim.x));
 }
 
 // xv_start[b] = the first vertex i with inc_ptr[i] + 2 i >= b * (inc_ptr[n] + 2 n) / grid
@@ -1181,7 +1243,15 @@ __global__ void __launch_bounds__(kThreads, (V <= 4 ? 4 : 3))
             b.theta_in = a.theta;
             b.theta = const_cast<T*>(a.theta_in);
         }
-        excess_body<T>(b, blockIdx.x, gridDim.x);
+        const uint32_t vpr = (uint32_t)(b.Kp / VecOf<T>::N);
+        const uint64_t total = (uint64_t)b.n * vpr, idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+        ExcessItem<kGatherPersistent> it{};
+        typename VecOf<T>::type x[kGatherPersistent];
+        if (idx < total) {
+            load_item(b, idx, total, vpr, it);
+            load_rows<T, typename VecOf<T>::type>(b, it.ev, it.q0, it.q1, it.v, x);
+        }
+        excess_body<T>(b, blockIdx.x, gridDim.x, it, x);
         if (!grid_sync(bar, a.barrier_ns, hold)) return;
         if ((int)blockIdx.x == nb) reduce_and_finalize(b);
         else edge_group_body<T, G, 1, V, true>(b, blockIdx.x, nb);
@@ -1522,10 +1592,10 @@ int64_t edge_parts(int cfg, int grid, int shares)
 
 // One wave of resident blocks (or fewer if the rows are fewer): the grid-
 // stride loop then spreads the rows evenly and leaves no partial last wave.
-int excess_grid(int32_t n, int Kp, int vec, int num_sms, int resident_blocks)
+int excess_grid(int32_t n, int Kp, int vec, int num_sms, int resident_blocks, int threads)
 {
     const int64_t total = (int64_t)n * (Kp / vec);
-    int64_t want = (total + kThreads - 1) / kThreads;
+    int64_t want = (total + threads - 1) / threads;
     const int64_t cap = (int64_t)num_sms * (resident_blocks > 0 ? resident_blocks : 4);
     int64_t g = want < cap ? want : cap;
     return (int)(g < 1 ? 1 : g);
@@ -1535,7 +1605,7 @@ template <typename T>
 int excess_resident_blocks()
 {
     int blocks = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, excess_kernel<T>, kThreads, 0) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, excess_kernel<T>, kGatherThreads, 0) != cudaSuccess) {
         cudaGetLastError();
         return 4;
     }
@@ -1543,31 +1613,6 @@ int excess_resident_blocks()
 }
 template int excess_resident_blocks<float>();
 template int excess_resident_blocks<double>();
-
-// A launch with or without programmatic dependent launch (PDL): with it,
-// the kernel may be scheduled while the previous kernel on the stream (or
-// in the graph) is still running; its griddepcontrol.wait then holds it
-// until that kernel has finished and its writes are visible.
-template <typename T>
-cudaError_t launch_one(void (*kernel)(SweepArgs<T>), int grid, int block, cudaStream_t stream, bool pdl,
-                       const SweepArgs<T>& a, size_t smem = 0)
-{
-    if (!pdl) {
-        kernel<<<grid, block, smem, stream>>>(a);
-        return cudaGetLastError();
-    }
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, a);
-}
 
 template <typename T, int S, int R, int C>
 cudaError_t launch_bulk(const SweepArgs<T>& a, cudaStream_t stream, bool pdl)
@@ -1586,7 +1631,7 @@ cudaError_t launch_excess(const SweepArgs<T>& a, cudaStream_t stream, bool pdl)
     case 3: return launch_bulk<T, 4, 4, 128>(a, stream, pdl);
     case 4: return launch_bulk<T, 2, 8, 32>(a, stream, pdl);
     case 5: return launch_bulk<T, 4, 8, 32>(a, stream, pdl);
-    default: return launch_one<T>(excess_kernel<T>, a.grid_v, kThreads, stream, pdl, a);
+    default: return launch_one<T>(excess_kernel<T>, a.grid_v, kGatherThreads, stream, pdl, a);
     }
 }
 

@@ -47,6 +47,31 @@ __device__ __forceinline__ double2 pack4(const double* x) { return make_double2(
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// A launch with or without programmatic dependent launch (PDL): with it,
+// the kernel may be scheduled while the previous kernel on the stream (or
+// in the graph) is still running; its griddepcontrol.wait then holds it
+// until that kernel has finished and its writes are visible.
+template <typename T>
+cudaError_t launch_one(void (*kernel)(SweepArgs<T>), int grid, int block, cudaStream_t stream, bool pdl,
+                       const SweepArgs<T>& a, size_t smem = 0)
+{
+    if (!pdl) {
+        kernel<<<grid, block, smem, stream>>>(a);
+        return cudaGetLastError();
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
 // L2 prefetch of the `bytes` bytes at p, one 128-byte line per thread and
 // round (thread `tid` of `nthreads`).  Only addresses inside the array are
 // passed; a prefetch never blocks the thread.
