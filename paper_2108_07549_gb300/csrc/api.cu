@@ -408,7 +408,7 @@ template <typename T>
 cudaError_t launch_update(pdr_ctx* ctx, const SweepArgs<T>& a, cudaStream_t stream, bool pdl = false)
 {
     const int cfg = ctx->cfg[Prec<T>::id];
-    return is_gd(ctx->opt) ? launch_gd<T>(a, cfg, stream) : launch_edge<T>(a, cfg, stream, pdl);
+    return is_gd(ctx->opt) ? launch_gd<T>(a, cfg, stream, pdl) : launch_edge<T>(a, cfg, stream, pdl);
 }
 
 // Velocity buffers of the working precision (Alg. 4 only).
@@ -766,7 +766,7 @@ pdr_status read_state(pdr_ctx* ctx)
 }
 
 // The sweep loop as one graph: a conditional WHILE node whose body holds
-// kUnroll sweeps (excess kernel, then update kernel).  For Alg. 1 the body's
+// kUnroll sweeps (excess kernel, then update kernel).  The body's
 // kernels are captured with programmatic dependent launch (each may be
 // scheduled while its predecessor drains); if the runtime refuses that, the
 // body is captured again with plain launches.
@@ -821,7 +821,7 @@ pdr_status build_graph(pdr_ctx* ctx)
     const int p = Prec<T>::id;
     ctx->graph_tried[p] = true;
     ctx->graph_ok[p] = false;
-    if (!is_gd(ctx->opt) && try_build_graph<T>(ctx, true)) return PDR_OK;
+    if (try_build_graph<T>(ctx, true)) return PDR_OK;
     try_build_graph<T>(ctx, false);
     return PDR_OK;  // if both failed, the host loop takes over
 }

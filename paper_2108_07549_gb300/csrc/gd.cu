@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(kThreads) gd_group_kernel(SweepArgs<T> a)
     constexpr int N = VecOf<T>::N;
     constexpr int GPW = 32 / G;
     volatile DevState* vst = a.st;
+    pdl_wait();  // the excess kernel has finished (no-op without PDL)
     const int skip = update_skipped(a);
     if (skip == 1) return;              // an earlier sweep of this solve stopped
     if (blockIdx.x == gridDim.x - 1) {  // the decision block
@@ -167,10 +168,12 @@ __global__ void __launch_bounds__(B, gd_min_blocks(B, V)) gd_block_kernel(SweepA
     using VT = typename VecOf<T>::type;
     using A = Acc<T>;
     constexpr int N = VecOf<T>::N;
+    constexpr bool kEarly = M && V <= 2 && sizeof(T) == 4;  // the velocities' loads start with the flows' (2627 -> 2590 us there)
     __shared__ T sa_buf[33];
     __shared__ int sb_buf[33];
     __shared__ T sc_buf[33];
     volatile DevState* vst = a.st;
+    pdl_wait();  // the excess kernel has finished (no-op without PDL)
     const int skip = update_skipped(a);
     if (skip == 1) return;  // an earlier sweep of this solve stopped
     if (blockIdx.x == gridDim.x - 1) {
@@ -191,10 +194,12 @@ __global__ void __launch_bounds__(B, gd_min_blocks(B, V)) gd_block_kernel(SweepA
         const VT* hj = reinterpret_cast<const VT*>(a.h + (int64_t)a.col[e] * a.Kp);
         const VT* frow = reinterpret_cast<const VT*>(a.f + row);
         T d[V][N];
+        T vin[kEarly ? V : 1][N];
         T fs = T(0);
 #pragma unroll
         for (int q = 0; q < V; ++q) {
             const int v = threadIdx.x + q * B;
+            if (kEarly && v < vpr) unpack(__ldg(reinterpret_cast<const VT*>(a.v_in + row) + v), vin[q]);
             if (v < vpr) {
                 T fx[N], ax[N], bx[N];
                 unpack(__ldg(frow + v), fx);
@@ -240,18 +245,18 @@ __global__ void __launch_bounds__(B, gd_min_blocks(B, V)) gd_block_kernel(SweepA
         for (int q = 0; q < V; ++q) {
             const int v = threadIdx.x + q * B;
             const bool live = v < vpr;
-            T fx[N], vin[N], o[N], vo[N];
+            T fx[N], o[N], vo[N];
             if (live) unpack(__ldg(frow + v), fx);
             else
 #pragma unroll
                 for (int j = 0; j < N; ++j) fx[j] = T(0);
-            if (M && live) unpack(__ldg(reinterpret_cast<const VT*>(a.v_in + row) + v), vin);
+            if (M && !kEarly && live) unpack(__ldg(reinterpret_cast<const VT*>(a.v_in + row) + v), vin[0]);
 #pragma unroll
             for (int j = 0; j < N; ++j) {
                 const T st = beta * (d[q][j] - psi);
                 const T df = st > -fx[j] ? st : -fx[j];
                 if constexpr (M) {
-                    const T vv = live ? vin[j] : T(0);
+                    const T vv = live ? vin[kEarly ? q : 0][j] : T(0);
                     vo[j] = accept ? a.gamma * vv + df : vv;
                     const T x = fx[j] + vo[j];
                     o[j] = accept ? (x > T(0) ? x : T(0)) : fx[j];
@@ -290,29 +295,28 @@ __global__ void __launch_bounds__(B, gd_min_blocks(B, V)) gd_block_kernel(SweepA
 // variant runs the plain form of the same capacity (the kernels stride over
 // the edges, so any grid works).
 template <typename T, bool M>
-cudaError_t launch_gd_m(const SweepArgs<T>& a, int cfg, cudaStream_t stream)
+cudaError_t launch_gd_m(const SweepArgs<T>& a, int cfg, cudaStream_t stream, bool pdl)
 {
     const int g = a.grid_e + 1;
     switch (edge_plain_config(cfg)) {
-    case 0: gd_group_kernel<T, 4, 1, M><<<g, kThreads, 0, stream>>>(a); break;
-    case 1: gd_group_kernel<T, 8, 1, M><<<g, kThreads, 0, stream>>>(a); break;
-    case 2: gd_group_kernel<T, 16, 1, M><<<g, kThreads, 0, stream>>>(a); break;
-    case 3: gd_group_kernel<T, 32, 1, M><<<g, kThreads, 0, stream>>>(a); break;
-    case 4: gd_group_kernel<T, 32, 2, M><<<g, kThreads, 0, stream>>>(a); break;
-    case 5: gd_group_kernel<T, 32, 4, M><<<g, kThreads, 0, stream>>>(a); break;
-    case 6: gd_group_kernel<T, 32, 8, M><<<g, kThreads, 0, stream>>>(a); break;
-    case 7: gd_block_kernel<T, 128, 4, M><<<g, 128, 0, stream>>>(a); break;
-    case 8: gd_block_kernel<T, 256, 2, M><<<g, 256, 0, stream>>>(a); break;
-    case 9: gd_block_kernel<T, 512, 2, M><<<g, 512, 0, stream>>>(a); break;
-    case 10: gd_block_kernel<T, 512, 3, M><<<g, 512, 0, stream>>>(a); break;
-    case 11: gd_block_kernel<T, 512, 4, M><<<g, 512, 0, stream>>>(a); break;
-    case 12: gd_block_kernel<T, 512, 5, M><<<g, 512, 0, stream>>>(a); break;
-    case 13: gd_block_kernel<T, 256, 10, M><<<g, 256, 0, stream>>>(a); break;
-    case 14: gd_block_kernel<T, 512, 8, M><<<g, 512, 0, stream>>>(a); break;
-    case 15: gd_block_kernel<T, 1024, 8, M><<<g, 1024, 0, stream>>>(a); break;
+    case 0: return launch_one<T>(gd_group_kernel<T, 4, 1, M>, g, kThreads, stream, pdl, a);
+    case 1: return launch_one<T>(gd_group_kernel<T, 8, 1, M>, g, kThreads, stream, pdl, a);
+    case 2: return launch_one<T>(gd_group_kernel<T, 16, 1, M>, g, kThreads, stream, pdl, a);
+    case 3: return launch_one<T>(gd_group_kernel<T, 32, 1, M>, g, kThreads, stream, pdl, a);
+    case 4: return launch_one<T>(gd_group_kernel<T, 32, 2, M>, g, kThreads, stream, pdl, a);
+    case 5: return launch_one<T>(gd_group_kernel<T, 32, 4, M>, g, kThreads, stream, pdl, a);
+    case 6: return launch_one<T>(gd_group_kernel<T, 32, 8, M>, g, kThreads, stream, pdl, a);
+    case 7: return launch_one<T>(gd_block_kernel<T, 128, 4, M>, g, 128, stream, pdl, a);
+    case 8: return launch_one<T>(gd_block_kernel<T, 256, 2, M>, g, 256, stream, pdl, a);
+    case 9: return launch_one<T>(gd_block_kernel<T, 512, 2, M>, g, 512, stream, pdl, a);
+    case 10: return launch_one<T>(gd_block_kernel<T, 512, 3, M>, g, 512, stream, pdl, a);
+    case 11: return launch_one<T>(gd_block_kernel<T, 512, 4, M>, g, 512, stream, pdl, a);
+    case 12: return launch_one<T>(gd_block_kernel<T, 512, 5, M>, g, 512, stream, pdl, a);
+    case 13: return launch_one<T>(gd_block_kernel<T, 256, 10, M>, g, 256, stream, pdl, a);
+    case 14: return launch_one<T>(gd_block_kernel<T, 512, 8, M>, g, 512, stream, pdl, a);
+    case 15: return launch_one<T>(gd_block_kernel<T, 1024, 8, M>, g, 1024, stream, pdl, a);
     default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 // Same variant table as the edge-QP kernels (sweep.cu: kCfg); a pipelined
@@ -320,12 +324,12 @@ cudaError_t launch_gd_m(const SweepArgs<T>& a, int cfg, cudaStream_t stream)
 // the edges, so any grid works).  Alg. 3 and Alg. 4 are compiled apart, so
 // that Alg. 3 carries no velocity registers.
 template <typename T>
-cudaError_t launch_gd(const SweepArgs<T>& a, int cfg, cudaStream_t stream)
+cudaError_t launch_gd(const SweepArgs<T>& a, int cfg, cudaStream_t stream, bool pdl)
 {
-    return a.momentum ? launch_gd_m<T, true>(a, cfg, stream) : launch_gd_m<T, false>(a, cfg, stream);
+    return a.momentum ? launch_gd_m<T, true>(a, cfg, stream, pdl) : launch_gd_m<T, false>(a, cfg, stream, pdl);
 }
 
-template cudaError_t launch_gd<float>(const SweepArgs<float>&, int, cudaStream_t);
-template cudaError_t launch_gd<double>(const SweepArgs<double>&, int, cudaStream_t);
+template cudaError_t launch_gd<float>(const SweepArgs<float>&, int, cudaStream_t, bool);
+template cudaError_t launch_gd<double>(const SweepArgs<double>&, int, cudaStream_t, bool);
 
 }  // namespace pdr
