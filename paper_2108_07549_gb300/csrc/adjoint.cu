@@ -169,6 +169,77 @@ __global__ void __launch_bounds__(kThreads) edge_backward_kernel(SweepArgs<T> a,
     }
 }
 
+// Warp per edge for rows of up to 32 V vectors, the row's cotangent and its
+// active-set bits in registers between the sum over the row and the write, so
+// that every input row is read once and no block barrier stands between them.
+// Bound by L2 and memory (six rows in, one out).  n 5000, m 25,000, K 600: 57 us
+// in the block form of 128 threads (two barriers per edge), 46 us here.
+template <typename T, int V, bool FUSED>
+__global__ void __launch_bounds__(kThreads, V <= 4 ? 4 : 3)
+    edge_backward_warp_kernel(SweepArgs<T> a, const T* __restrict__ theta, const T* __restrict__ fbar, T* cbar,
+                              const T* __restrict__ Dbar, double* __restrict__ ubar)
+{
+    using VT = typename VecOf<T>::type;
+    constexpr int N = VecOf<T>::N;
+    static_assert(V * N <= 32, "one bit per held value");
+    const int lane = threadIdx.x & 31;
+    const int vpr = a.Kp / N;
+    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t e = w0; e < a.m; e += nw) {
+        const T th = theta[e];
+        const int32_t ti = a.src[e], tj = a.col[e];
+        const bool congested = th > T(0);
+        const T cut = congested ? th : T(0);
+        const VT* fr = reinterpret_cast<const VT*>(a.f + e * a.Kp);
+        const VT* hi = reinterpret_cast<const VT*>(a.h + (int64_t)ti * a.Kp);
+        const VT* hj = reinterpret_cast<const VT*>(a.h + (int64_t)tj * a.Kp);
+        const VT* fb = FUSED ? nullptr : reinterpret_cast<const VT*>(fbar + e * a.Kp);
+        VT* cb = reinterpret_cast<VT*>(cbar + e * a.Kp);
+        const VT* di = FUSED ? reinterpret_cast<const VT*>(Dbar + (int64_t)ti * a.Kp) : nullptr;
+        const VT* dj = FUSED ? reinterpret_cast<const VT*>(Dbar + (int64_t)tj * a.Kp) : nullptr;
+        T g[V][N];
+        uint32_t act = 0;  // bit q*N + j: value j of vector q is in the active set
+        T sb = T(0);
+        int na = 0;
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            const int v = lane + q * 32;
+            if (v < vpr) {
+                T f[N], x[N], y[N];
+                unpack(fr[v], f);
+                unpack(hi[v], x);
+                unpack(hj[v], y);
+                fbar_vec<T, FUSED>(fb, cb, di, dj, v, g[q]);
+#pragma unroll
+                for (int j = 0; j < N; ++j)
+                    if (fma(T(0.5), x[j] - y[j], f[j]) > cut) {  // the edge-QP kernel's c
+                        act |= 1u << (q * N + j);
+                        sb += g[q][j];
+                        ++na;
+                    }
+            } else {
+#pragma unroll
+                for (int j = 0; j < N; ++j) g[q][j] = T(0);
+            }
+        }
+        sb = group_sum<32>(sb);
+        na = group_sum<32>(na);
+        const T corr = (congested && na > 0) ? sb / T((a.ck ? 0 : 2) + na) : T(0);
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            const int v = lane + q * 32;
+            if (v < vpr) {
+                T o[N];
+#pragma unroll
+                for (int j = 0; j < N; ++j) o[j] = ((act >> (q * N + j)) & 1u) ? g[q][j] - corr : T(0);
+                cb[v] = pack4(o);
+            }
+        }
+        if (lane == 0) ubar[e] += (double)corr;
+    }
+}
+
 // Block of B threads per edge for long rows (thread l holds row vectors l +
 // q*B): the same step as edge_backward_kernel, but the row's cotangent and
 // its active-set bits stay in registers between the block-wide sum and the
@@ -238,6 +309,28 @@ __global__ void __launch_bounds__(B, (1024 / B > 1 ? 1024 / B : 1))
     }
 }
 
+// acc += the W list entries from q on: in-edges (ev >= 0) took -h_j/2, out-edges (~e) took +h_i/2.
+template <typename T, int W>
+__device__ __forceinline__ void gather_backward(const SweepArgs<T>& a, const T* __restrict__ cbar, int64_t q, int64_t v,
+                                                T (&acc)[VecOf<T>::N])
+{
+    using VT = typename VecOf<T>::type;
+    constexpr int N = VecOf<T>::N;
+    int32_t ev[W];
+    T x[W][N];
+#pragma unroll
+    for (int u = 0; u < W; ++u) ev[u] = a.inc[q + u];
+#pragma unroll
+    for (int u = 0; u < W; ++u) {
+        const int64_t e = ev[u] >= 0 ? ev[u] : ~ev[u];
+        unpack(reinterpret_cast<const VT*>(cbar + e * a.Kp)[v], x[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < W; ++u)
+#pragma unroll
+        for (int j = 0; j < N; ++j) acc[j] += ev[u] >= 0 ? -x[u][j] : x[u][j];
+}
+
 // Thread per (vertex, vector): Dbar = (sum_out cbar - sum_in cbar) / (2 delta),
 // the incidence list traversed in its stored order as by the excess kernel.
 template <typename T>
@@ -257,30 +350,12 @@ __global__ void __launch_bounds__(kThreads) vertex_backward_kernel(SweepArgs<T> 
         for (int j = 0; j < N; ++j) acc[j] = T(0);
         const int64_t q1 = a.inc_ptr[i + 1];
         int64_t q = a.inc_ptr[i];
-        for (; q + 4 <= q1; q += 4) {  // four rows in flight
-            int32_t ev[4];
-            T x[4][N];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) ev[u] = a.inc[q + u];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int64_t e = ev[u] >= 0 ? ev[u] : ~ev[u];
-                unpack(reinterpret_cast<const VT*>(cbar + e * a.Kp)[v], x[u]);
-            }
-            // in-edges (ev >= 0) took -h_j/2, out-edges (~e) took +h_i/2
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int j = 0; j < N; ++j) acc[j] = ev[u] >= 0 ? acc[j] - x[u][j] : acc[j] + x[u][j];
+        for (; q + 8 <= q1; q += 8) gather_backward<T, 8>(a, cbar, q, v, acc);  // eight rows in flight
+        if (q + 4 <= q1) {
+            gather_backward<T, 4>(a, cbar, q, v, acc);
+            q += 4;
         }
-        for (; q < q1; ++q) {
-            const int32_t ev = a.inc[q];
-            const int64_t e = ev >= 0 ? ev : ~ev;
-            T x[N];
-            unpack(reinterpret_cast<const VT*>(cbar + e * a.Kp)[v], x);
-#pragma unroll
-            for (int j = 0; j < N; ++j) acc[j] = ev >= 0 ? acc[j] - x[j] : acc[j] + x[j];
-        }
+        for (; q < q1; ++q) gather_backward<T, 1>(a, cbar, q, v, acc);
         const T s = T(0.5) * a.inv_deg[i];
         T o[N];
 #pragma unroll
@@ -307,6 +382,16 @@ cudaError_t launch_seed(const SweepArgs<T>& a, T* fbar, double* ubar, double* db
     return cudaGetLastError();
 }
 
+template <typename T, int V>
+void launch_backward_warp(const SweepArgs<T>& a, const T* theta, const T* fbar, T* cbar, T* Dbar, double* ubar,
+                          int fused, cudaStream_t s)
+{
+    const int64_t want = (a.m + kThreads / 32 - 1) / (kThreads / 32), cap = 1 << 20;
+    const int g = (int)(want < cap ? want : cap);
+    if (fused) edge_backward_warp_kernel<T, V, true><<<g, kThreads, 0, s>>>(a, theta, fbar, cbar, Dbar, ubar);
+    else edge_backward_warp_kernel<T, V, false><<<g, kThreads, 0, s>>>(a, theta, fbar, cbar, Dbar, ubar);
+}
+
 template <typename T, int B, int V>
 void launch_backward_block(const SweepArgs<T>& a, const T* theta, const T* fbar, T* cbar, T* Dbar, double* ubar,
                            int fused, int num_sms, cudaStream_t s)
@@ -317,16 +402,16 @@ void launch_backward_block(const SweepArgs<T>& a, const T* theta, const T* fbar,
     else edge_backward_block_kernel<T, B, V, false><<<g, B, 0, s>>>(a, theta, fbar, cbar, Dbar, ubar);
 }
 
-// The edge step's form: the block form with the smallest row capacity that
-// holds Kp, for rows longer than two vectors per lane of a warp; else (and
-// beyond the largest block capacity) the warp form.
+// The edge step's form by the row's length in vectors: a warp with the row in
+// registers up to 8 vectors per lane (0..6); the block form with the smallest
+// capacity that holds the row (7..12); beyond the largest the warp form that
+// reads twice (-1).
 template <typename T>
-int backward_block_form(int Kp)
+int backward_form(int Kp)
 {
     const int vpr = Kp / VecOf<T>::N;
-    if (vpr <= 64) return -1;
-    const int cap[] = {128 * 2, 128 * 4, 256 * 4, 512 * 4, 512 * 5, 512 * 8, 1024 * 8};  // vectors, B x V
-    for (int i = 0; i < 7; ++i)
+    const int cap[] = {32, 64, 96, 128, 160, 192, 256, 128 * 4, 256 * 4, 512 * 4, 512 * 5, 512 * 8, 1024 * 8};
+    for (int i = 0; i < 13; ++i)
         if (vpr <= cap[i]) return i;
     return -1;
 }
@@ -336,14 +421,20 @@ cudaError_t launch_backward_sweep(const SweepArgs<T>& a, const T* theta, const T
                                   double* ubar, double* dbar, uint32_t* mask, int fused, int num_sms, cudaStream_t s)
 {
     const int ge = blocks(a.m * 32, kThreads, num_sms);
-    switch (a.m > 0 ? backward_block_form<T>(a.Kp) : -1) {
-    case 0: launch_backward_block<T, 128, 2>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
-    case 1: launch_backward_block<T, 128, 4>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
-    case 2: launch_backward_block<T, 256, 4>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
-    case 3: launch_backward_block<T, 512, 4>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
-    case 4: launch_backward_block<T, 512, 5>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
-    case 5: launch_backward_block<T, 512, 8>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
-    case 6: launch_backward_block<T, 1024, 8>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
+    switch (a.m > 0 ? backward_form<T>(a.Kp) : -1) {
+    case 0: launch_backward_warp<T, 1>(a, theta, fbar, cbar, Dbar, ubar, fused, s); break;
+    case 1: launch_backward_warp<T, 2>(a, theta, fbar, cbar, Dbar, ubar, fused, s); break;
+    case 2: launch_backward_warp<T, 3>(a, theta, fbar, cbar, Dbar, ubar, fused, s); break;
+    case 3: launch_backward_warp<T, 4>(a, theta, fbar, cbar, Dbar, ubar, fused, s); break;
+    case 4: launch_backward_warp<T, 5>(a, theta, fbar, cbar, Dbar, ubar, fused, s); break;
+    case 5: launch_backward_warp<T, 6>(a, theta, fbar, cbar, Dbar, ubar, fused, s); break;
+    case 6: launch_backward_warp<T, 8>(a, theta, fbar, cbar, Dbar, ubar, fused, s); break;
+    case 7: launch_backward_block<T, 128, 4>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
+    case 8: launch_backward_block<T, 256, 4>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
+    case 9: launch_backward_block<T, 512, 4>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
+    case 10: launch_backward_block<T, 512, 5>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
+    case 11: launch_backward_block<T, 512, 8>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
+    case 12: launch_backward_block<T, 1024, 8>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
     default:
         if (fused) edge_backward_kernel<T, true><<<ge, kThreads, 0, s>>>(a, theta, fbar, cbar, Dbar, ubar, mask);
         else edge_backward_kernel<T, false><<<ge, kThreads, 0, s>>>(a, theta, fbar, cbar, Dbar, ubar, mask);

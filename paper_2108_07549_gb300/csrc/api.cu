@@ -1307,7 +1307,8 @@ pdr_status backward_T(pdr_ctx* ctx, int64_t Tn, int32_t C, double* L, double* gr
         if (!(q = (T*)grab(sizeof(T) * 2 * mm))) return cleanup(), ctx->fail(PDR_ERR_OOM, "sweep-state allocation failed");
     // otherwise checkpoints of the flows and of the roots and warm starts at t = 0, C, 2C, ...
     const bool ckpt = grads && !keep_all;
-    std::vector<T*> ck(ckpt ? nseg : 0), thck(ckpt ? nseg : 0), seg, th, hseg;
+    const int64_t nck = ckpt && nseg > 0 ? nseg - 1 : 0;  // the last segment starts where the forward pass is
+    std::vector<T*> ck(nck), thck(nck), seg, th, hseg;
     for (auto& q : ck)
         if (!(q = (T*)grab(sizeof(T) * fm))) return cleanup(), ctx->fail(PDR_ERR_OOM, "checkpoint allocation failed");
     for (auto& q : thck)
@@ -1321,7 +1322,7 @@ pdr_status backward_T(pdr_ctx* ctx, int64_t Tn, int32_t C, double* L, double* gr
         for (auto& q : seg)
             if (!(q = (T*)grab(sizeof(T) * fm))) return cleanup(), ctx->fail(PDR_ERR_OOM, "segment allocation failed");
         for (auto& q : th)
-            if (!(q = (T*)grab(sizeof(T) * mm))) return cleanup(), ctx->fail(PDR_ERR_OOM, "segment allocation failed");
+            if (!(q = (T*)grab(sizeof(T) * 2 * mm))) return cleanup(), ctx->fail(PDR_ERR_OOM, "segment allocation failed");
         hseg.resize(C);  // the heights of every sweep of a segment, kept from its recomputation
         for (auto& q : hseg)
             if (!(q = (T*)grab(sizeof(T) * hn))) return cleanup(), ctx->fail(PDR_ERR_OOM, "segment allocation failed");
@@ -1346,8 +1347,8 @@ pdr_status backward_T(pdr_ctx* ctx, int64_t Tn, int32_t C, double* L, double* gr
             a.h = hs[t];
             if (t > 0) a.theta_in = ths[t - 1];
             a.theta = ths[t];
-            CKB(launch_excess<T>(a, ctx->stream));
-            CKB(launch_edge<T>(a, ctx->cfg[Prec<T>::id], ctx->stream));
+            CKB(launch_excess<T>(a, ctx->stream, t > 0));
+            CKB(launch_edge<T>(a, ctx->cfg[Prec<T>::id], ctx->stream, true));
         }
         if (Tn > 0) {  // f^(T) and the last roots become the current state
             CKB(cudaMemcpyAsync(Prec<T>::f(ctx, ctx->cur), fs[Tn], sizeof(T) * fm, cudaMemcpyDeviceToDevice,
@@ -1356,16 +1357,38 @@ pdr_status backward_T(pdr_ctx* ctx, int64_t Tn, int32_t C, double* L, double* gr
                                 ctx->stream));
         }
     }
-    for (int64_t t = 0; !keep_all && t < Tn; ++t) {
+    // The kernels of a run of sweeps but its first are launched programmatically
+    // dependent, as in the captured loop.  One sweep of segment t0: flows, heights and roots to the segment's own buffers.
+    auto segment_sweep = [&](int64_t t0, int64_t t, const T* theta0) -> cudaError_t {
+        SweepArgs<T> a = make_args<T>(ctx, MODE_FORCED);
+        a.f = seg[t - t0];
+        a.f_out = seg[t - t0 + 1];
+        a.h = hseg[t - t0];
+        a.theta_in = t > t0 ? th[t - t0 - 1] : theta0;
+        a.theta = th[t - t0];
+        const cudaError_t e = launch_excess<T>(a, ctx->stream, t > t0);
+        return e != cudaSuccess ? e : launch_edge<T>(a, ctx->cfg[Prec<T>::id], ctx->stream, true);
+    };
+    // the last segment's sweeps keep their states on the way forward
+    const int64_t t_last = ckpt && Tn > 0 ? (nseg - 1) * C : Tn;
+    for (int64_t t = 0; !keep_all && t < t_last; ++t) {
         if (grads && t % C == 0) {  // the flows and the warm starts sweep t reads
             CKB(cudaMemcpyAsync(ck[t / C], Prec<T>::f(ctx, ctx->cur), sizeof(T) * fm, cudaMemcpyDeviceToDevice, ctx->stream));
             CKB(cudaMemcpyAsync(thck[t / C], ctx->theta[ctx->cur], sizeof(T) * 2 * ctx->m, cudaMemcpyDeviceToDevice,
                                 ctx->stream));
         }
         SweepArgs<T> a = make_args<T>(ctx, MODE_FORCED);
-        CKB(launch_excess<T>(a, ctx->stream));
-        CKB(launch_edge<T>(a, ctx->cfg[Prec<T>::id], ctx->stream));
+        CKB(launch_excess<T>(a, ctx->stream, t > 0 && !(grads && t % C == 0)));
+        CKB(launch_edge<T>(a, ctx->cfg[Prec<T>::id], ctx->stream, true));
         ctx->cur ^= 1;
+    }
+    if (!keep_all && t_last < Tn) {
+        CKB(cudaMemcpyAsync(seg[0], Prec<T>::f(ctx, ctx->cur), sizeof(T) * fm, cudaMemcpyDeviceToDevice, ctx->stream));
+        for (int64_t t = t_last; t < Tn; ++t) CKB(segment_sweep(t_last, t, reinterpret_cast<const T*>(ctx->theta[ctx->cur])));
+        CKB(cudaMemcpyAsync(Prec<T>::f(ctx, ctx->cur), seg[Tn - t_last], sizeof(T) * fm, cudaMemcpyDeviceToDevice,
+                            ctx->stream));
+        CKB(cudaMemcpyAsync(ctx->theta[ctx->cur], th[Tn - t_last - 1], sizeof(T) * 2 * ctx->m, cudaMemcpyDeviceToDevice,
+                            ctx->stream));
     }
     // L = z(f^(T)) and the seeds
     {
@@ -1388,20 +1411,9 @@ pdr_status backward_T(pdr_ctx* ctx, int64_t Tn, int32_t C, double* L, double* gr
     // or segment by segment from the last
     for (int64_t sgi = nseg - 1; ckpt && sgi >= 0; --sgi) {
         const int64_t t0 = sgi * C, t1 = (t0 + C < Tn) ? t0 + C : Tn;
-        CKB(cudaMemcpyAsync(seg[0], ck[sgi], sizeof(T) * fm, cudaMemcpyDeviceToDevice, ctx->stream));
-        CKB(cudaMemcpyAsync(ctx->theta[0], thck[sgi], sizeof(T) * 2 * ctx->m, cudaMemcpyDeviceToDevice, ctx->stream));
-        for (int64_t t = t0; t < t1; ++t) {  // recompute f^(t0+1..t1-1); keep each sweep's heights and roots
-            const int rb = (int)((t - t0) & 1);
-            SweepArgs<T> a = make_args<T>(ctx, MODE_FORCED);
-            a.f = seg[t - t0];
-            a.f_out = seg[t - t0 + 1];
-            a.h = hseg[t - t0];
-            a.theta_in = reinterpret_cast<const T*>(ctx->theta[rb]);
-            a.theta = reinterpret_cast<T*>(ctx->theta[rb ^ 1]);
-            CKB(launch_excess<T>(a, ctx->stream));
-            CKB(launch_edge<T>(a, ctx->cfg[Prec<T>::id], ctx->stream));
-            CKB(cudaMemcpyAsync(th[t - t0], ctx->theta[rb ^ 1], sizeof(T) * ctx->m, cudaMemcpyDeviceToDevice,
-                                ctx->stream));
+        if (sgi < nseg - 1) {  // recompute f^(t0+1..t1-1); keep each sweep's heights and roots
+            CKB(cudaMemcpyAsync(seg[0], ck[sgi], sizeof(T) * fm, cudaMemcpyDeviceToDevice, ctx->stream));
+            for (int64_t t = t0; t < t1; ++t) CKB(segment_sweep(t0, t, thck[sgi]));
         }
         for (int64_t t = t1 - 1; t >= t0; --t) {
             SweepArgs<T> a = make_args<T>(ctx, MODE_EVAL);
