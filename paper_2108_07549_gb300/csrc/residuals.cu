@@ -35,7 +35,7 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kVParts = 3;  // per vertex block: zsum, cons_abs, cons_rel
-constexpr int kEParts = 5;  // per edge block: psi2, cap_abs, cap_rel, cost, fmin
+constexpr int kEParts = 5;  // per edge block: psi2, cost, cap_abs, cap_rel, fmin
 
 __device__ __forceinline__ double wsum(double x)
 {
@@ -43,10 +43,28 @@ __device__ __forceinline__ double wsum(double x)
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
     return x;
 }
-__device__ __forceinline__ double wmax(double x)
+// Of two values, each in every lane: half the additions, in the same tree.
+__device__ __forceinline__ void wsum2(double& a, double& b)
 {
+    const bool upper = (threadIdx.x & 16) != 0;
+    double x = (upper ? b : a) + __shfl_xor_sync(kFull, upper ? a : b, 16);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(kFull, x, o));
+    for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+    a = __shfl_sync(kFull, x, 0);
+    b = __shfl_sync(kFull, x, 16);
+}
+// The larger of a value that is not negative and another (NaN loses), compared
+// by their bit patterns: comparisons of doubles run on the FP64 pipe.
+__device__ __forceinline__ double max_nn(double x, double y)
+{
+    const long long b = __double_as_longlong(y);
+    return b > __double_as_longlong(x) && b <= 0x7ff0000000000000ll ? y : x;
+}
+__device__ __forceinline__ double wmax(double x)  // 0 at least
+{
+    x = max_nn(0.0, x);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x = max_nn(x, __shfl_xor_sync(kFull, x, o));
     return x;
 }
 __device__ __forceinline__ double wmin(double x)
@@ -56,25 +74,33 @@ __device__ __forceinline__ double wmin(double x)
     return x;
 }
 
-// Block reduction of up to 5 values with per-slot operations (0 sum, 1 max,
-// 2 min); the results are valid in thread 0.
-template <int NV>
-__device__ void block_reduce(double* v, const int* op, double (*smem)[32])
+// The first NS of NV values are summed, the next NX maximised (none is
+// negative), the rest minimised, over a warp.
+template <int NV, int NS, int NX>
+__device__ __forceinline__ void warp_reduce(double* v)
+{
+#pragma unroll
+    for (int q = 0; q + 1 < NS; q += 2) wsum2(v[q], v[q + 1]);
+    if constexpr (NS & 1) v[NS - 1] = wsum(v[NS - 1]);
+#pragma unroll
+    for (int q = NS; q < NV; ++q) v[q] = q < NS + NX ? wmax(v[q]) : wmin(v[q]);
+}
+// The same over a block; the results are valid in thread 0.  Bound by the FP64
+// pipe (every warp's additions, two per clock and SM): sums in pairs and maxima
+// by bit patterns take 10 of its instructions per warp for five values, not 25.
+template <int NV, int NS, int NX>
+__device__ void block_reduce(double* v, double (*smem)[32])
 {
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
+    warp_reduce<NV, NS, NX>(v);
 #pragma unroll
-    for (int q = 0; q < NV; ++q) {
-        v[q] = op[q] == 0 ? wsum(v[q]) : op[q] == 1 ? wmax(v[q]) : wmin(v[q]);
+    for (int q = 0; q < NV; ++q)
         if (l == 0) smem[q][w] = v[q];
-    }
     __syncthreads();
     if (w == 0) {
 #pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            const double idn = op[q] == 2 ? INFINITY : 0.0;
-            double x = l < nw ? smem[q][l] : idn;
-            v[q] = op[q] == 0 ? wsum(x) : op[q] == 1 ? wmax(x) : wmin(x);
-        }
+        for (int q = 0; q < NV; ++q) v[q] = l < nw ? smem[q][l] : q < NS + NX ? 0.0 : INFINITY;
+        warp_reduce<NV, NS, NX>(v);
     }
     __syncthreads();
 }
@@ -228,8 +254,7 @@ __global__ void __launch_bounds__(256)
         *reinterpret_cast<float4*>(h32 + (int64_t)i * Kp + k0) = make_float4(hf[0], hf[1], hf[2], hf[3]);
     }
     double v[3] = {zsum, cabs, crel};
-    const int op[3] = {0, 1, 1};
-    block_reduce<3>(v, op, smem);
+    block_reduce<3, 1, 2>(v, smem);
     if (threadIdx.x == 0)
         for (int q = 0; q < kVParts; ++q) part[(int64_t)blockIdx.x * kVParts + q] = v[q];
 }
@@ -307,8 +332,7 @@ __global__ void __launch_bounds__(256)
         }
     }
     double v[3] = {zsum, cabs, crel};
-    const int op[3] = {0, 1, 1};
-    block_reduce<3>(v, op, smem);
+    block_reduce<3, 1, 2>(v, smem);
     if (threadIdx.x == 0)
         for (int q = 0; q < kVParts; ++q) part[(int64_t)blockIdx.x * kVParts + q] = v[q];
 }
@@ -434,9 +458,8 @@ __global__ void __launch_bounds__(256)
             fmn = fmin(fmn, mn);
         }
     }
-    double v[5] = {psi2, capa, capr, cost, fmn};
-    const int op[5] = {0, 1, 1, 0, 2};
-    block_reduce<5>(v, op, smem);
+    double v[5] = {psi2, cost, capa, capr, fmn};
+    block_reduce<5, 2, 2>(v, smem);
     if (threadIdx.x == 0)
         for (int q = 0; q < kEParts; ++q) part[(int64_t)blockIdx.x * kEParts + q] = v[q];
 }
@@ -468,33 +491,31 @@ __global__ void __launch_bounds__(1024)
     double zv = 0.0, cabs = 0.0, crel = 0.0;
     for (int b = threadIdx.x; b < grid_v; b += blockDim.x) {
         zv += part[(int64_t)b * kVParts + 0];
-        cabs = fmax(cabs, part[(int64_t)b * kVParts + 1]);
-        crel = fmax(crel, part[(int64_t)b * kVParts + 2]);
+        cabs = max_nn(cabs, part[(int64_t)b * kVParts + 1]);
+        crel = max_nn(crel, part[(int64_t)b * kVParts + 2]);
     }
     const double* pe = part + (int64_t)grid_v * kVParts;
     double psi2 = 0.0, capa = 0.0, capr = 0.0, cost = 0.0, fmn = INFINITY;
     for (int b = threadIdx.x; b < grid_e; b += blockDim.x) {
         psi2 += pe[(int64_t)b * kEParts + 0];
-        capa = fmax(capa, pe[(int64_t)b * kEParts + 1]);
-        capr = fmax(capr, pe[(int64_t)b * kEParts + 2]);
-        cost += pe[(int64_t)b * kEParts + 3];
+        cost += pe[(int64_t)b * kEParts + 1];
+        capa = max_nn(capa, pe[(int64_t)b * kEParts + 2]);
+        capr = max_nn(capr, pe[(int64_t)b * kEParts + 3]);
         fmn = fmin(fmn, pe[(int64_t)b * kEParts + 4]);
     }
     double v1[5] = {gain, gabs, zv, cabs, crel};
-    const int op1[5] = {0, 0, 0, 1, 1};
-    block_reduce<5>(v1, op1, smem);
-    double v2[5] = {psi2, capa, capr, cost, fmn};
-    const int op2[5] = {0, 1, 1, 0, 2};
-    block_reduce<5>(v2, op2, smem);
+    block_reduce<5, 3, 2>(v1, smem);
+    double v2[5] = {psi2, cost, capa, capr, fmn};
+    block_reduce<5, 2, 2>(v2, smem);
     if (threadIdx.x == 0) {
         out->z = 0.5 * (v2[0] + v1[2]);
-        out->cap_abs = v2[1];
-        out->cap_rel = v2[2];
+        out->cap_abs = v2[2];
+        out->cap_rel = v2[3];
         out->cons_abs = v1[3];
         out->cons_rel = v1[4];
         out->f_min = a.m > 0 ? v2[4] : 0.0;
-        out->margin = v1[0] - v2[3];
-        out->margin_scale = v1[1] + v2[3];
+        out->margin = v1[0] - v2[1];
+        out->margin_scale = v1[1] + v2[1];
     }
 }
 
@@ -508,7 +529,7 @@ void launch_passes(const ResidTask<T>* tasks, const ResidTask<T>& one, int count
     if constexpr (sizeof(T) == 4) resid_vertex_pair_kernel<TABLE><<<dim3(gv, count), 256, 0, stream>>>(tasks, one);
     else resid_vertex_kernel<TABLE><<<dim3(gv, count), 256, 0, stream>>>(tasks, one);
     resid_edge_kernel<T, TABLE><<<dim3(ge, count), 256, 0, stream>>>(tasks, one);
-    resid_final_kernel<T, TABLE><<<count, longest > 256 ? 1024 : 256, 0, stream>>>(tasks, one);
+    resid_final_kernel<T, TABLE><<<count, longest > 2048 ? 1024 : longest > 256 ? 512 : 256, 0, stream>>>(tasks, one);
 }
 
 template <typename T>
