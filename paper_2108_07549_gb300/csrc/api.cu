@@ -2509,8 +2509,19 @@ struct pdr_batch {
 
 namespace {
 
-constexpr int kBatchUnroll = 2;  // sweeps per instance per iteration of the batch's while loop
 constexpr int kBatchPool = 32;   // capture streams
+// Branches of a batch's graph.  The streams take turns at the instances; of
+// those whose flows and heights take kBatchLargeBytes or more only kBatchLarge
+// are in flight at a time, so that an instance's rows are still in L2 in its
+// next sweeps.  Sweeps per iteration of the loop: 8, less in a large batch
+// (graph nodes are paid for once, at the first solve); the join at the end of
+// an iteration waits for the slowest branch.
+// us, 24 instances of n 100-5000, K 10-1000, 30 sweeps / 96 of n 100-500,
+// K 10-100, 100 sweeps: all streams and 2 sweeps 14,704 / 6531; this rule 14,122 /
+// 6379; all instances on 3 streams 13,691 / 9916, on 16 14,642 / 6294.
+constexpr int kBatchLarge = 3;
+constexpr double kBatchLargeBytes = 12.0 * 1024 * 1024;
+int batch_unroll(int running) { return running <= 64 ? 8 : running <= 128 ? 4 : 2; }
 
 pdr_status batch_fail(pdr_status code, const std::string& msg)
 {
@@ -2602,7 +2613,7 @@ SweepArgs<T> batch_args(pdr_batch* b, pdr_ctx* ctx, int use_cond, cudaGraphCondi
 }
 
 // One graph: a conditional while node whose body forks one branch per
-// running instance (kBatchUnroll sweeps each) and joins them.
+// running instance (batch_unroll sweeps each) and joins them.
 template <typename T>
 void batch_build_graph(pdr_batch* b, const std::vector<char>& run)
 {
@@ -2635,10 +2646,15 @@ void batch_build_graph(pdr_batch* b, const std::vector<char>& run)
     {
         cudaError_t e = cudaEventRecord(ev[0], b->cap_stream);
         for (size_t p = 0; p < b->pool.size() && e == cudaSuccess; ++p) e = cudaStreamWaitEvent(b->pool[p], ev[0], 0);
-        for (int32_t i = 0, r = 0; i < b->count && e == cudaSuccess; ++i) {
+        const int unroll = batch_unroll((int)std::count(run.begin(), run.end(), 1));
+        const size_t pool = b->pool.size(), large = pool > 2 * kBatchLarge ? kBatchLarge : 0;
+        for (size_t i = 0, rl = 0, rs = 0; i < run.size() && e == cudaSuccess; ++i) {
             if (!run[i]) continue;
-            cudaStream_t s = b->pool[(r++) % b->pool.size()];
-            for (int q = 0; q < kBatchUnroll && e == cudaSuccess; ++q) {
+            const pdr_ctx* c = b->ctx[i];
+            const double bytes = (2.0 * (double)c->m + (double)c->n) * (double)c->Kp * sizeof(T);
+            const bool big = large > 0 && bytes >= kBatchLargeBytes;
+            cudaStream_t s = b->pool[big ? (rl++) % large : large + (rs++) % (pool - large)];
+            for (int q = 0; q < unroll && e == cudaSuccess; ++q) {
                 SweepArgs<T> a = batch_args<T>(b, b->ctx[i], 1, h, q & 1);
                 e = launch_excess<T>(a, s);
                 if (e == cudaSuccess) e = launch_update<T>(b->ctx[i], a, s);
