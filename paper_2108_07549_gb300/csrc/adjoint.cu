@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(kThreads) seed_edge_kernel(SweepArgs<T> a, T* 
 template <typename T>
 __global__ void demand_kernel(SweepArgs<T> a, const T* __restrict__ x, double* __restrict__ dbar, int accumulate)
 {
+    pdl_wait();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < a.K; k += gridDim.x * blockDim.x) {
         const double v = (double)x[(int64_t)a.s[k] * a.Kp + k] - (double)x[(int64_t)a.t[k] * a.Kp + k];
         dbar[k] = accumulate ? dbar[k] + v : v;
@@ -112,6 +113,7 @@ __global__ void __launch_bounds__(kThreads) edge_backward_kernel(SweepArgs<T> a,
     const int lane = threadIdx.x & 31;
     const int vpr = a.Kp / N;
     const int nq = (vpr + 31) / 32;
+    pdl_wait();
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t e = w0; e < a.m; e += nw) {
@@ -186,6 +188,7 @@ __global__ void __launch_bounds__(kThreads, V <= 4 ? 4 : 3)
     const int vpr = a.Kp / N;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    pdl_wait();  // the kernels before have finished (no-op without PDL)
     for (int64_t e = w0; e < a.m; e += nw) {
         const T th = theta[e];
         const int32_t ti = a.src[e], tj = a.col[e];
@@ -256,6 +259,7 @@ __global__ void __launch_bounds__(B, (1024 / B > 1 ? 1024 / B : 1))
     __shared__ T sa_buf[33];
     __shared__ int sb_buf[33];
     const int vpr = a.Kp / N;
+    pdl_wait();
     for (int64_t e = blockIdx.x; e < a.m; e += gridDim.x) {
         const T th = theta[e];
         const bool congested = th > T(0);
@@ -341,6 +345,7 @@ __global__ void __launch_bounds__(kThreads) vertex_backward_kernel(SweepArgs<T> 
     constexpr int N = VecOf<T>::N;
     const int64_t vpr = a.Kp / N;
     const int64_t total = (int64_t)a.n * vpr;
+    pdl_wait();
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (int64_t)gridDim.x * blockDim.x) {
         const int32_t i = (int32_t)(idx / vpr);
@@ -382,14 +387,31 @@ cudaError_t launch_seed(const SweepArgs<T>& a, T* fbar, double* ubar, double* db
     return cudaGetLastError();
 }
 
+// A launch with programmatic dependent launch: the kernel's blocks may be
+// scheduled while its predecessor drains, and wait for it in pdl_wait.
+template <typename... P, typename... X>
+void launch_dependent(void (*kernel)(P...), int grid, int block, cudaStream_t s, X&&... x)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = s;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(x)...);
+}
+
 template <typename T, int V>
 void launch_backward_warp(const SweepArgs<T>& a, const T* theta, const T* fbar, T* cbar, T* Dbar, double* ubar,
                           int fused, cudaStream_t s)
 {
     const int64_t want = (a.m + kThreads / 32 - 1) / (kThreads / 32), cap = 1 << 20;
     const int g = (int)(want < cap ? want : cap);
-    if (fused) edge_backward_warp_kernel<T, V, true><<<g, kThreads, 0, s>>>(a, theta, fbar, cbar, Dbar, ubar);
-    else edge_backward_warp_kernel<T, V, false><<<g, kThreads, 0, s>>>(a, theta, fbar, cbar, Dbar, ubar);
+    if (fused) launch_dependent(edge_backward_warp_kernel<T, V, true>, g, kThreads, s, a, theta, fbar, cbar, Dbar, ubar);
+    else launch_dependent(edge_backward_warp_kernel<T, V, false>, g, kThreads, s, a, theta, fbar, cbar, Dbar, ubar);
 }
 
 template <typename T, int B, int V>
@@ -398,8 +420,8 @@ void launch_backward_block(const SweepArgs<T>& a, const T* theta, const T* fbar,
 {
     const int64_t per_sm = 1024 / B > 1 ? 1024 / B : 1;  // resident under the kernel's launch bounds
     const int g = (int)(a.m < per_sm * num_sms ? a.m : per_sm * num_sms);
-    if (fused) edge_backward_block_kernel<T, B, V, true><<<g, B, 0, s>>>(a, theta, fbar, cbar, Dbar, ubar);
-    else edge_backward_block_kernel<T, B, V, false><<<g, B, 0, s>>>(a, theta, fbar, cbar, Dbar, ubar);
+    if (fused) launch_dependent(edge_backward_block_kernel<T, B, V, true>, g, B, s, a, theta, fbar, cbar, Dbar, ubar);
+    else launch_dependent(edge_backward_block_kernel<T, B, V, false>, g, B, s, a, theta, fbar, cbar, Dbar, ubar);
 }
 
 // The edge step's form by the row's length in vectors: a warp with the row in
@@ -436,12 +458,12 @@ cudaError_t launch_backward_sweep(const SweepArgs<T>& a, const T* theta, const T
     case 11: launch_backward_block<T, 512, 8>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
     case 12: launch_backward_block<T, 1024, 8>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
     default:
-        if (fused) edge_backward_kernel<T, true><<<ge, kThreads, 0, s>>>(a, theta, fbar, cbar, Dbar, ubar, mask);
-        else edge_backward_kernel<T, false><<<ge, kThreads, 0, s>>>(a, theta, fbar, cbar, Dbar, ubar, mask);
+        if (fused) launch_dependent(edge_backward_kernel<T, true>, ge, kThreads, s, a, theta, fbar, cbar, Dbar, ubar, mask);
+        else launch_dependent(edge_backward_kernel<T, false>, ge, kThreads, s, a, theta, fbar, cbar, Dbar, ubar, mask);
     }
-    vertex_backward_kernel<T><<<blocks((int64_t)a.n * (a.Kp / VecOf<T>::N), kThreads, num_sms), kThreads, 0, s>>>(
-        a, cbar, Dbar);
-    demand_kernel<T><<<blocks(a.K, kThreads, num_sms), kThreads, 0, s>>>(a, Dbar, dbar, 1);
+    launch_dependent(vertex_backward_kernel<T>, blocks((int64_t)a.n * (a.Kp / VecOf<T>::N), kThreads, num_sms), kThreads, s,
+                     a, cbar, Dbar);
+    launch_dependent(demand_kernel<T>, blocks(a.K, kThreads, num_sms), kThreads, s, a, Dbar, dbar, 1);
     return cudaGetLastError();
 }
 

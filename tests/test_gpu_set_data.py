@@ -49,3 +49,21 @@ def test_device_set_data_scales_as_the_host_path(pdr, m_side):
             with pytest.raises(pdr.PdrError) as e:
                 s.set_data_device(bu.data_ptr(), bd.data_ptr())
             assert e.value.status == pdr.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("x", [0.0, -0.0, 5e-324, 1e308, -5e-324, -1.0, float("inf"), -float("inf"), float("nan")])
+def test_device_set_data_domain(pdr, x):
+    """A capacity is finite and not below 0 (-0 included), a demand finite and above 0."""
+    import torch
+
+    inst = I.grid5_k10(1.0)
+    with pdr.Solver.from_instance(inst) as s:
+        for u_side in (True, False):
+            u, d = torch.from_numpy(inst.u.copy()).cuda(), torch.from_numpy(inst.d.copy()).cuda()
+            (u if u_side else d)[3] = x
+            if np.isfinite(x) and (x >= 0 if u_side else x > 0):
+                s.set_data_device(u.data_ptr(), d.data_ptr())
+            else:
+                with pytest.raises(pdr.PdrError) as e:
+                    s.set_data_device(u.data_ptr(), d.data_ptr())
+                assert e.value.status == pdr.ERR_INVALID_ARG
