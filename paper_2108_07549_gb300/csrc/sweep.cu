@@ -1720,11 +1720,14 @@ template int edge_ring_grid<double>(int, int64_t, int, int);
 constexpr int share_limit(int G, int V) { return V >= 8 ? 1 : V >= 4 ? 2 : 4; }
 
 // Lanes' shares of variant cfg for m edges (1: the plain form): FP64 only, the
-// most that leave a warp to each of the SMs' four schedulers.  (FP32 has its
+// most that leave a warp to each of the SMs' four schedulers (fewer edges are a
+// chain of latencies, which more rows per lane only lengthen).  (FP32 has its
 // ring form, and its fixed cost per edge is on pipes that are not the bound.)
 // Bound: the FP64 pipe, two operations per clock and SM.  Together with the
 // comparisons made on bit patterns (exceeds), n 500, m 3000, K 100: 41 us per
-// sweep (about 100 FP64 warp instructions per edge) to 23.
+// sweep (about 100 FP64 warp instructions per edge) to 23, and 20 with the
+// excess pass's gathers.  The pipe is 29 % busy then: chains of FP64 and shuffle
+// latencies are left.
 template <typename T>
 int edge_shares(int cfg, int64_t m, int num_sms)
 {
