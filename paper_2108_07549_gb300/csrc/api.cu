@@ -771,9 +771,22 @@ pdr_status read_state(pdr_ctx* ctx)
     return PDR_OK;
 }
 
+// Programmatic dependent launch of a run of sweeps: not for the edge QP's block
+// forms on rows that stream from HBM, where blocks that wait in their SMs slow
+// the kernel still running more than an early launch gains (with / without, us:
+// n 10,000, m 39,600, K 10,000, 20 sweeps 26,701 / 25,978; n 20,000, m 100,000,
+// K 2000, 20 sweeps 16,417 / 15,722, 50 sweeps of the reverse mode's forward
+// pass 32,780 / 31,350).
+template <typename T>
+bool pdl_pays(const pdr_ctx* ctx)
+{
+    const int p = Prec<T>::id;
+    return is_gd(ctx->opt) || !edge_config_block(ctx->cfg[p]) || ctx->pf[p] == 0;
+}
+
 // The sweep loop as one graph: a conditional WHILE node whose body holds
 // kUnroll sweeps (excess kernel, then update kernel).  The body's
-// kernels are captured with programmatic dependent launch (each may be
+// kernels are captured with programmatic dependent launch where it pays (each may be
 // scheduled while its predecessor drains); if the runtime refuses that, the
 // body is captured again with plain launches.
 template <typename T>
@@ -827,7 +840,7 @@ pdr_status build_graph(pdr_ctx* ctx)
     const int p = Prec<T>::id;
     ctx->graph_tried[p] = true;
     ctx->graph_ok[p] = false;
-    if (try_build_graph<T>(ctx, true)) return PDR_OK;
+    if (pdl_pays<T>(ctx) && try_build_graph<T>(ctx, true)) return PDR_OK;
     try_build_graph<T>(ctx, false);
     return PDR_OK;  // if both failed, the host loop takes over
 }
@@ -1343,6 +1356,8 @@ pdr_status backward_T(pdr_ctx* ctx, int64_t Tn, int32_t C, double* L, double* gr
         if (!fbar || !cbar || !Dbar || !ubar || !dbar || !mask)
             return cleanup(), ctx->fail(PDR_ERR_OOM, "adjoint allocation failed");
     }
+    // the kernels of a run of sweeps but its first, as in the captured loop
+    const bool pdl = pdl_pays<T>(ctx);
     // forward from f = 0 (pdr_backward reset the flows), cold roots
     if (keep_all) {
         CKB(cudaMemcpyAsync(fs[0], Prec<T>::f(ctx, ctx->cur), sizeof(T) * fm, cudaMemcpyDeviceToDevice, ctx->stream));
@@ -1353,8 +1368,8 @@ pdr_status backward_T(pdr_ctx* ctx, int64_t Tn, int32_t C, double* L, double* gr
             a.h = hs[t];
             if (t > 0) a.theta_in = ths[t - 1];
             a.theta = ths[t];
-            CKB(launch_excess<T>(a, ctx->stream, t > 0));
-            CKB(launch_edge<T>(a, ctx->cfg[Prec<T>::id], ctx->stream, true));
+            CKB(launch_excess<T>(a, ctx->stream, pdl && t > 0));
+            CKB(launch_edge<T>(a, ctx->cfg[Prec<T>::id], ctx->stream, pdl));
         }
         if (Tn > 0) {  // f^(T) and the last roots become the current state
             CKB(cudaMemcpyAsync(Prec<T>::f(ctx, ctx->cur), fs[Tn], sizeof(T) * fm, cudaMemcpyDeviceToDevice,
@@ -1363,8 +1378,7 @@ pdr_status backward_T(pdr_ctx* ctx, int64_t Tn, int32_t C, double* L, double* gr
                                 ctx->stream));
         }
     }
-    // The kernels of a run of sweeps but its first are launched programmatically
-    // dependent, as in the captured loop.  One sweep of segment t0: flows, heights and roots to the segment's own buffers.
+    // One sweep of segment t0: flows, heights and roots to the segment's own buffers.
     auto segment_sweep = [&](int64_t t0, int64_t t, const T* theta0) -> cudaError_t {
         SweepArgs<T> a = make_args<T>(ctx, MODE_FORCED);
         a.f = seg[t - t0];
@@ -1372,8 +1386,8 @@ pdr_status backward_T(pdr_ctx* ctx, int64_t Tn, int32_t C, double* L, double* gr
         a.h = hseg[t - t0];
         a.theta_in = t > t0 ? th[t - t0 - 1] : theta0;
         a.theta = th[t - t0];
-        const cudaError_t e = launch_excess<T>(a, ctx->stream, t > t0);
-        return e != cudaSuccess ? e : launch_edge<T>(a, ctx->cfg[Prec<T>::id], ctx->stream, true);
+        const cudaError_t e = launch_excess<T>(a, ctx->stream, pdl && t > t0);
+        return e != cudaSuccess ? e : launch_edge<T>(a, ctx->cfg[Prec<T>::id], ctx->stream, pdl);
     };
     // the last segment's sweeps keep their states on the way forward
     const int64_t t_last = ckpt && Tn > 0 ? (nseg - 1) * C : Tn;
@@ -1384,8 +1398,8 @@ pdr_status backward_T(pdr_ctx* ctx, int64_t Tn, int32_t C, double* L, double* gr
                                 ctx->stream));
         }
         SweepArgs<T> a = make_args<T>(ctx, MODE_FORCED);
-        CKB(launch_excess<T>(a, ctx->stream, t > 0 && !(grads && t % C == 0)));
-        CKB(launch_edge<T>(a, ctx->cfg[Prec<T>::id], ctx->stream, true));
+        CKB(launch_excess<T>(a, ctx->stream, pdl && t > 0 && !(grads && t % C == 0)));
+        CKB(launch_edge<T>(a, ctx->cfg[Prec<T>::id], ctx->stream, pdl));
         ctx->cur ^= 1;
     }
     if (!keep_all && t_last < Tn) {

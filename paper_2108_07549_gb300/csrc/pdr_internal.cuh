@@ -201,6 +201,7 @@ int edge_group_lanes(int cfg);           // lanes per edge of a lane-group varia
 template <typename T>
 int64_t edge_prefetch_distance(int cfg, int num_sms);  // edges solved by one wave of resident blocks
 bool edge_config_pipelined(int cfg);
+bool edge_config_block(int cfg);         // a block per edge
 bool edge_config_staged(int cfg);       // the bulk-copy staged block forms
 int excess_grid(int32_t n, int Kp, int vec, int num_sms, int resident_blocks, int threads);
 // Persistent sweep kernel (sweep.cu): excess and edge QP of every sweep in one

@@ -1918,6 +1918,7 @@ int edge_plain_config(int cfg)
 }
 
 bool edge_config_pipelined(int cfg) { return cfg >= 0 && cfg < kNumCfg && kCfg[cfg].P == 1; }
+bool edge_config_block(int cfg) { return cfg >= 0 && cfg < kNumCfg && !kCfg[cfg].G; }
 bool edge_config_staged(int cfg) { return cfg >= 0 && cfg < kNumCfg && kCfg[cfg].P == 2; }
 
 cudaError_t launch_convert_f32_to_f64(const float* a, double* b, int64_t count, cudaStream_t stream)
