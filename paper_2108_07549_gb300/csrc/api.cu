@@ -159,7 +159,7 @@ struct pdr_ctx {
     DevState* st = nullptr;
     DevState* hst = nullptr;  // pinned mirror
     bool owns_state = true;   // false: st, hst, r_out and hr_out are slices of a batch's arrays
-    bool psi_stale = false;   // the congestion partials are not those of the current flows (cluster engine)
+    bool psi_stale = false;   // the congestion partials are not those of the current flows (ensure_psi)
     double* trace = nullptr;
     int64_t trace_cap = 0;
     // residuals
@@ -502,7 +502,7 @@ pdr_status refresh_psi_current(pdr_ctx* ctx)
 }
 
 // Before a kernel that reads the congestion partials: the cluster engine, which
-// keeps its own, leaves them behind.
+// keeps its own, and a batch's instance that stopped by a rule leave them behind.
 pdr_status ensure_psi(pdr_ctx* ctx)
 {
     if (!ctx->psi_stale) return PDR_OK;
@@ -2913,8 +2913,13 @@ pdr_status batch_run(pdr_batch* b, const std::vector<char>& run_all, const std::
     }
     const pdr_status s = batch_read_states(b);
     if (s != PDR_OK) return s;
-    for (int32_t i = 0; i < b->count; ++i)
-        if (run[i]) b->ctx[i]->cur = (int)((b->ctx[i]->hst->t - t_start[i]) & 1);
+    for (int32_t i = 0; i < b->count; ++i) {
+        if (!run[i]) continue;
+        pdr_ctx* c = b->ctx[i];
+        c->cur = (int)((c->hst->t - t_start[i]) & 1);
+        // as in run_phase: the sweep that stopped by a rule left the partials of flows that were discarded
+        c->psi_stale = c->hst->reason != STOP_MAX_SWEEPS;
+    }
     return PDR_OK;
 }
 
