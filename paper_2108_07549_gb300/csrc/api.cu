@@ -177,6 +177,7 @@ struct pdr_ctx {
     bool graph_tried[2] = {false, false};
     bool graph_ok[2] = {false, false};
     bool graph_pdl[2] = {false, false};  // the graph's kernels use programmatic dependent launch
+    uint64_t launch_gen = 0;  // counts the changes that outdate captured launch arguments (destroy_graphs)
 
     pdr_result last{};
     std::string err;
@@ -1228,6 +1229,7 @@ pdr_status copy_rows_in(pdr_ctx* ctx, const double* in, int64_t rows, T* ddst)
 
 pdr_status destroy_graphs(pdr_ctx* ctx)
 {
+    ++ctx->launch_gen;
     for (int p = 0; p < 2; ++p) {
         if (ctx->exec[p]) cudaGraphExecDestroy(ctx->exec[p]);
         if (ctx->graph[p]) cudaGraphDestroy(ctx->graph[p]);
@@ -2514,7 +2516,7 @@ struct pdr_batch {
     // one graph per precision, over the instances it was captured for
     cudaGraph_t graph[2] = {nullptr, nullptr};
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
-    std::vector<char> graph_mask[2];
+    std::vector<uint64_t> graph_key[2];  // batch_graph_key
     bool graph_tried[2] = {false, false}, graph_ok[2] = {false, false};
     // cluster engine
     void* bargs = nullptr;   // device ClusterArgs [count]
@@ -2621,7 +2623,17 @@ void batch_destroy_graph(pdr_batch* b, int p)
     b->exec[p] = nullptr;
     b->graph[p] = nullptr;
     b->graph_tried[p] = b->graph_ok[p] = false;
-    b->graph_mask[p].clear();
+    b->graph_key[p].clear();
+}
+
+// What a batch's graph was captured for: per instance 0, or the state of the
+// launch arguments of an instance that runs in it.
+std::vector<uint64_t> batch_graph_key(const pdr_batch* b, const std::vector<char>& run)
+{
+    std::vector<uint64_t> key(run.size(), 0);
+    for (size_t i = 0; i < run.size(); ++i)
+        if (run[i]) key[i] = 1 + b->ctx[i]->launch_gen;
+    return key;
 }
 
 template <typename T>
@@ -2639,7 +2651,7 @@ void batch_build_graph(pdr_batch* b, const std::vector<char>& run)
 {
     const int p = Prec<T>::id;
     b->graph_tried[p] = true;
-    b->graph_mask[p] = run;
+    b->graph_key[p] = batch_graph_key(b, run);
     cudaGraph_t g = nullptr;
     cudaGraphConditionalHandle h;
     cudaGraphNode_t node;
@@ -2886,7 +2898,7 @@ pdr_status batch_run(pdr_batch* b, const std::vector<char>& run_all, const std::
     set_counter_kernel<<<1, 1, 0, b->stream>>>(b->active, running);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return batch_fail(PDR_ERR_CUDA, std::string("batch: ") + cudaGetErrorString(e));
-    if (use_graph && (!b->graph_tried[p] || b->graph_mask[p] != run)) {
+    if (use_graph && (!b->graph_tried[p] || b->graph_key[p] != batch_graph_key(b, run))) {
         batch_destroy_graph(b, p);
         batch_build_graph<T>(b, run);
     }

@@ -58,3 +58,25 @@ def test_congestion_after_a_stop_is_that_of_the_returned_flows(pdr, precision, u
             np.testing.assert_allclose(tr, s.trace(), rtol=1e-12, err_msg=x.name)
         assert r2["sweeps"] == want["sweeps"]
         np.testing.assert_allclose(r2["z"], want["z"], rtol=1e-12)
+
+
+@pytest.mark.parametrize("change", [dict(algo=3), dict(algo=1), dict(algo=2), dict(edge_variant=4),
+                                    dict(excess_variant=2), dict(trace_len=40)])
+def test_options_of_an_instance_reach_its_next_batch_solve(pdr, change):
+    opts = dict(LOOP, eps_obj=0.0, resid_tol=0.0, max_sweeps=25)
+    group = insts()
+    with pdr.Batch(group, **opts) as B:
+        B.solve()
+        view = B.solver(1)
+        view.set_options(**change)
+        B.reset()
+        B.solve()
+        flows = [B.solver(i).flows() for i in range(len(group))]
+        trace = view.trace() if "trace_len" in change else None
+    for i, x in enumerate(group):
+        with pdr.Solver.from_instance(x, **dict(opts, **(change if i == 1 else {}))) as s:
+            s.solve()
+            np.testing.assert_array_equal(flows[i], s.flows(), err_msg=x.name)
+            if i == 1 and trace is not None:
+                assert len(trace) == 26
+                np.testing.assert_allclose(trace, s.trace(), rtol=1e-12)
