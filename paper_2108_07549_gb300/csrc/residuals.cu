@@ -148,6 +148,15 @@ constexpr float kSlack = 0.99999619f;  // 1 - 2^-18
 // reaches the row's largest lower bound can be the maximum.
 constexpr float kHeightSlack = 4.76837158e-7f;  // 2^-21
 
+// h_i - h_j from Delta and 1/delta, each height rounded before the difference:
+// the certificate's potentials are then one fixed vector, whose differences
+// along a path telescope.  (A product fused into the subtraction would enter
+// unrounded, and a path just as long as the demand's drop could seem shorter.)
+__device__ __forceinline__ double height_drop(double di, double wi, double dj, double wj)
+{
+    return __dsub_rn(__dmul_rn(di, wi), __dmul_rn(dj, wj));
+}
+
 // Vertex pass, FP32 flows: one thread per (vertex, four commodities).
 // Delta_ik = sum over in-edges (ascending id) - sum over out-edges
 // (ascending) + the source/sink term (eq. (3), (3h)), the flows summed
@@ -417,13 +426,13 @@ __global__ void __launch_bounds__(256)
             mn = (double)mn32;
             if (need_l) {
                 const float low = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(lb)));  // lb >= 0
-                if (at >= 0 && up >= low) l = fmax(l, h64[ro + at] * wi - h64[co + at] * wj);
+                if (at >= 0 && up >= low) l = fmax(l, height_drop(h64[ro + at], wi, h64[co + at], wj));
                 if (__any_sync(0xffffffffu, up2 > 0.f && up2 >= low)) {  // a lane holds several such elements
                     const float* si = h32 + ro;
                     const float* sj = h32 + co;
                     for (int k = lane; k < K; k += 32) {
                         const float x0 = si[k] - sj[k], sl = kHeightSlack * (fabsf(si[k]) + fabsf(sj[k]));
-                        if (x0 + sl > 0.f && x0 + sl >= low) l = fmax(l, h64[ro + k] * wi - h64[co + k] * wj);
+                        if (x0 + sl > 0.f && x0 + sl >= low) l = fmax(l, height_drop(h64[ro + k], wi, h64[co + k], wj));
                     }
                 }
             }
@@ -484,7 +493,7 @@ __global__ void __launch_bounds__(1024)
     for (int k = threadIdx.x; k < a.K; k += blockDim.x) {
         const int32_t i = a.s[k], j = a.t[k];
         const double wi = sizeof(T) == 4 ? r.inv_deg_d[i] : 1.0, wj = sizeof(T) == 4 ? r.inv_deg_d[j] : 1.0;
-        const double diff = h64[(int64_t)i * a.Kp + k] * wi - h64[(int64_t)j * a.Kp + k] * wj;
+        const double diff = height_drop(h64[(int64_t)i * a.Kp + k], wi, h64[(int64_t)j * a.Kp + k], wj);
         gain += dem_d[k] * diff;
         gabs += dem_d[k] * fabs(diff);
     }
