@@ -532,6 +532,8 @@ __global__ void __launch_bounds__(1024)
 
 int resid_part_count(int32_t grid_v, int32_t grid_e) { return grid_v * kVParts + grid_e * kEParts; }
 
+constexpr int kMaxGridY = 65535;
+
 template <typename T, bool TABLE>
 void launch_passes(const ResidTask<T>* tasks, const ResidTask<T>& one, int count, int gv, int ge, int longest, cudaStream_t stream)
 {
@@ -552,8 +554,10 @@ cudaError_t launch_residuals(const ResidTask<T>* tasks, const ResidTask<T>* host
     }
     longest = gv > longest ? gv : longest;
     longest = ge > longest ? ge : longest;
-    if (tasks) launch_passes<T, true>(tasks, *host, count, gv, ge, longest, stream);
-    else launch_passes<T, false>(tasks, *host, 1, gv, ge, longest, stream);
+    if (!tasks) launch_passes<T, false>(tasks, *host, 1, gv, ge, longest, stream);
+    // the instance is the grid's y index, which ends at 65,535
+    for (int at = 0; tasks && at < count; at += kMaxGridY)
+        launch_passes<T, true>(tasks + at, *host, count - at < kMaxGridY ? count - at : kMaxGridY, gv, ge, longest, stream);
     return cudaGetLastError();
 }
 
