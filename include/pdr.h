@@ -289,6 +289,20 @@ pdr_status pdr_debug_barrier(pdr_ctx *ctx, int64_t limit_ns, int32_t withhold);
  * Errors: PDR_ERR_INVALID_ARG (nth < 0). */
 pdr_status pdr_debug_fail_alloc(int64_t nth);
 
+/* The same for launches of the cluster engine (pdr_options.use_graph): the nth
+ * from now on is refused before it reaches the device.  A solve whose first
+ * launch is refused runs on the graph engine, and so do the later ones of its
+ * context.  nth = 0 turns the injection off; process-wide.
+ * Errors: PDR_ERR_INVALID_ARG (nth < 0). */
+pdr_status pdr_debug_fail_cluster(int64_t nth);
+
+/* Test read-out: the engine that ran the sweeps of `precision` (PDR_PREC_FP32
+ * or PDR_PREC_FP64) in the context's latest solve that had any: 0 host loop, 1
+ * graph, 2 persistent kernel, 3 cluster; -1 before the first.  blocks: the
+ * cluster's size, 0 for the other engines.  Either may be NULL.
+ * Errors: PDR_ERR_INVALID_ARG. */
+pdr_status pdr_debug_engine(pdr_ctx *ctx, int32_t precision, int32_t *engine, int32_t *blocks);
+
 /* Selected rows of the current state: out[q*K + k] = f_{edges[q],k}
  * (which = 0) or the Alg. 4 velocity v_{edges[q],k} (which = 1), for
  * q < count (double).  For checking large instances edge by edge without

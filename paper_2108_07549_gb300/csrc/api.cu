@@ -199,6 +199,8 @@ struct pdr_ctx {
     struct {
         int32_t max_n = 0, max_m = -1, max_chunks = 0;
     } cl[4];
+    bool cl_refused = false;  // a launch of it was refused on this device: not tried again
+    int32_t engine[2] = {-1, -1}, engine_blocks[2] = {0, 0};  // what ran last, per precision (pdr_debug_engine)
     // reverse-mode workspace (pdr_backward: checkpoints, segment states,
     // cotangents), kept for later calls: the i-th buffer a call asks for is
     // reused when it is large enough, so calls with the same T, checkpoint
@@ -229,12 +231,14 @@ namespace {
 // Host-side failure injection (pdr_debug_fail_alloc): when positive, the
 // device allocation that brings it to 0 fails as if the device were full.
 std::atomic<int64_t> g_fail_alloc{0};
+// The same for launches of the cluster engine (pdr_debug_fail_cluster).
+std::atomic<int64_t> g_fail_cluster{0};
 
-bool injected_alloc_failure()
+bool injected_failure(std::atomic<int64_t>& nth)
 {
-    int64_t k = g_fail_alloc.load();
+    int64_t k = nth.load();
     while (k > 0)
-        if (g_fail_alloc.compare_exchange_weak(k, k - 1)) return k == 1;
+        if (nth.compare_exchange_weak(k, k - 1)) return k == 1;
     return false;
 }
 
@@ -243,7 +247,7 @@ T* dalloc(pdr_ctx* ctx, size_t count, pdr_status* st)
 {
     void* p = nullptr;
     if (count == 0) count = 1;
-    if (injected_alloc_failure()) {
+    if (injected_failure(g_fail_alloc)) {
         *st = PDR_ERR_OOM;
         ctx->err = "cudaMalloc: injected allocation failure";
         return nullptr;
@@ -956,7 +960,7 @@ bool cluster_shape(const pdr_ctx* ctx, int c, bool shared_sm, ClusterShape* out)
 bool cluster_eligible(const pdr_ctx* ctx)
 {
     const int cfg = ctx->cfg[0];
-    if (is_gd(ctx->opt) || cfg < 0 || edge_plain_config(cfg) > 5) return false;
+    if (is_gd(ctx->opt) || cfg < 0 || edge_plain_config(cfg) > 5 || ctx->cl_refused) return false;
     if (ctx->opt.use_graph != 3 && (ctx->opt.use_graph != 1 || ctx->opt.excess_variant >= 0)) return false;
     ClusterShape s;
     return cluster_shape(ctx, 3, false, &s);
@@ -989,21 +993,40 @@ ClusterArgs cluster_args(pdr_ctx* ctx, const ClusterShape& s, int par, bool firs
     return a;
 }
 
+cudaError_t try_launch_cluster(int cfg, const ClusterShape& s, int bytes, const ClusterArgs* table, const int* ids,
+                               const ClusterArgs& one, int count, cudaStream_t stream)
+{
+    if (injected_failure(g_fail_cluster)) return cudaErrorLaunchOutOfResources;
+    return launch_cluster(cfg, s.shares, table, ids, one, count, s.csize, s.threads, bytes, stream);
+}
+
 // FP32 sweeps by the cluster engine until the stop rules fire, in launches of
-// kClusterChunk sweeps; the flows start in buffer 0.
-pdr_status run_cluster(pdr_ctx* ctx, int64_t t_start)
+// kClusterChunk sweeps; the flows start in buffer 0.  *ran = false if the first
+// launch was refused, e.g. where the device's partition cannot hold the cluster
+// (the caller then uses the graph engine).
+pdr_status run_cluster(pdr_ctx* ctx, int64_t t_start, bool* ran)
 {
     const ClusterShape s = cluster_alone(ctx);
+    *ran = false;
     for (bool first = true;; first = false) {
         const int par = first ? 0 : (int)((ctx->hst->t - t_start) & 1);
-        CK(launch_cluster(ctx->cfg[0], s.shares, nullptr, nullptr, cluster_args(ctx, s, par, first), 1, s.csize, s.threads, s.bytes,
-                          ctx->stream));
+        const cudaError_t le = try_launch_cluster(ctx->cfg[0], s, s.bytes, nullptr, nullptr, cluster_args(ctx, s, par, first), 1,
+                                                  ctx->stream);
+        if (le != cudaSuccess) {
+            if (!first) return ctx->cuda_fail("launch_cluster", le);
+            cudaGetLastError();
+            ctx->cl_refused = true;
+            return PDR_OK;
+        }
+        *ran = true;
         const pdr_status st = read_state(ctx);  // synchronises the stream
         if (st != PDR_OK) return st;
         if (ctx->hst->stop) break;
     }
     ctx->cur = (int)((ctx->hst->t - t_start) & 1);
     ctx->psi_stale = true;
+    ctx->engine[0] = 3;
+    ctx->engine_blocks[0] = s.csize;
     return PDR_OK;
 }
 
@@ -1096,15 +1119,21 @@ pdr_status run_phase(pdr_ctx* ctx, int64_t t_start)
     // FP64 sweeps stay on the graph engine: a block is held to one SM's FP64
     // rate, a small fraction of its FP32 rate on this GPU, and loses to the
     // kernels that spread a sweep over every SM
-    if (p == Prec<float>::id && cluster_eligible(ctx)) return run_cluster(ctx, t_start);
+    if (p == Prec<float>::id && cluster_eligible(ctx)) {
+        bool ran = false;
+        s = run_cluster(ctx, t_start, &ran);
+        if (s != PDR_OK || ran) return s;
+    }
     s = ensure_psi(ctx);
     if (s != PDR_OK) return s;
+    ctx->engine_blocks[p] = 0;
     if (persistent_ok(ctx, p)) {
         bool ran = false;
         s = run_persistent<T>(ctx, &ran);
         if (s != PDR_OK) return s;
         if (ran) {
             ctx->cur = (int)((ctx->hst->t - t_start) & 1);
+            ctx->engine[p] = 2;
             return PDR_OK;
         }
     }
@@ -1112,7 +1141,8 @@ pdr_status run_phase(pdr_ctx* ctx, int64_t t_start)
         s = build_graph<T>(ctx);
         if (s != PDR_OK) return s;
     }
-    if (ctx->opt.use_graph && ctx->graph_ok[p]) {
+    ctx->engine[p] = ctx->opt.use_graph && ctx->graph_ok[p] ? 1 : 0;
+    if (ctx->engine[p] == 1) {
         CK(cudaGraphLaunch(ctx->exec[p], ctx->stream));
         s = read_state(ctx);
     } else {
@@ -2005,6 +2035,23 @@ pdr_status pdr_debug_wait(pdr_ctx* ctx, int64_t cycles, int32_t hold_end)
     return PDR_OK;
 }
 
+pdr_status pdr_debug_fail_cluster(int64_t nth)
+{
+    if (nth < 0) return PDR_ERR_INVALID_ARG;
+    g_fail_cluster.store(nth);
+    return PDR_OK;
+}
+
+pdr_status pdr_debug_engine(pdr_ctx* ctx, int32_t precision, int32_t* engine, int32_t* blocks)
+{
+    if (!ctx) return PDR_ERR_INVALID_ARG;
+    if (precision != PDR_PREC_FP32 && precision != PDR_PREC_FP64)
+        return ctx->fail(PDR_ERR_INVALID_ARG, "precision must be FP32 or FP64");
+    if (engine) *engine = ctx->engine[precision];
+    if (blocks) *blocks = ctx->engine_blocks[precision];
+    return PDR_OK;
+}
+
 pdr_status pdr_debug_barrier(pdr_ctx* ctx, int64_t limit_ns, int32_t withhold)
 {
     if (!ctx) return PDR_ERR_INVALID_ARG;
@@ -2746,8 +2793,9 @@ void batch_shapes(const pdr_batch* b, const std::vector<int32_t>& live, std::vec
 // The instances of `blk` (set up by batch_run) on the cluster engine:
 // launches of kClusterChunk sweeps, one per (variant, cluster size, threads)
 // on its own stream so that they run side by side, until every instance
-// stopped.  A finished instance's blocks leave and free their SM.
-pdr_status batch_cluster_run(pdr_batch* b, const std::vector<char>& blk, const std::vector<int64_t>& t_start)
+// stopped.  A finished instance's blocks leave and free their SM.  Instances
+// whose first launch was refused leave `blk` (the caller takes the graph).
+pdr_status batch_cluster_run(pdr_batch* b, std::vector<char>& blk, const std::vector<int64_t>& t_start)
 {
     std::vector<int32_t> live;
     for (int32_t i = 0; i < b->count; ++i)
@@ -2804,9 +2852,17 @@ pdr_status batch_cluster_run(pdr_batch* b, const std::vector<char>& blk, const s
             cudaStream_t sg = b->pool[group % b->pool.size()];
             if (!event(group + 1)) break;
             e = cudaStreamWaitEvent(sg, ev[0], 0);
-            if (e == cudaSuccess)
-                e = launch_cluster(b->ctx[order[at]]->cfg[0], s.shares, dargs, b->bids + at, ClusterArgs{}, (int)(end - at), s.csize,
-                                   s.threads, bytes, sg);
+            if (e == cudaSuccess) {
+                e = try_launch_cluster(b->ctx[order[at]]->cfg[0], s, bytes, dargs, b->bids + at, ClusterArgs{}, (int)(end - at), sg);
+                if (e != cudaSuccess && first) {
+                    e = cudaSuccess;
+                    cudaGetLastError();
+                    for (size_t q = at; q < end; ++q) {
+                        blk[order[q]] = 0;
+                        b->ctx[order[q]]->cl_refused = true;
+                    }
+                }
+            }
             if (e == cudaSuccess) e = cudaEventRecord(ev[1 + group], sg);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, ev[1 + group], 0);
             at = end;
@@ -2816,8 +2872,12 @@ pdr_status batch_cluster_run(pdr_batch* b, const std::vector<char>& blk, const s
         if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
         if (e != cudaSuccess) return cuda_err("cluster engine", e);
         std::vector<int32_t> next;
-        for (int32_t i : live)
+        for (int32_t i : live) {
+            if (!blk[i]) continue;
+            b->ctx[i]->engine[0] = 3;
+            b->ctx[i]->engine_blocks[0] = shapes[i].csize;
             if (!b->ctx[i]->hst->stop) next.push_back(i);
+        }
         live.swap(next);
         first = false;
     }
@@ -2876,7 +2936,6 @@ pdr_status batch_run(pdr_batch* b, const std::vector<char>& run_all, const std::
             run[i] = 0;
             any_blk = true;
         }
-    unsigned int running = 0;
     for (int32_t i = 0; i < b->count; ++i) {
         if (!run_all[i]) continue;
         pdr_ctx* c = b->ctx[i];
@@ -2884,14 +2943,17 @@ pdr_status batch_run(pdr_batch* b, const std::vector<char>& run_all, const std::
         if (s != PDR_OK) return s;
         s = flows_to_buffer0<T>(c);
         if (s != PDR_OK) return s;
-        if (run[i]) {
-            s = ensure_psi(c);
-            if (s != PDR_OK) return s;
-            ++running;
-        }
     }
     if (any_blk) {
         const pdr_status s = batch_cluster_run(b, blk, t_start);
+        if (s != PDR_OK) return s;
+    }
+    unsigned int running = 0;
+    for (int32_t i = 0; i < b->count; ++i) {
+        if (!run_all[i] || blk[i]) continue;
+        run[i] = 1;
+        ++running;
+        const pdr_status s = ensure_psi(b->ctx[i]);
         if (s != PDR_OK) return s;
     }
     if (running == 0) return PDR_OK;
@@ -2931,6 +2993,8 @@ pdr_status batch_run(pdr_batch* b, const std::vector<char>& run_all, const std::
         c->cur = (int)((c->hst->t - t_start[i]) & 1);
         // as in run_phase: the sweep that stopped by a rule left the partials of flows that were discarded
         c->psi_stale = c->hst->reason != STOP_MAX_SWEEPS;
+        c->engine[p] = use_graph && b->graph_ok[p] ? 1 : 0;
+        c->engine_blocks[p] = 0;
     }
     return PDR_OK;
 }

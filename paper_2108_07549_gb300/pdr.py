@@ -39,7 +39,7 @@ EXPORTS = (
     "pdr_batch_create", "pdr_batch_solve", "pdr_batch_reset", "pdr_batch_context", "pdr_batch_tuning",
     "pdr_batch_destroy", "pdr_set_data", "pdr_backward", "pdr_num_edge_variants", "pdr_edge_variant_capacity",
     "pdr_state_size", "pdr_get_state", "pdr_set_state", "pdr_debug_wait", "pdr_time_sweeps",
-    "pdr_debug_fail_alloc", "pdr_debug_barrier",
+    "pdr_debug_fail_alloc", "pdr_debug_barrier", "pdr_debug_fail_cluster", "pdr_debug_engine",
 )
 
 
@@ -112,6 +112,8 @@ def load(path: str = LIB_PATH):
         "pdr_debug_barrier": ([vp, i64, i32], i32),
         "pdr_time_sweeps": ([vp, i64, P(dbl), P(dbl)], i32),
         "pdr_debug_fail_alloc": ([i64], i32),
+        "pdr_debug_fail_cluster": ([i64], i32),
+        "pdr_debug_engine": ([vp, i32, P(i32), P(i32)], i32),
         "pdr_heights": ([vp, vp], i32),
         "pdr_congestion": ([vp, vp], i32),
         "pdr_objective": ([vp, P(dbl)], i32),
@@ -318,6 +320,12 @@ class Solver:
         """pdr_debug_barrier (test hook): time limit of the persistent engine's grid
         barrier, and whether block 0 withholds its arrival."""
         self._check(self._lib.pdr_debug_barrier(self._h, int(limit_ns), int(bool(withhold))))
+
+    def debug_engine(self, precision: int = 0):
+        """(engine, cluster blocks) that ran the latest sweeps of a precision (pdr_debug_engine)."""
+        e, b = C.c_int32(), C.c_int32()
+        self._check(self._lib.pdr_debug_engine(self._h, int(precision), C.byref(e), C.byref(b)))
+        return e.value, b.value
 
     def flow_rows(self, edges, velocities: bool = False) -> np.ndarray:
         """Rows f[e, :] (or the Alg. 4 velocities v[e, :]) for the given edge ids ([len(edges), K])."""
