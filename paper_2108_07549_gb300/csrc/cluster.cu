@@ -40,6 +40,7 @@
 // row adds or takes away +0); the parts of z are grouped otherwise (z agrees
 // to rounding).
 #include "edge_root.cuh"
+#include "widen.cuh"
 
 namespace pdr {
 namespace {
@@ -146,38 +147,31 @@ __device__ __forceinline__ float warp_max_pos(float x)  // of values >= 0
     return __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(x)));
 }
 
-// Sum of two unevaluated pairs: the high parts added error-free (TwoSum), the
-// errors and low parts added in FP32.  The pair is not renormalised, so a chain
-// of these waits on one addition per step (Acc's add: nine), and the low part
-// stays below 2^-24 of the sum times the number of terms.
-__device__ __forceinline__ float2 pair_add(float2 a, float2 b)
+// The sum over lanes whose numbers differ in the bits `from`, from / 2, .. 1.
+__device__ __forceinline__ Acc<float>::V xor_sum(Acc<float>::V z, int from)
 {
-    const float s = __fadd_rn(a.x, b.x), bb = __fsub_rn(s, a.x);
-    const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(b.x, bb));
-    return make_float2(s, __fadd_rn(e, __fadd_rn(a.y, b.y)));
-}
-__device__ __forceinline__ float2 pair_xor(float2 a, int o)
-{
-    return make_float2(__shfl_xor_sync(kFull, a.x, o), __shfl_xor_sync(kFull, a.y, o));
+#pragma unroll
+    for (int o = from; o > 0; o >>= 1) z = Acc<float>::add(z, Acc<float>::shfl(z, o));
+    return z;
 }
 
 // The full decision, on the state in shared memory, after `lag` sweeps that
-// passed the rules without it: the last of them had 2 z = zl.x + zl.y and the
-// maxima cons and cap, the sweep before it 2 z = zb.x + zb.y, and rmin is the
-// smallest max(cons, cap) among them.  By one lane; decide = 0 only settles.
-__device__ __noinline__ void full_decision(DevState* st, double* trace, int lag, float2 zl, float2 zb, float lcons, float lcap,
-                                           float rmin, int decide, float2 z, float cons, float cap, int* stop_now)
+// passed the rules without it: the last of them had 2 z = zl and the maxima
+// lcons and lcap, the sweep before it 2 z = zb, and rmin is the smallest
+// max(cons, cap) among them.  By one lane; decide = 0 only settles.
+__device__ __noinline__ void full_decision(DevState* st, double* trace, int lag, double zl, double zb, float lcons, float lcap,
+                                           float rmin, int decide, double z, float cons, float cap, int* stop_now)
 {
     if (lag > 0) {
         st->t += lag;
         st->evals += lag;
-        st->z = st->z_prev = 0.5 * ((double)zl.x + (double)zl.y);
-        if (lag > 1) st->dz = st->z - 0.5 * ((double)zb.x + (double)zb.y);
+        st->z = st->z_prev = 0.5 * zl;
+        if (lag > 1) st->dz = st->z - 0.5 * zb;
         st->cons_rel = (double)lcons;
         st->cap_rel = (double)lcap;
         if (st->plat_window > 0 && (double)rmin < st->plat_cur) st->plat_cur = (double)rmin;
     }
-    if (decide && apply_stop_rules(*st, MODE_SOLVE, trace, 0.5 * ((double)z.x + (double)z.y), (double)cons, (double)cap))
+    if (decide && apply_stop_rules(*st, MODE_SOLVE, trace, 0.5 * z, (double)cons, (double)cap))
         *stop_now = 1;
 }
 
@@ -468,30 +462,31 @@ __global__ void __launch_bounds__(1024, 1)
         const bool trace_on = ca.a.trace != nullptr && st.trace_len > 0;  // (in every block: all decide alike)
         int4* const slot = reinterpret_cast<int4*>(sm + L.slot);
         float2* const dpart = reinterpret_cast<float2*>(sm + L.dpart);
-        // An ordinary sweep passes the rules in FP32, on registers: z as the pair
-        // its sum is, dz as a pair difference.  Whatever is not clear of its
-        // threshold by more than the rounding of that (1 % is far more), and every
-        // sweep that is traced, takes the full decision in FP64, which costs more
-        // than a whole phase of a tiny instance.  eps <= 0 never fires; a tolerance
-        // rounded down to a float decides floats as it would in FP64.
+        // z is summed as the standalone kernels sum it: FP32 pairs within a block,
+        // the blocks' sums in FP64, and its change dz is formed in FP64.  An ordinary
+        // sweep then passes the rules in FP32 on registers: whatever is not clear of
+        // its threshold by more than the rounding of that (1 % is far more), and every
+        // sweep that is traced, takes the full decision in FP64, which costs more than
+        // a whole phase of a tiny instance.  eps <= 0 never fires; a tolerance rounded
+        // down to a float decides floats as it would in FP64.
         const float eps = st.eps_obj > 0.0 ? 2.02f * __double2float_ru(st.eps_obj) : -1.f;
         const float epr = st.eps_rel > 0.0 ? 1.01f * __double2float_ru(st.eps_rel) : -1.f;
         const float tol = st.resid_tol > 0.0 ? __double2float_rd(st.resid_tol) : -1.f;
         const bool fall = st.stop_on_rise != 0;
-        float2 zl = make_float2(0.f, 0.f), zb = zl;  // 2 z of the last two sweeps (lag of them unsettled)
+        double zl = 0.0, zb = 0.0;  // 2 z of the last two sweeps (lag of them unsettled)
         float lcons = 0.f, lcap = 0.f, rmin = 0.f;
         int lag = 0, left = 0;  // left: sweeps before the sweep cap or the end of a plateau window
         auto decide = [&]() {
             int4 p = make_int4(0, 0, 0, 0);
             if (lane < csize) p = slot[lane];
-            float2 z = make_float2(__int_as_float(p.x), __int_as_float(p.y));
+            double z = widen(__int_as_float(p.x)) + widen(__int_as_float(p.y));
             const float cons = warp_max_pos(__int_as_float(p.z)), cap = warp_max_pos(__int_as_float(p.w));
             if constexpr (CL) {
-                for (int o = csize >> 1; o > 0; o >>= 1) z = pair_add(z, pair_xor(z, o));
+                for (int o = csize >> 1; o > 0; o >>= 1) z += __shfl_xor_sync(kFull, z, o);
             }
-            z = make_float2(__shfl_sync(kFull, z.x, 0), __shfl_sync(kFull, z.y, 0));
-            const float dz = (z.x - zl.x) + (z.y - zl.y), slack = 1e-13f * z.x, least = fmaxf(eps, epr * z.x);
-            if (left > 0 && fabsf(z.x) < 1e38f && (least < 0.f || fabsf(dz) > least + slack) &&
+            z = __shfl_sync(kFull, z, 0);
+            const float dz = (float)(z - zl), zf = (float)z, slack = 1e-13f * zf, least = fmaxf(eps, epr * zf);
+            if (left > 0 && fabsf(zf) < 1e38f && (least < 0.f || fabsf(dz) > least + slack) &&
                 !(cap <= tol && cons <= tol) && !(fall && dz > -slack)) {
                 zb = zl;
                 zl = z;
@@ -527,37 +522,36 @@ __global__ void __launch_bounds__(1024, 1)
                 break;
             }
             // the threads' parts, then the block's sum to every block
-            float2 z = make_float2(0.f, 0.f);
             constexpr int kParts = 1024 / (32 * kDecWarps);
-            float2 p[kParts];
+            A::V part[kParts];
 #pragma unroll
             for (int l = 0; l < kParts; ++l) {
                 const int at = dt + l * 32 * kDecWarps;
-                p[l] = at < workers ? reinterpret_cast<const float2*>(sm + L.sum)[at] : make_float2(0.f, 0.f);
+                const float2 x = at < workers ? reinterpret_cast<const float2*>(sm + L.sum)[at] : make_float2(0.f, 0.f);
+                part[l] = A::V{x.x, x.y};
             }
 #pragma unroll
-            for (int l = 0; l < kParts; ++l) z = pair_add(z, p[l]);
+            for (int w = kParts / 2; w > 0; w >>= 1)
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) z = pair_add(z, pair_xor(z, o));
-            if (lane == 0) dpart[dw] = z;
+                for (int l = 0; l < w; ++l) part[l] = A::add(part[l], part[l + w]);
+            const A::V z = xor_sum(part[0], 16);
+            if (lane == 0) dpart[dw] = A::store(z);
             asm volatile("bar.sync 1, %0;" ::"n"(32 * kDecWarps) : "memory");
             if (dw == 0) {
-                float2 mx = make_float2(0.f, 0.f), p = make_float2(0.f, 0.f);
+                float2 mx = make_float2(0.f, 0.f);
                 if (lane < nww) mx = reinterpret_cast<const float2*>(sm + L.mx)[lane];
-                p = dpart[lane & (kDecWarps - 1)];
-                float2 zz = p;
-#pragma unroll
-                for (int o = kDecWarps / 2; o > 0; o >>= 1) zz = pair_add(zz, pair_xor(zz, o));
+                const float2 p = dpart[lane & (kDecWarps - 1)];
+                const A::V zz = xor_sum(A::V{p.x, p.y}, kDecWarps / 2);
                 const float cons = warp_max_pos(mx.x), cap = warp_max_pos(mx.y);
                 if (lane < csize) {
                     if constexpr (CL)
                         asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
                                          map_rank(smem_u32(slot) + 16u * rank, lane)),
-                                     "r"(__float_as_int(zz.x)), "r"(__float_as_int(zz.y)), "r"(__float_as_int(cons)),
+                                     "r"(__float_as_int(zz.hi)), "r"(__float_as_int(zz.lo)), "r"(__float_as_int(cons)),
                                      "r"(__float_as_int(cap))
                                      : "memory");
                     else
-                        *slot = make_int4(__float_as_int(zz.x), __float_as_int(zz.y), __float_as_int(cons),
+                        *slot = make_int4(__float_as_int(zz.hi), __float_as_int(zz.lo), __float_as_int(cons),
                                           __float_as_int(cap));
                 }
             }

@@ -92,3 +92,27 @@ def test_a_refusal_in_mid_solve_is_an_error(pdr):
             pdr.load().pdr_debug_fail_cluster(0)
         s.reset()
         assert s.solve()["sweeps"] == 8192 + 10 and s.debug_engine() == (CLUSTER, 1)
+
+
+# ------------------------------------------------------------------ the objective's sum
+
+
+def test_blocks_sums_are_added_in_64_bits(pdr):
+    """An objective whose terms are powers of two over 51 binary places, the largest and the smallest in different
+    blocks: a 64-bit sum of the blocks' pairs is exact.  Vertices of a ring with two arcs out and two in, no
+    capacity: a flow f on one arc adds f^2 as congestion and 4 (f/4)^2 at each of its ends."""
+    n, K = 256, 32
+    tail = np.repeat(np.arange(n), 2)
+    row_ptr, col = I._csr(n, tail, (tail + np.tile([1, 2], n)) % n)
+    f = np.zeros((2 * n, K))
+    for vertex, k, x in ((0, 0, 1.0), (2, 1, 2.0**-12), (250, 2, 2.0**-25)):
+        f[2 * vertex, k] = x
+    s, t = np.full(K, 100), np.full(K, 150)
+    d = np.full(K, 2.0**-60)  # squares far below the last place
+    for use_graph, engine in ((0, HOST), (1, CLUSTER)):
+        with pdr.Solver(n, row_ptr, col, np.zeros(2 * n), s, t, d, use_graph=use_graph, max_sweeps=1, trace_len=2,
+                        **FREE) as solver:
+            solver.set_flows(f)
+            solver.solve()
+            assert solver.debug_engine()[0] == engine and (engine == HOST or solver.debug_engine()[1] > 1)
+            assert solver.trace()[0] == 0.75 * (1.0 + 2.0**-24 + 2.0**-50)
