@@ -116,3 +116,63 @@ def test_blocks_sums_are_added_in_64_bits(pdr):
             solver.solve()
             assert solver.debug_engine()[0] == engine and (engine == HOST or solver.debug_engine()[1] > 1)
             assert solver.trace()[0] == 0.75 * (1.0 + 2.0**-24 + 2.0**-50)
+
+
+# ------------------------------------------------------------------ against the captured loop
+
+
+def parallel(n, extra, K, seed):
+    """n vertices with `extra` arcs among them (many parallel): fewer vertices than a cluster has blocks."""
+    rng = np.random.default_rng([seed, n, K])
+    src = np.concatenate([np.arange(n), rng.integers(0, n, extra)])
+    dst = np.concatenate([(np.arange(n) + 1) % n, rng.integers(0, n, extra)])
+    keep = src != dst
+    row_ptr, col = I._csr(n, src[keep], dst[keep])
+    s = rng.integers(0, n, K)
+    t = (s + rng.integers(1, n, K)) % n
+    u = rng.uniform(0, 4, col.shape[0]) * (rng.random(col.shape[0]) < 0.7) / 20
+    return I.Instance(name=f"par{n}_{K}", n=n, row_ptr=row_ptr, col=col, u=u, s=s.astype(np.int32),
+                      t=t.astype(np.int32), d=rng.uniform(0.5, 3, K), factor=1.0, load=u, hops=np.ones(K, np.int64))
+
+
+CASES = {"grid5": (1, lambda: I.grid5_k10(1.3)), "tight": (1, lambda: I.grid5_k10(0.6)),
+         "few3": (8, lambda: parallel(3, 1500, 32, 1)), "few6": (8, lambda: parallel(6, 1200, 61, 2)),
+         "large": (8, lambda: digraph(400, 90, 3)), "wide": (8, lambda: digraph(60, 500, 4))}
+
+
+@pytest.mark.parametrize("name", CASES)
+@pytest.mark.parametrize("algo", [0, 3])
+def test_flows_equal_the_graph_over_several_launches(pdr, algo, name):
+    """Two whole launches of 8192 sweeps and an odd remainder, then a second solve from the returned flows."""
+    blocks, make = CASES[name]
+    inst = make()
+    got = []
+    for kw in (dict(use_graph=1), dict(use_graph=1, excess_variant=0)):
+        with pdr.Solver.from_instance(inst, algo=algo, max_sweeps=2 * 8192 + 1, **kw, **FREE) as s:
+            r1 = s.solve()
+            f1 = s.flows()
+            s.set_options(max_sweeps=8192 + 2)
+            r2 = s.solve()
+            got.append((r1, f1, r2, s.flows(), s.debug_engine()))
+    a, b = got
+    assert a[4] == (CLUSTER, blocks) and b[4] == (GRAPH, 0)
+    assert a[0]["sweeps"] == b[0]["sweeps"] == 2 * 8192 + 1 and a[2]["sweeps"] == b[2]["sweeps"] == 8192 + 2
+    np.testing.assert_array_equal(a[1], b[1])
+    np.testing.assert_array_equal(a[3], b[3])
+    for q in (0, 2):
+        assert a[q]["z"] == b[q]["z"] and a[q]["cap_rel"] == b[q]["cap_rel"] and a[q]["cons_rel"] == b[q]["cons_rel"]
+        assert abs(a[q]["dz"] - b[q]["dz"]) <= 1e-12 * max(1.0, a[q]["z"])
+
+
+@pytest.mark.parametrize("name", CASES)
+@pytest.mark.parametrize("rules", [dict(eps_rel=1e-3), dict(resid_tol=0.5), dict(eps_rel=1e-6, trace_len=9000)])
+def test_rules_fire_where_the_graph_s_do(pdr, rules, name):
+    inst = CASES[name][1]()
+    got = []
+    for kw in (dict(use_graph=1), dict(use_graph=1, excess_variant=0)):
+        with pdr.Solver.from_instance(inst, max_sweeps=9000, **dict(FREE, **rules), **kw) as s:
+            r = s.solve()
+            got.append((r["sweeps"], r["stop_reason"], s.flows(), s.trace() if "trace_len" in rules else np.ones(1)))
+    assert got[0][:2] == got[1][:2]
+    np.testing.assert_array_equal(got[0][2], got[1][2])
+    np.testing.assert_allclose(got[0][3], got[1][3], rtol=1e-12)
