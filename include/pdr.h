@@ -258,13 +258,16 @@ pdr_status pdr_get_state(pdr_ctx *ctx, void *buf, int64_t bytes);
 pdr_status pdr_set_state(pdr_ctx *ctx, const void *buf, int64_t bytes);
 
 /* Test hook for the time limit of the device-side waits.
- * - Waits: the bulk-copy excess forms (pdr_options.excess_variant 1..5)
- *   waits on shared-memory barriers.
+ * - Waits: those on shared-memory barriers, for bulk copies.  The bulk-copy
+ *   excess forms (pdr_options.excess_variant 1..5) have them, the edge QP's
+ *   staged forms, and its ring form, which FP32 variants 3..6 take when there
+ *   are edges enough for the device's warps.
  * - Default limit: 2^32 SM clock cycles, about 2 s.
  * - cycles: sets that limit; 1000 <= cycles <= 2^32.
- * - hold_end = 1: the form's producer never posts the end marker of its
- *   ring.  Every block's consumers then wait out the limit, with no copy in
- *   flight, and the call that ran the sweep returns PDR_ERR_TIMEOUT.
+ * - hold_end = 1: an excess form's producer never posts the end marker of
+ *   its ring, and the warps of the edge QP's ring form never start their
+ *   first copies.  The waits for them run out, with no copy in flight, and the
+ *   call that ran the sweep returns PDR_ERR_TIMEOUT.
  * - hold_end = 0: normal operation.
  * Errors: PDR_ERR_INVALID_ARG. */
 pdr_status pdr_debug_wait(pdr_ctx *ctx, int64_t cycles, int32_t hold_end);

@@ -184,8 +184,8 @@ struct pdr_ctx {
     // checkpoint / resume: the next pdr_solve continues the restored sweep
     // counter and objective instead of starting afresh
     bool resume_pending = false;
-    // device-side wait limit (cycles) and the end-marker hold of the bulk-copy
-    // excess form; changed only by pdr_debug_wait (tests of the time limit)
+    // limit (cycles) and hold of the sweep kernels' shared-memory barrier waits;
+    // changed only by pdr_debug_wait (tests of the time limit)
     long long wait_cycles = kWaitCycles;
     int hold_end = 0;
     // persistent engine's grid barrier; changed only by pdr_debug_barrier
@@ -772,7 +772,7 @@ pdr_status read_state(pdr_ctx* ctx)
     CK(cudaMemcpyAsync(ctx->hst, ctx->st, sizeof(DevState), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     if (ctx->hst->fault)
-        return ctx->fail(PDR_ERR_TIMEOUT, "excess kernel: a shared-memory barrier wait ran out of its time limit");
+        return ctx->fail(PDR_ERR_TIMEOUT, "sweep kernel: a shared-memory barrier wait ran out of its time limit");
     return PDR_OK;
 }
 

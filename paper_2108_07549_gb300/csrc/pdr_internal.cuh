@@ -143,9 +143,11 @@ struct SweepArgs {
     int excess_form;    // excess kernel: 0 = per-thread gathers, 1..3 = bulk-copy pipeline
                         // (stages x row segments per block: 4 x 8, 2 x 8, 4 x 4)
     const int32_t* xv_start;  // [grid_v + 1] bulk-copy form: first vertex of each block
-    long long wait_cycles;    // bulk-copy form: time limit of a barrier wait, in SM clock cycles
-    int hold_end;             // bulk-copy form, tests only: the producer never posts its end
-                              // marker, so the consumers' last wait runs out (no copy in flight)
+    long long wait_cycles;    // bulk-copy forms of both kernels and the edge QP's ring: time limit of
+                              // a barrier wait, in SM clock cycles
+    int hold_end;             // tests only, a wait that runs out with no copy in flight: the bulk excess
+                              // forms' producer never posts its end marker, the ring's warps never
+                              // start their first copies
     long long barrier_ns;     // persistent engine: time limit of a grid-barrier wait, in ns
     int hold_barrier;         // persistent engine, tests only: block 0 leaves without arriving
                               // at its first grid barrier, so the other blocks' waits run out

@@ -352,9 +352,9 @@ __global__ void __launch_bounds__(C + 32) excess_bulk_kernel(SweepArgs<T> a)
     typename A::V zacc = A::zero();
     T cons = T(0);
     bool ok = true;
+    uint32_t j = 0;  // producer: batches posted, the end marker among them
     if (producer) {
         // producer warp; every branch below is warp-uniform
-        uint32_t j = 0;
         // units in segment-major order: every vertex of the range for segment 0, then 1, ...
         for (int c = 0; c < nseg && ok; ++c) {
             const int width = min(W, a.Kp - c * W);
@@ -426,15 +426,14 @@ __global__ void __launch_bounds__(C + 32) excess_bulk_kernel(SweepArgs<T> a)
             const uint32_t ph = (j / S) & 1u;
             if (j >= (uint32_t)S && !__all_sync(kFull, mbar_wait(&empty[slot], ph ^ 1u, a.wait_cycles))) {
                 ok = false;
-            } else if (lane == 0 && !a.hold_end) {  // hold_end: a test of the consumers' time limit
-                desc[slot].flags = kXEnd;
-                desc[slot].nrows = 0;
-                mbar_arrive(&full[slot]);
+            } else if (!a.hold_end) {  // hold_end: a test of the consumers' time limit
+                if (lane == 0) {
+                    desc[slot].flags = kXEnd;
+                    desc[slot].nrows = 0;
+                    mbar_arrive(&full[slot]);
+                }
+                ++j;
             }
-        }
-        if (!ok) {
-            // wait (limited) for the copies of the last S batches, then leave
-            for (uint32_t q = j > (uint32_t)S ? j - S : 0; q < j; ++q) mbar_wait(&full[q % S], (q / S) & 1u, a.wait_cycles);
         }
     } else {
         // consumers: thread tid holds values tid*N .. tid*N+N-1 of the segment;
@@ -443,7 +442,7 @@ __global__ void __launch_bounds__(C + 32) excess_bulk_kernel(SweepArgs<T> a)
         int cs = 0;
 #pragma unroll
         for (int q = 0; q < N; ++q) acc[q] = T(0);
-        for (uint32_t j = 0;; ++j) {
+        for (;; ++j) {
             const int slot = (int)(j % S);
             const uint32_t ph = (j / S) & 1u;
             if (!__all_sync(kFull, mbar_wait(&full[slot], ph, a.wait_cycles))) {
@@ -511,6 +510,10 @@ __global__ void __launch_bounds__(C + 32) excess_bulk_kernel(SweepArgs<T> a)
             a.st->fault = 1;
             stop_from_kernel(a);
         }
+        // whoever gave up: the copies of the last S batches land before the block leaves
+        // (to the default limit, however short a.wait_cycles was made)
+        if (producer)
+            for (uint32_t q = j > (uint32_t)S ? j - S : 0; q < j; ++q) mbar_wait(&full[q % S], (q / S) & 1u, kWaitCycles);
     }
     excess_tail<T>(a, block, gridDim.x, zacc, cons, TailPart<T>(a, block, gridDim.x));
 }
@@ -696,7 +699,8 @@ __global__ void __launch_bounds__(R > 1 ? kShareThreads : kThreads) edge_group_k
 // warps (edge_pipe_kernel).  Per element the arithmetic is the plain form's,
 // so the flows are bit-identical to it.  Each wait is limited
 // (a.wait_cycles); a warp whose wait runs out records the fault, ends the
-// solve, waits (limited) for its copies and leaves.
+// solve, waits for its copies (to the default limit, however short the other
+// one was made) and leaves.
 template <typename T>
 __host__ __device__ constexpr size_t ring_stage_bytes(int Kp)  // f, h_i, h_j
 {
@@ -744,7 +748,7 @@ __global__ void __launch_bounds__(kThreads) edge_ring_kernel(SweepArgs<T> a)
     };
     pdl_wait();     // the excess kernel has finished (no-op without PDL)
     pdl_trigger();  // one wave
-    if (any && lane == 0) stage(e, si, sj);
+    if (any && lane == 0 && !a.hold_end) stage(e, si, sj);  // hold_end: a test of the time limit
     __syncwarp();
     const int skip = update_skipped(a);
     if (decision) {
@@ -752,7 +756,7 @@ __global__ void __launch_bounds__(kThreads) edge_ring_kernel(SweepArgs<T> a)
         return;
     }
     if (skip) {  // the first copy, then leave
-        if (any) mbar_wait(&full[w], 0, a.wait_cycles);
+        if (any && !a.hold_end) mbar_wait(&full[w], 0, kWaitCycles);
         return;
     }
     const int den = a.ck ? 0 : 2;
@@ -775,7 +779,7 @@ __global__ void __launch_bounds__(kThreads) edge_ring_kernel(SweepArgs<T> a)
                 stop_from_kernel(a);
             }
             __syncwarp();
-            mbar_wait(&full[w], phase, a.wait_cycles);
+            if (!a.hold_end) mbar_wait(&full[w], phase, kWaitCycles);
             break;
         }
         phase ^= 1u;
@@ -1324,7 +1328,7 @@ __global__ void __launch_bounds__(B, 1) edge_staged_kernel(SweepArgs<T> a)
                 a.st->fault = 1;
                 stop_from_kernel(a);
             }
-            mbar_wait(&full, phase, a.wait_cycles);  // the copy in flight, then leave
+            mbar_wait(&full, phase, kWaitCycles);  // the copy in flight, then leave
             return;
         }
         phase ^= 1u;
