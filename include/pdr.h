@@ -206,7 +206,9 @@ pdr_status pdr_solve(pdr_ctx *ctx, pdr_result *out);
 pdr_status pdr_sweeps(pdr_ctx *ctx, int64_t count);
 
 /* Sets every flow to 0, every velocity to 0 and every learning rate to
- * beta_init, and the iteration counter to 0 (the start of Alg. 1, 3 and 4). */
+ * beta_init, and the iteration counter to 0 (the start of Alg. 1, 3 and 4).
+ * Does not wait for the stream.  Errors: PDR_ERR_CUDA, also where the stream
+ * is being captured (as by every call that waits for it); PDR_ERR_OOM. */
 pdr_status pdr_reset(pdr_ctx *ctx);
 
 /* Copies host flows f[m*K] (double, edge-major) into the context, rounding

@@ -1798,6 +1798,15 @@ pdr_status pdr_set_options(pdr_ctx* ctx, const pdr_options* opt)
 pdr_status pdr_reset(pdr_ctx* ctx)
 {
     if (!ctx) return PDR_ERR_INVALID_ARG;
+    // nothing below waits for the stream, so a capture would take the launch
+    // and leave the flows as they are: refused, as by the calls that wait
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    cudaError_t ce = cudaStreamIsCapturing(ctx->stream, &cs);
+    if (ce == cudaSuccess && cs != cudaStreamCaptureStatusNone) ce = cudaErrorStreamCaptureUnsupported;
+    if (ce != cudaSuccess) {
+        cudaGetLastError();
+        return ctx->cuda_fail("pdr_reset", ce);
+    }
     ctx->cur_prec = start_prec(ctx->opt);
     pdr_status s = ctx->cur_prec ? ensure_fp64(ctx) : ensure_fp32(ctx);
     if (s != PDR_OK) return s;
