@@ -782,11 +782,28 @@ pdr_status read_state(pdr_ctx* ctx)
 // n 10,000, m 39,600, K 10,000, 20 sweeps 26,701 / 25,978; n 20,000, m 100,000,
 // K 2000, 20 sweeps 16,417 / 15,722, 50 sweeps of the reverse mode's forward
 // pass 32,780 / 31,350).
+//
+// Alg. 3 / Alg. 4: not behind the bulk copies, and not in FP64 where the blocks
+// of a lane-group or 128-thread form make 45 to 100 % of a wave.  An early launch places the update kernel's blocks where the excess pass
+// has left room; part of a wave then need not lie evenly, and the FP64 pipe of the
+// fullest SM decides (that explanation is inferred from where it happens).
+// Sweep, us, Alg. 3, with / without (n, m, K), FP32 gathers: 400, 1520, 60: 7.33
+// / 7.76; 2500, 15,000, 250: 23.4 / 24.0; bulk copies: 784, 3024, 500: 12.9 /
+// 12.1; 2500, 15,000, 2000: 131 / 111; 8000, 40,000, 2000: 353 / 284; FP64: 625,
+// 2400, 130: 43.8 / 33.6; 500, 3000, 100: 40.4 / 34.2; 225, 840, 600: 62.6 / 44.3;
+// 324, 1224, 600: 66.6 / 62.7; less of a wave: 484, 1848, 130: 31.7 / 32.2; 144,
+// 528, 600: 31.0 / 31.5; a wave: 400, 1520, 600: 69.7 / 70.6; 512 threads: 225,
+// 840, 1100: 85.3 / 85.7.
 template <typename T>
 bool pdl_pays(const pdr_ctx* ctx)
 {
     const int p = Prec<T>::id;
-    return is_gd(ctx->opt) || !edge_config_block(ctx->cfg[p]) || ctx->pf[p] == 0;
+    if (is_gd(ctx->opt)) {
+        const int form = edge_plain_config(ctx->cfg[p]), wave = (form == 7 ? 10 : 4) * ctx->num_sms;
+        if (ctx->xform != 0) return false;
+        if (sizeof(T) == 8 && form <= 7 && 20 * ctx->grid_e[p] > 9 * wave && ctx->grid_e[p] < wave) return false;
+    }
+    return !edge_config_block(ctx->cfg[p]) || ctx->pf[p] == 0;
 }
 
 // The sweep loop as one graph: a conditional WHILE node whose body holds
