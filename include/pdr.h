@@ -267,9 +267,9 @@ pdr_status pdr_set_state(pdr_ctx *ctx, const void *buf, int64_t bytes);
  * - Default limit: 2^32 SM clock cycles, about 2 s.
  * - cycles: sets that limit; 1000 <= cycles <= 2^32.
  * - hold_end = 1: an excess form's producer never posts the end marker of
- *   its ring, and the warps of the edge QP's ring form never start their
- *   first copies.  The waits for them run out, with no copy in flight, and the
- *   call that ran the sweep returns PDR_ERR_TIMEOUT.
+ *   its ring, and the barriers of the edge QP's ring form want one arrival
+ *   more than a copy makes.  The waits run out, the copies in flight land, and
+ *   the call that ran the sweep returns PDR_ERR_TIMEOUT.
  * - hold_end = 0: normal operation.
  * Errors: PDR_ERR_INVALID_ARG. */
 pdr_status pdr_debug_wait(pdr_ctx *ctx, int64_t cycles, int32_t hold_end);

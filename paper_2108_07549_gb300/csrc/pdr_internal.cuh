@@ -145,9 +145,9 @@ struct SweepArgs {
     const int32_t* xv_start;  // [grid_v + 1] bulk-copy form: first vertex of each block
     long long wait_cycles;    // bulk-copy forms of both kernels and the edge QP's ring: time limit of
                               // a barrier wait, in SM clock cycles
-    int hold_end;             // tests only, a wait that runs out with no copy in flight: the bulk excess
-                              // forms' producer never posts its end marker, the ring's warps never
-                              // start their first copies
+    int hold_end;             // tests only, a wait that runs out whatever the copies do: the bulk excess
+                              // forms' producer never posts its end marker, the ring's barriers want
+                              // an arrival that is made when the warp has given up
     long long barrier_ns;     // persistent engine: time limit of a grid-barrier wait, in ns
     int hold_barrier;         // persistent engine, tests only: block 0 leaves without arriving
                               // at its first grid barrier, so the other blocks' waits run out

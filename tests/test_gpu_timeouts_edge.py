@@ -1,9 +1,9 @@
 """Time limits of the edge QP's shared-memory waits, and that a limit made
 shorter than a copy takes leaves no copy behind.
 
-pdr_debug_wait with hold_end keeps every warp of the ring form from starting
-its first copies: its wait runs out with nothing in flight, and the call
-returns PDR_ERR_TIMEOUT.  With a limit of a thousand cycles ordinary
+pdr_debug_wait with hold_end makes the ring form's barriers want one arrival
+more than a copy makes: every warp's wait runs out, its copies land, and the
+call returns PDR_ERR_TIMEOUT.  With a limit of a thousand cycles ordinary
 waits may run out too; a kernel that gives up still waits for the copies it
 started.  Nothing faults, traps or hangs the GPU."""
 
