@@ -154,6 +154,7 @@ struct pdr_ctx {
     int64_t n_psi[2] = {1, 1};
     int pgrid[2] = {0, 0};         // persistent kernel grid per precision (0: not available)
     int ring[2] = {0, 0};          // edge kernel: the ring form (per precision)
+    bool ring_crowds[2] = {false, false};  // kRingCrowd
     int64_t pf[2] = {0, 0};        // edge-kernel L2 prefetch distance per precision (edges)
     GridBarrier* bar = nullptr;    // its grid barrier
     DevState* st = nullptr;
@@ -521,12 +522,24 @@ int64_t prefetch_policy(const pdr_ctx* ctx, int cfg)
     return rows * sizeof(T) > kL2Bytes ? edge_prefetch_distance<T>(cfg, ctx->num_sms) : 0;
 }
 
+// A ring whose warps take one edge each and fill more than this share of the
+// device's does not go with the bulk-copy excess form (select_excess_form).
+constexpr double kRingCrowd = 0.75;
+constexpr int kBulkRowBytes = 1800, kBulkVerticesPerSm = 5;
+bool bulk_rows(const pdr_ctx* ctx)  // FP32
+{
+    return ctx->Kp * 4 >= kBulkRowBytes && ctx->n >= kBulkVerticesPerSm * ctx->num_sms;
+}
+
 // Grid, partials and form (plain or ring) of edge variant cfg.
 template <typename T>
 void set_edge_grid(pdr_ctx* ctx, int cfg, const pdr_options& o)
 {
     const int p = Prec<T>::id;
-    const int ring = is_gd(o) ? 0 : edge_ring_grid<T>(cfg, ctx->m, ctx->Kp, ctx->num_sms);
+    int resident = 0;
+    int ring = is_gd(o) ? 0 : edge_ring_grid<T>(cfg, ctx->m, ctx->Kp, ctx->num_sms, &resident);
+    ctx->ring_crowds[p] = ring > 0 && (int64_t)ring * (kThreads / 32) >= ctx->m && ring > kRingCrowd * resident;
+    if (ctx->ring_crowds[p] && cfg <= 5 && bulk_rows(ctx)) ring = 0;
     ctx->ring[p] = ring > 0 ? 1 : 0;
     ctx->shares[p] = is_gd(o) || ring > 0 ? 1 : edge_shares<T>(cfg, ctx->m, ctx->num_sms);
     ctx->grid_e[p] = ring > 0 ? ring : edge_grid<T>(cfg, ctx->m, ctx->num_sms, ctx->shares[p]);
@@ -559,7 +572,7 @@ pdr_status select_edge_variants(pdr_ctx* ctx, const pdr_options& o)
     ctx->cfg[1] = c64;
     set_edge_grid<float>(ctx, c32, o);
     if (c64 >= 0) set_edge_grid<double>(ctx, c64, o);
-    else ctx->grid_e[1] = 1, ctx->n_psi[1] = 1, ctx->ring[1] = 0, ctx->shares[1] = 1;
+    else ctx->grid_e[1] = 1, ctx->n_psi[1] = 1, ctx->ring[1] = 0, ctx->ring_crowds[1] = false, ctx->shares[1] = 1;
     // L2 prefetch of later waves' rows pays only when the rows come from HBM:
     // when both flow buffers and the heights fit in L2 (as they stay across
     // sweeps) the prefetches are pure overhead
@@ -784,9 +797,10 @@ pdr_status read_state(pdr_ctx* ctx)
 // pass 32,780 / 31,350).
 //
 // Alg. 3 / Alg. 4: not behind the bulk copies, and not in FP64 where the blocks
-// of a lane-group or 128-thread form make 45 to 100 % of a wave.  An early launch places the update kernel's blocks where the excess pass
-// has left room; part of a wave then need not lie evenly, and the FP64 pipe of the
-// fullest SM decides (that explanation is inferred from where it happens).
+// of a lane-group or 128-thread form make 45 to 100 % of a wave.  An early launch
+// places the update kernel's blocks where the excess pass has left room; part of a
+// wave then need not lie evenly, and the FP64 pipe of the fullest SM decides (that
+// explanation is inferred from where it happens).
 // Sweep, us, Alg. 3, with / without (n, m, K), FP32 gathers: 400, 1520, 60: 7.33
 // / 7.76; 2500, 15,000, 250: 23.4 / 24.0; bulk copies: 784, 3024, 500: 12.9 /
 // 12.1; 2500, 15,000, 2000: 131 / 111; 8000, 40,000, 2000: 353 / 284; FP64: 625,
@@ -1064,17 +1078,24 @@ bool persistent_ok(const pdr_ctx* ctx, int p)
 //   39,600, 300: 42 / 47; 8000, 40,000, 400: 52.7 / 52.9; 8000, 40,000, 500:
 //   60.9 / 56.9; 10,000, 39,600, 600: 74 / 64; 625, 2400, 4000: 38.7 / 44.3;
 //   20,000, 100,000, 2000: 699 / 651.
+//   But not with a crowded ring (kRingCrowd), and then with the edge QP's plain
+//   form up to 4 vectors per lane (gathers and plain / gathers and ring / bulk and
+//   ring): 961, 3720, 480: 11.4 / 12.3 / 13.7; 1024, 3968, 500: 12.0 / 12.4 / 14.2;
+//   1225, 4760, 500: 12.7 / 13.4 / 15.0; 1600, 4800, 500: 14.7 / 15.2 / 16.5; 800,
+//   4800, 500: 13.6 / 14.3 / 15.4; 8 vectors: 1100, 3300, 700: 17.2 / 14.5 / 15.9;
+//   900, 3480, 640: 14.8 / 12.4 / 13.3.  Where the ring fills less of the device:
+//   900, 3480, 500: gathers and ring 12.1, bulk and ring 11.5.
 // - FP64, bound by its pipe: bulk copies once the gathers need several rounds of
 //   their resident threads.  500, 3000, 100: 20.2 / 23.7; 900, 3480, 500: 58.9 /
 //   67.5; 2000, 8000, 200: 67.2 / 68.6; 10,000, 40,000, 200: 280 / 266; 20,000,
 //   60,000, 50: 143 / 133.
 constexpr int kDefaultExcessForm = 2;
-constexpr int kBulkRowBytes = 1800, kBulkVerticesPerSm = 5, kBulkRounds = 4;
+constexpr int kBulkRounds = 4;
 pdr_status select_excess_form(pdr_ctx* ctx, const pdr_options& o)
 {
     const bool bulk = o.precision == PDR_PREC_FP64
                           ? (int64_t)ctx->n * (ctx->Kp / 2) > (int64_t)kBulkRounds * ctx->grid_v[1] * kGatherThreads
-                          : ctx->Kp * 4 >= kBulkRowBytes && ctx->n >= kBulkVerticesPerSm * ctx->num_sms;
+                          : bulk_rows(ctx) && !ctx->ring_crowds[0];
     const int v = o.excess_variant >= 0 ? o.excess_variant
                   : bulk && ctx->xgrid[kDefaultExcessForm] > 0 ? kDefaultExcessForm : 0;
     if (v > 0 && ctx->xgrid[v] <= 0)
@@ -1779,7 +1800,7 @@ pdr_status pdr_set_options(pdr_ctx* ctx, const pdr_options* opt)
                             o.beta_min != ctx->opt.beta_min || o.beta_max != ctx->opt.beta_max ||
                             o.alpha_inc != ctx->opt.alpha_inc || o.alpha_dec != ctx->opt.alpha_dec ||
                             o.gamma != ctx->opt.gamma;
-    if (o.excess_variant != ctx->opt.excess_variant || o.precision != ctx->opt.precision) {
+    if (variant_changed || o.excess_variant != ctx->opt.excess_variant || o.precision != ctx->opt.precision) {
         const pdr_status xs = select_excess_form(ctx, o);
         if (xs != PDR_OK) return xs;
         destroy_graphs(ctx);

@@ -192,7 +192,7 @@ int edge_grid(int cfg, int64_t m, int num_sms, int shares);  // grid size of tha
 template <typename T>
 int edge_shares(int cfg, int64_t m, int num_sms);  // shares of a lane of that variant (1, 2 or 4)
 template <typename T>
-int edge_ring_grid(int cfg, int64_t m, int Kp, int num_sms);  // the ring form's, 0 where it does not apply
+int edge_ring_grid(int cfg, int64_t m, int Kp, int num_sms, int* resident);  // the ring form's, 0 where it does not apply
 template <typename T>
 int64_t edge_parts(int cfg, int grid, int shares);  // number of partials that grid writes
 template <typename T>

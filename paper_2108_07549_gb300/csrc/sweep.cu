@@ -1715,13 +1715,14 @@ int ring_blocks(int Kp, int num_sms)
 // 25,000, 600: 66.8 / 45.2; 12,000, 36,000, 530: 96.0 / 73.5; 20,000, 100,000,
 // 500: 185 / 170; 900, 3480, 501 (0.7 of its warps): 11.6 / 10.8.
 template <typename T>
-int edge_ring_grid(int cfg, int64_t m, int Kp, int num_sms)
+int edge_ring_grid(int cfg, int64_t m, int Kp, int num_sms, int* resident)
 {
     if (sizeof(T) != 4 || cfg < 3 || cfg > 6 || ring_smem<T>(Kp) > (size_t)kRingSmemMax) return 0;
     const int blocks = cfg == 3   ? ring_blocks<T, 1>(Kp, num_sms)
                        : cfg == 4 ? ring_blocks<T, 2>(Kp, num_sms)
                        : cfg == 5 ? ring_blocks<T, 4>(Kp, num_sms)
                                   : ring_blocks<T, 8>(Kp, num_sms);
+    *resident = blocks;
     const int64_t warps = (int64_t)blocks * (kThreads / 32);
     if (blocks < 2 || (double)m < kRingWaves * (double)warps) return 0;
     // the same number of edges for every warp, as nearly as it goes
@@ -1729,8 +1730,8 @@ int edge_ring_grid(int cfg, int64_t m, int Kp, int num_sms)
     const int64_t g = (need + kThreads / 32 - 1) / (kThreads / 32);
     return (int)(g < blocks - 1 ? g : blocks - 1);
 }
-template int edge_ring_grid<float>(int, int64_t, int, int);
-template int edge_ring_grid<double>(int, int64_t, int, int);
+template int edge_ring_grid<float>(int, int64_t, int, int, int*);
+template int edge_ring_grid<double>(int, int64_t, int, int, int*);
 
 // Shares built for a lane-group variant: at most 16 row elements per lane.
 constexpr int share_limit(int G, int V) { return V >= 8 ? 1 : V >= 4 ? 2 : 4; }
