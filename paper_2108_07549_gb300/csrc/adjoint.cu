@@ -16,8 +16,7 @@
 //   flows    dL/df^(t)_e,k = cbar_e,k + Dbar_{j,k} - Dbar_{i,k} (eq. (3)), formed
 //            on the fly by the next (earlier) sweep's edge step.
 // The seeds at T are dz/df = psi + h_j - h_i (eq. "cpgrad"), dz/du = -psi
-// and dz/dd_k = h_{s_k,k} - h_{t_k,k}.  One warp per edge row, two passes
-// over the row (the second from L1/L2), so any K works.
+// and dz/dd_k = h_{s_k,k} - h_{t_k,k}.
 #include "sweep_common.cuh"
 
 namespace pdr {
@@ -75,15 +74,13 @@ __global__ void demand_kernel(SweepArgs<T> a, const T* __restrict__ x, double* _
     }
 }
 
-// Warp per edge: Alg. 2's Jacobian applied to fbar = dL/df^(t+1) (see the
-// file comment).  fbar is either read (the seed, at t + 1 = T) or formed on
-// the fly from the previous backward step's results, fbar = cbar^(t+1) +
-// Dbar^(t+1)_j - Dbar^(t+1)_i (`fused`), which saves writing and reading it.
-// cbar is updated in place: each element is read (as part of fbar) and then
-// written by the same lane.  Pass 1 decides every element's membership of the
-// active set (c > cut) from f and both height rows and records it as warp
-// ballots in `mask` (N words per 32 vectors of the row); pass 2 re-reads only
-// fbar's rows.
+// The edge step: Alg. 2's Jacobian applied to fbar = dL/df^(t+1) (see the file
+// comment).  fbar is either read (the seed, at t + 1 = T) or formed on the fly
+// from the previous backward step's results, fbar = cbar^(t+1) + Dbar^(t+1)_j -
+// Dbar^(t+1)_i (`fused`), which saves writing and reading it.  cbar is updated in
+// place: each element is read (as part of fbar) and then written by the same
+// thread.  f and both height rows decide an element's membership of the active
+// set (c > cut).
 template <typename T, bool FUSED>
 __device__ __forceinline__ void fbar_vec(const typename VecOf<T>::type* fb, const typename VecOf<T>::type* cb,
                                          const typename VecOf<T>::type* di, const typename VecOf<T>::type* dj, int v,
@@ -99,75 +96,6 @@ __device__ __forceinline__ void fbar_vec(const typename VecOf<T>::type* fb, cons
         for (int j = 0; j < N; ++j) g[j] = c[j] + y[j] - x[j];
     } else {
         unpack(fb[v], g);
-    }
-}
-
-template <typename T, bool FUSED>
-__global__ void __launch_bounds__(kThreads) edge_backward_kernel(SweepArgs<T> a, const T* __restrict__ theta,
-                                                                 const T* __restrict__ fbar, T* cbar,
-                                                                 const T* __restrict__ Dbar, double* __restrict__ ubar,
-                                                                 uint32_t* __restrict__ mask)
-{
-    using VT = typename VecOf<T>::type;
-    constexpr int N = VecOf<T>::N;
-    const int lane = threadIdx.x & 31;
-    const int vpr = a.Kp / N;
-    const int nq = (vpr + 31) / 32;
-    pdl_wait();
-    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t e = w0; e < a.m; e += nw) {
-        const T th = theta[e];
-        const bool congested = th > T(0);
-        const T cut = congested ? th : T(0);
-        const int32_t ti = a.src[e], tj = a.col[e];
-        const VT* fr = reinterpret_cast<const VT*>(a.f + e * a.Kp);
-        const VT* hi = reinterpret_cast<const VT*>(a.h + (int64_t)ti * a.Kp);
-        const VT* hj = reinterpret_cast<const VT*>(a.h + (int64_t)tj * a.Kp);
-        const VT* fb = FUSED ? nullptr : reinterpret_cast<const VT*>(fbar + e * a.Kp);
-        VT* cb = reinterpret_cast<VT*>(cbar + e * a.Kp);
-        const VT* di = FUSED ? reinterpret_cast<const VT*>(Dbar + (int64_t)ti * a.Kp) : nullptr;
-        const VT* dj = FUSED ? reinterpret_cast<const VT*>(Dbar + (int64_t)tj * a.Kp) : nullptr;
-        uint32_t* me = mask + e * (int64_t)nq * N;
-        T sb = T(0);
-        int na = 0;
-        for (int q = 0; q < nq; ++q) {  // every lane takes every round: the ballots need the whole warp
-            const int v = q * 32 + lane;
-            const bool live = v < vpr;
-            T f[N] = {}, x[N] = {}, y[N] = {}, g[N] = {};
-            if (live) {
-                unpack(fr[v], f);
-                unpack(hi[v], x);
-                unpack(hj[v], y);
-                fbar_vec<T, FUSED>(fb, cb, di, dj, v, g);
-            }
-#pragma unroll
-            for (int j = 0; j < N; ++j) {
-                const bool act = live && fma(T(0.5), x[j] - y[j], f[j]) > cut;  // the edge-QP kernel's c
-                if (act) {
-                    sb += g[j];
-                    ++na;
-                }
-                const uint32_t b = __ballot_sync(kFull, act);
-                if (lane == j) me[q * N + j] = b;
-            }
-        }
-        __syncwarp();  // the ballots written above are read by every lane below
-        sb = group_sum<32>(sb);
-        na = group_sum<32>(na);
-        // Alg. 2: theta = (S_A - u)/(2 + |A|); capacity kept: (S_A - u)/|A|.  With
-        // the capacity kept and u = 0 no element is active and nothing flows back.
-        const T corr = (congested && na > 0) ? sb / T((a.ck ? 0 : 2) + na) : T(0);
-        for (int q = 0; q < nq; ++q) {
-            const int v = q * 32 + lane;
-            if (v >= vpr) continue;
-            T g[N], o[N];
-            fbar_vec<T, FUSED>(fb, cb, di, dj, v, g);
-#pragma unroll
-            for (int j = 0; j < N; ++j) o[j] = ((me[q * N + j] >> lane) & 1u) ? g[j] - corr : T(0);
-            cb[v] = pack4(o);
-        }
-        if (lane == 0) ubar[e] += (double)corr;
     }
 }
 
@@ -244,7 +172,7 @@ __global__ void __launch_bounds__(kThreads, V <= 4 ? 4 : 3)
 }
 
 // Block of B threads per edge for long rows (thread l holds row vectors l +
-// q*B): the same step as edge_backward_kernel, but the row's cotangent and
+// q*B): the same step, the row's cotangent and
 // its active-set bits stay in registers between the block-wide sum and the
 // write, so every input row is read once (the warp form reads fbar, or cbar
 // and both Dbar rows, a second time).
@@ -426,8 +354,8 @@ void launch_backward_block(const SweepArgs<T>& a, const T* theta, const T* fbar,
 
 // The edge step's form by the row's length in vectors: a warp with the row in
 // registers up to 8 vectors per lane (0..6); the block form with the smallest
-// capacity that holds the row (7..12); beyond the largest the warp form that
-// reads twice (-1).
+// capacity that holds the row (7..12), which the longest row of the edge
+// variants fills.
 template <typename T>
 int backward_form(int Kp)
 {
@@ -440,10 +368,11 @@ int backward_form(int Kp)
 
 template <typename T>
 cudaError_t launch_backward_sweep(const SweepArgs<T>& a, const T* theta, const T* fbar, T* cbar, T* Dbar,
-                                  double* ubar, double* dbar, uint32_t* mask, int fused, int num_sms, cudaStream_t s)
+                                  double* ubar, double* dbar, int fused, int num_sms, cudaStream_t s)
 {
-    const int ge = blocks(a.m * 32, kThreads, num_sms);
-    switch (a.m > 0 ? backward_form<T>(a.Kp) : -1) {
+    const int form = backward_form<T>(a.Kp);
+    if (form < 0) return cudaErrorInvalidValue;
+    switch (a.m > 0 ? form : -1) {  // no edges: the vertex step alone
     case 0: launch_backward_warp<T, 1>(a, theta, fbar, cbar, Dbar, ubar, fused, s); break;
     case 1: launch_backward_warp<T, 2>(a, theta, fbar, cbar, Dbar, ubar, fused, s); break;
     case 2: launch_backward_warp<T, 3>(a, theta, fbar, cbar, Dbar, ubar, fused, s); break;
@@ -457,9 +386,7 @@ cudaError_t launch_backward_sweep(const SweepArgs<T>& a, const T* theta, const T
     case 10: launch_backward_block<T, 512, 5>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
     case 11: launch_backward_block<T, 512, 8>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
     case 12: launch_backward_block<T, 1024, 8>(a, theta, fbar, cbar, Dbar, ubar, fused, num_sms, s); break;
-    default:
-        if (fused) launch_dependent(edge_backward_kernel<T, true>, ge, kThreads, s, a, theta, fbar, cbar, Dbar, ubar, mask);
-        else launch_dependent(edge_backward_kernel<T, false>, ge, kThreads, s, a, theta, fbar, cbar, Dbar, ubar, mask);
+    default: break;
     }
     launch_dependent(vertex_backward_kernel<T>, blocks((int64_t)a.n * (a.Kp / VecOf<T>::N), kThreads, num_sms), kThreads, s,
                      a, cbar, Dbar);
@@ -470,8 +397,8 @@ cudaError_t launch_backward_sweep(const SweepArgs<T>& a, const T* theta, const T
 template cudaError_t launch_seed<float>(const SweepArgs<float>&, float*, double*, double*, int, cudaStream_t);
 template cudaError_t launch_seed<double>(const SweepArgs<double>&, double*, double*, double*, int, cudaStream_t);
 template cudaError_t launch_backward_sweep<float>(const SweepArgs<float>&, const float*, const float*, float*, float*,
-                                                  double*, double*, uint32_t*, int, int, cudaStream_t);
+                                                  double*, double*, int, int, cudaStream_t);
 template cudaError_t launch_backward_sweep<double>(const SweepArgs<double>&, const double*, const double*, double*,
-                                                   double*, double*, double*, uint32_t*, int, int, cudaStream_t);
+                                                   double*, double*, double*, int, int, cudaStream_t);
 
 }  // namespace pdr

@@ -147,7 +147,7 @@ struct pdr_ctx {
     // partials typed by the working precision: 8 bytes per entry covers both
     double *part_cons = nullptr, *part_capb = nullptr, *part_psi = nullptr, *part_cap = nullptr;
     int grid_v[2] = {1, 1}, grid_e[2] = {1, 1}, cfg[2] = {-1, -1}, shares[2] = {1, 1};
-    // excess kernel form (0: gathers, 1..3: bulk copies); grid and vertex split of each bulk form
+    // excess kernel form (0: gathers, 1..5: bulk copies); grid and vertex split of each bulk form
     int xform = 0;
     int xgrid[kExcessForms] = {};
     int32_t* xv_start[kExcessForms] = {};
@@ -1404,7 +1404,6 @@ pdr_status backward_T(pdr_ctx* ctx, int64_t Tn, int32_t C, double* L, double* gr
         if (!(q = (T*)grab(sizeof(T) * 2 * mm))) return cleanup(), ctx->fail(PDR_ERR_OOM, "checkpoint allocation failed");
     T *fbar = nullptr, *cbar = nullptr, *Dbar = nullptr;
     double *ubar = nullptr, *dbar = nullptr;
-    uint32_t* mask = nullptr;
     if (ckpt) {
         seg.resize(C + 1);
         th.resize(C);
@@ -1422,8 +1421,7 @@ pdr_status backward_T(pdr_ctx* ctx, int64_t Tn, int32_t C, double* L, double* gr
         Dbar = (T*)grab(sizeof(T) * hn);
         ubar = (double*)grab(sizeof(double) * mm);
         dbar = (double*)grab(sizeof(double) * ctx->K);
-        mask = (uint32_t*)grab(sizeof(uint32_t) * mm * backward_mask_words(ctx->Kp, 16 / sizeof(T)));
-        if (!fbar || !cbar || !Dbar || !ubar || !dbar || !mask)
+        if (!fbar || !cbar || !Dbar || !ubar || !dbar)
             return cleanup(), ctx->fail(PDR_ERR_OOM, "adjoint allocation failed");
     }
     // the kernels of a run of sweeps but its first, as in the captured loop
@@ -1495,8 +1493,8 @@ pdr_status backward_T(pdr_ctx* ctx, int64_t Tn, int32_t C, double* L, double* gr
         SweepArgs<T> a = make_args<T>(ctx, MODE_EVAL);
         a.f = fs[t];
         a.h = hs[t];
-        CKB(launch_backward_sweep<T>(a, ths[t], fbar, cbar, Dbar, ubar, dbar, mask, t == Tn - 1 ? 0 : 1,
-                                     ctx->num_sms, ctx->stream));
+        CKB(launch_backward_sweep<T>(a, ths[t], fbar, cbar, Dbar, ubar, dbar, t == Tn - 1 ? 0 : 1, ctx->num_sms,
+                                     ctx->stream));
     }
     // or segment by segment from the last
     for (int64_t sgi = nseg - 1; ckpt && sgi >= 0; --sgi) {
@@ -1510,8 +1508,8 @@ pdr_status backward_T(pdr_ctx* ctx, int64_t Tn, int32_t C, double* L, double* gr
             a.f = seg[t - t0];
             a.h = hseg[t - t0];  // h^(t), from the recomputation above
             // the first step reads the seed; later ones form dL/df^(t+1) from cbar and Dbar
-            CKB(launch_backward_sweep<T>(a, th[t - t0], fbar, cbar, Dbar, ubar, dbar, mask, t == Tn - 1 ? 0 : 1,
-                                         ctx->num_sms, ctx->stream));
+            CKB(launch_backward_sweep<T>(a, th[t - t0], fbar, cbar, Dbar, ubar, dbar, t == Tn - 1 ? 0 : 1, ctx->num_sms,
+                                         ctx->stream));
         }
     }
     // the gradients go to host or device memory alike (unified addressing)
@@ -2937,9 +2935,6 @@ pdr_status batch_cluster_run(pdr_batch* b, std::vector<char>& blk, const std::ve
     return done(PDR_OK);
 }
 
-// Alg. 1 in precision T for the instances with run_all[i] set, from the states
-// their callers initialised (instance i's sweep counter starting at
-// t_start[i]); the others keep their stopped state.
 // Every instance's solver state, in one copy.
 pdr_status batch_read_states(pdr_batch* b)
 {
@@ -2969,6 +2964,9 @@ pdr_status batch_residuals(pdr_batch* b)
     return PDR_OK;
 }
 
+// Alg. 1 in precision T for the instances with run_all[i] set, from the states
+// their callers initialised (instance i's sweep counter starting at
+// t_start[i]); the others keep their stopped state.
 template <typename T>
 pdr_status batch_run(pdr_batch* b, const std::vector<char>& run_all, const std::vector<int64_t>& t_start)
 {

@@ -21,7 +21,7 @@
 
 namespace pdr {
 
-constexpr int kThreads = 256;  // block size of every sweep kernel
+constexpr int kThreads = 256;  // block size of the sweep kernels that state no other
 constexpr int kGatherThreads = 64;  // gather form of the excess pass: small blocks spread a few hundred vertices over the SMs
 constexpr int kShareThreads = 64;  // block size of the lane-group forms with several shares per lane
 constexpr int kExcessForms = 6;     // excess kernel forms: 0 gathers, 1..5 bulk copies
@@ -140,8 +140,8 @@ struct SweepArgs {
     void* part_psi;     // [n_psi] per edge warp/block: sum psi^2 (float2 pair or double)
     T* part_cap;        // [n_psi] per edge warp/block: max psi/scale
     int32_t grid_v, grid_e;
-    int excess_form;    // excess kernel: 0 = per-thread gathers, 1..3 = bulk-copy pipeline
-                        // (stages x row segments per block: 4 x 8, 2 x 8, 4 x 4)
+    int excess_form;    // excess kernel: 0 = per-thread gathers, 1..5 = bulk-copy pipeline (stages x row
+                        // segments per block: 4 x 8, 2 x 8, 4 x 4; 2 x 8 and 4 x 8 of short segments)
     const int32_t* xv_start;  // [grid_v + 1] bulk-copy form: first vertex of each block
     long long wait_cycles;    // bulk-copy forms of both kernels and the edge QP's ring: time limit of
                               // a barrier wait, in SM clock cycles
@@ -272,9 +272,7 @@ template <typename T>
 cudaError_t launch_seed(const SweepArgs<T>& a, T* fbar, double* ubar, double* dbar, int num_sms, cudaStream_t s);
 template <typename T>
 cudaError_t launch_backward_sweep(const SweepArgs<T>& a, const T* theta, const T* fbar, T* cbar, T* Dbar, double* ubar,
-                                  double* dbar, uint32_t* mask, int fused, int num_sms, cudaStream_t s);
-// words of the active-set ballots launch_backward_sweep keeps per edge
-inline int64_t backward_mask_words(int Kp, int vec) { return (int64_t)((Kp / vec + 31) / 32) * vec; }
+                                  double* dbar, int fused, int num_sms, cudaStream_t s);
 
 // Residuals and certificate (residuals.cu).
 struct ResidOut {

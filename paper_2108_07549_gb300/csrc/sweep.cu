@@ -283,7 +283,6 @@ constexpr size_t excess_bulk_smem()
     return (size_t)S * R * xseg_bytes<C>() + (size_t)S * (2 * sizeof(uint64_t) + sizeof(XDesc));
 }
 
-// S stages of R row segments of C x 16 bytes
 // Waits for the copies of the last S of `end` batches.  (Out of line: inline, these
 // waits cost the bulk kernel 0.7 % at n 5000, m 25,000, K 600, though they never run.)
 __device__ __noinline__ void land_batches(uint64_t* full, uint32_t end, uint32_t S)
@@ -291,6 +290,7 @@ __device__ __noinline__ void land_batches(uint64_t* full, uint32_t end, uint32_t
     for (uint32_t q = end > S ? end - S : 0; q < end; ++q) mbar_wait(&full[q % S], (q / S) & 1u, kWaitCycles);
 }
 
+// S stages of R row segments of C x 16 bytes
 template <typename T, int S, int R, int C>
 __global__ void __launch_bounds__(C + 32) excess_bulk_kernel(SweepArgs<T> a)
 {
@@ -1718,10 +1718,10 @@ template <typename T>
 int edge_ring_grid(int cfg, int64_t m, int Kp, int num_sms, int* resident)
 {
     if (sizeof(T) != 4 || cfg < 3 || cfg > 6 || ring_smem<T>(Kp) > (size_t)kRingSmemMax) return 0;
-    const int blocks = cfg == 3   ? ring_blocks<T, 1>(Kp, num_sms)
-                       : cfg == 4 ? ring_blocks<T, 2>(Kp, num_sms)
-                       : cfg == 5 ? ring_blocks<T, 4>(Kp, num_sms)
-                                  : ring_blocks<T, 8>(Kp, num_sms);
+    const int blocks = cfg == 3   ? ring_blocks<float, 1>(Kp, num_sms)
+                       : cfg == 4 ? ring_blocks<float, 2>(Kp, num_sms)
+                       : cfg == 5 ? ring_blocks<float, 4>(Kp, num_sms)
+                                  : ring_blocks<float, 8>(Kp, num_sms);
     *resident = blocks;
     const int64_t warps = (int64_t)blocks * (kThreads / 32);
     if (blocks < 2 || (double)m < kRingWaves * (double)warps) return 0;
@@ -1772,14 +1772,16 @@ template <typename T>
 cudaError_t launch_edge(const SweepArgs<T>& a, int cfg, cudaStream_t stream, bool pdl)
 {
     const int g = a.grid_e + 1;  // edge blocks plus the decision block
-    if (a.ring && a.mode != MODE_PSI) {
-        const size_t smem = ring_smem<T>(a.Kp);
-        switch (cfg) {
-        case 3: return launch_one<T>(edge_ring_kernel<T, 1>, g, kThreads, stream, pdl, a, smem);
-        case 4: return launch_one<T>(edge_ring_kernel<T, 2>, g, kThreads, stream, pdl, a, smem);
-        case 5: return launch_one<T>(edge_ring_kernel<T, 4>, g, kThreads, stream, pdl, a, smem);
-        case 6: return launch_one<T>(edge_ring_kernel<T, 8>, g, kThreads, stream, pdl, a, smem);
-        default: return cudaErrorInvalidValue;
+    if constexpr (sizeof(T) == 4) {
+        if (a.ring && a.mode != MODE_PSI) {
+            const size_t smem = ring_smem<T>(a.Kp);
+            switch (cfg) {
+            case 3: return launch_one<T>(edge_ring_kernel<T, 1>, g, kThreads, stream, pdl, a, smem);
+            case 4: return launch_one<T>(edge_ring_kernel<T, 2>, g, kThreads, stream, pdl, a, smem);
+            case 5: return launch_one<T>(edge_ring_kernel<T, 4>, g, kThreads, stream, pdl, a, smem);
+            case 6: return launch_one<T>(edge_ring_kernel<T, 8>, g, kThreads, stream, pdl, a, smem);
+            default: return cudaErrorInvalidValue;
+            }
         }
     }
     switch (cfg) {
