@@ -191,11 +191,14 @@ def load_peaks():
         return 6800.0, "fallback"
 
 
+SWEEP_SOURCES = ("sweep.cu", "edge_root.cuh", "pdr_internal.cuh", "sweep_common.cuh", "widen.cuh")
+
+
 def source_digest():
     """Digest of the sweep kernels' sources (the files the ncu counters depend on)."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2108_07549_gb300", "csrc")
-    for name in ("sweep.cu", "sweep_common.cuh", "pdr_internal.cuh"):
+    for name in SWEEP_SOURCES:
         with open(os.path.join(csrc, name), "rb") as fh:
             h.update(name.encode())
             h.update(fh.read())
@@ -450,10 +453,11 @@ def compare_engines(args, inst, pdr, torch, stream):
     out = {"kind": "sweep-loop engine comparison", "sweeps": S, "dtype": "f32", "us_per_sweep": {}}
     for c in cases:
         row = {"m": c.m, "K": c.K}
-        for name, eng in (("host_loop", 0), ("graph", 1), ("persistent", 2), ("cluster", 3)):
+        # graph: with the gathers, since an excess form asked for keeps a small instance on the graph
+        for name, eng, form in (("host_loop", 0, -1), ("graph", 1, 0), ("persistent", 2, -1), ("cluster", 3, -1)):
             with torch.cuda.stream(stream):
                 with pdr.Solver.from_instance(c, stream=stream.cuda_stream, precision=pdr.PREC_FP32, eps_obj=0.0,
-                                              resid_tol=0.0, max_sweeps=S, use_graph=eng) as sv:
+                                              resid_tol=0.0, max_sweeps=S, use_graph=eng, excess_variant=form) as sv:
                     sv.solve()
                     times = []
                     for q in range(3):
@@ -800,9 +804,9 @@ def l2_resident_block(pdr, torch, stream, inst, flush, steps=5, S=2000):
 def residual_block(pdr, torch, stream, big, budget_sweeps=2000):
     """Time to residual 1e-6 (cap_rel and cons_rel <= 1e-6, or a Farkas
     certificate) on the 5x5 grid and its infeasible twin (GPU FP64, GPU FP32
-    with the FP64 tail on the CUDA-graph engine, the same with its FP32
-    sweeps on the cluster engine -- one block holding the instance in shared
-    memory -- and the FP64 oracle), and on the headline instance the
+    with the FP64 tail -- its FP32 sweeps by the cluster engine, one block
+    holding the instance in shared memory -- the same with them on the CUDA
+    graph, and the FP64 oracle), and on the headline instance the
     residuals reached within a fixed budget of FP32 sweeps, with the oracle's
     residuals at the same early sweep beside the GPU's."""
     import oracle
@@ -812,12 +816,13 @@ def residual_block(pdr, torch, stream, big, budget_sweeps=2000):
     g = I.grid5_k10(1.3, seed=0)
     for label, inst in (("grid5_k10_feasible_1.3x", g), ("grid5_k10_infeasible_0.6x", g.with_factor(0.6))):
         row = {}
-        for prec, code, eng in (("gpu_fp64", pdr.PREC_FP64, 1), ("gpu_fp32_fp64tail", pdr.PREC_FP32_FP64TAIL, 1),
-                                ("gpu_fp32_fp64tail_cluster_engine", pdr.PREC_FP32_FP64TAIL, 3)):
+        # an excess form asked for keeps a small instance on the graph
+        for prec, code, form in (("gpu_fp64", pdr.PREC_FP64, -1), ("gpu_fp32_fp64tail", pdr.PREC_FP32_FP64TAIL, -1),
+                                 ("gpu_fp32_fp64tail_graph_engine", pdr.PREC_FP32_FP64TAIL, 0)):
             with torch.cuda.stream(stream):
                 with pdr.Solver.from_instance(inst, stream=stream.cuda_stream, precision=code, eps_obj=0.0,
                                               resid_tol=1e-6, eps_rel=1e-13, max_sweeps=600000,
-                                              use_graph=eng) as sv:
+                                              excess_variant=form) as sv:
                     sv.solve()  # warm-up (graph capture)
                     sv.reset()
                     r = sv.solve()
