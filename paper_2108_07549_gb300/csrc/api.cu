@@ -507,8 +507,9 @@ pdr_status refresh_psi_current(pdr_ctx* ctx)
     return ctx->cur_prec ? refresh_psi<double>(ctx) : refresh_psi<float>(ctx);
 }
 
-// Before a kernel that reads the congestion partials: the cluster engine, which
-// keeps its own, and a batch's instance that stopped by a rule leave them behind.
+// Before a kernel that reads the congestion partials: the cluster and persistent
+// engines, which keep their own, and a batch's instance that stopped by a rule
+// leave them behind.
 pdr_status ensure_psi(pdr_ctx* ctx)
 {
     if (!ctx->psi_stale) return PDR_OK;
@@ -1139,8 +1140,10 @@ pdr_status run_persistent(pdr_ctx* ctx, bool* ran)
         if (hb.failed) return ctx->fail(PDR_ERR_TIMEOUT, "persistent sweep kernel: a grid barrier timed out");
         if (ctx->hst->stop) break;
     }
-    // the other engines read the congestion partials in the standalone layout
-    return refresh_psi<T>(ctx, nullptr, true);
+    // the other engines read the congestion partials in the standalone layout, and
+    // those of the flows that the caller makes the current ones
+    ctx->psi_stale = true;
+    return PDR_OK;
 }
 
 // One phase of Alg. 1 in precision T, from the state set by init_state
