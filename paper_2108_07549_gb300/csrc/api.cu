@@ -9,7 +9,8 @@
 // loop condition, so a whole solve is one launch and one host
 // synchronisation.  If the runtime cannot build that graph, the same kernels
 // are launched from a host loop that reads the stop flag back between
-// chunks of sweeps.
+// chunks of sweeps.  The FP32 sweeps of a small instance run on one
+// thread-block cluster instead (cluster.cu).
 #include "pdr.h"
 #include "pdr_internal.cuh"
 
