@@ -29,7 +29,8 @@
 // Measured against the graph engine's two launches per sweep (us per sweep, FP32,
 // 2000 sweeps; n, m, K): 25, 80, 10: 1.5 against 8.8 (one block); 100, 360, 30:
 // 2.1 against 8.6; 200, 600, 50: 3.5 against 9.7; 300, 1200, 56: 5.4 against
-// 10.2 (8 blocks); 400, 1600, 90: 9.1 against 10.3.  In the large ones the reads
+// 10.2 (8 blocks); 400, 1600, 90: 9.1 against 10.3 (the graph's gathers have become
+// faster since: 6.5 in the first, 7.8 in the third).  In the large ones the reads
 // from the other blocks' shared memory bound it (a block's half of the rows
 // comes in at roughly 14 bytes per clock), in the small ones the chain of phase
 // B: one pass of the search and its decisions, about 1500 cycles.
